@@ -63,7 +63,7 @@ struct BatchGroupDev {
     const BfRItem *ritems;
     const BfItem *litems[16];
     const int *ints;
-    const double *dbl;
+    const uint2 *words;
     const int *depth_parity;
     double2 *ai;                      // [nalm][nmaps]
     int nmaps;
@@ -92,12 +92,12 @@ __device__ void warp_item(const BatchDev &bd, const BatchWork &w, double *wsm, i
     if (w.type == W_RES) {
         const BfRItem it = G.ritems[w.idx];
         double *ubuf = G.depth_parity[it.m * 2 + it.t] ? M.u1 : M.u0;
-        shtb_dev::bf_r_item<NB, true>(it, G.v.lmax, G.v.nhalf, G.ints, G.dbl, G.ai, G.nmaps, M.b0, ubuf, M.qt,
+        shtb_dev::bf_r_item<NB, true>(it, G.v.lmax, G.v.nhalf, G.ints, G.words, G.ai, G.nmaps, M.b0, ubuf, M.qt,
                                       lane);
     } else {
         const double *uin = (w.aux % 2) ? M.u1 : M.u0;
         double *uout = ((w.aux - 1) % 2) ? M.u1 : M.u0;
-        shtb_dev::bf_level_item<NB, true>(G.litems[w.aux - 1][w.idx], G.v.lmax, G.v.nhalf, G.ints, G.dbl, uin,
+        shtb_dev::bf_level_item<NB, true>(G.litems[w.aux - 1][w.idx], G.v.lmax, G.v.nhalf, G.ints, G.words, uin,
                                           uout, M.qt, wsm, lane);
     }
 }
@@ -314,7 +314,7 @@ int build_schedule(shtb_batch_s *b, int warps, int width, int lpt)
         D.ritems = bf.ritems;
         for (int l = 0; l < 16; ++l) D.litems[l] = l < bf.depth_max ? bf.level_items[l] : nullptr;
         D.ints = bf.ints;
-        D.dbl = bf.dbl;
+        D.words = bf.words();
         D.depth_parity = bf.depth_parity;
         D.nmaps = G.nmaps;
         void *d;
@@ -454,11 +454,9 @@ int build_schedule(shtb_batch_s *b, int warps, int width, int lpt)
     b->dev.err = b->dev.counters + ncounters + 1;
     b->dev.spin_limit = b->opts.spin_limit > 0 ? b->opts.spin_limit : 20000000LL;
     // level-item scratch per warp: the batch's longest candidate list x the
-    // most doubles per candidate any of its map groups needs (C + 1 from 4
-    // maps up, 2 C below; C = 2 x maps)
+    // components of its widest map group
     if (cmax > 16 || maxnc > shtb::kMaxCand) return shtb_fail(SHTB_EINVAL, "map group or candidate list too large");
-    b->dev.scratch = maxnc * std::max(shtb_dev::level_scratch_per_cand(cmax),
-                                      shtb_dev::level_scratch_per_cand(std::min(cmax, 4)));
+    b->dev.scratch = maxnc * cmax;
     b->ncounters = ncounters;
     b->stall_counter = 0;             // the first plan group's gather
     b->warps = warps;

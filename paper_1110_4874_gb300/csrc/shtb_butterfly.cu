@@ -7,13 +7,14 @@
 //   bf_level_kernel  one item = two sibling nodes sharing a candidate list:
 //                    v = T_top^T u_top + T_bot^T u_bot, split into the parent
 //                    level's two u vectors (or q^t on a leaf block at level 1);
-//                    identity part = adds, dense part = k x nd dot products
+//                    identity part = adds, dense part = k x nd products
 //                    (Appendix: the identity-embedded interpolation matrices);
 // and the ring stage of each map group then reads q_m(+z) = q^0 + q^1 and
 // q_m(-z) = q^0 - q^1 (Eq. q-even-odd2) straight from the two parity halves.
 // One warp per work item; all maps of a group (up to 8, 2 real components
 // each) are carried per entry so every stored matrix element is read once
-// per group and used for 2 x maps FMAs.  All stages are FP64-bound on GB300.
+// per group.  The dense products run on the tensor cores in exact fixed-point
+// digits (shtb_bf_fix.cuh).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -24,33 +25,7 @@
 
 namespace {
 
-using shtb_dev::Tile;
-
 constexpr int kBfWarps = 4;
-// with one or two maps, a warp takes this many consecutive level items or
-// residual blocks (their dot products packed on its lanes)
-constexpr int kBfLevelPack = 2;
-constexpr int kBfResidualPack = 8;
-
-template <int NB>
-__host__ __device__ constexpr int items_per_warp_level()
-{
-    return NB <= 2 ? kBfLevelPack : 1;
-}
-
-template <int NB>
-__host__ __device__ constexpr int items_per_warp_residual()
-{
-    return NB <= 2 ? kBfResidualPack : 1;
-}
-
-// level-item scratch of one warp (doubles)
-template <int NB>
-__host__ __device__ constexpr size_t level_scratch_doubles(int maxnc)
-{
-    return (size_t)items_per_warp_level<NB>() * maxnc * shtb_dev::level_scratch_per_cand(2 * NB);
-}
-
 
 // Staging between the caller's stacked a_lm [map][idx] and the butterfly's
 // interleaved ai [idx][map]: tiles of T coefficients x MB maps pass through
@@ -113,54 +88,35 @@ unsigned stage_grid(const shtb_plan_s *p, int nmaps)
 }
 
 template <int NB>
-__global__ void __launch_bounds__(32 * kBfWarps)
+__global__ void __launch_bounds__(32 * kBfWarps, 4)
 bf_r_kernel(PlanView v, const BfRItem *__restrict__ items, int nitems, const int *__restrict__ ints,
-            const double *__restrict__ dbl, const double2 *__restrict__ ai, int nmaps, int b0,
+            const uint2 *__restrict__ words, const double2 *__restrict__ ai, int nmaps, int b0,
             double *__restrict__ ubuf0, double *__restrict__ ubuf1, const int *__restrict__ depth_par,
             double *__restrict__ qt)
 {
     const int lane = threadIdx.x & 31;
     const int w = blockIdx.x * kBfWarps + (threadIdx.x >> 5);
-    if constexpr (NB <= 2) {
-        constexpr int G = kBfResidualPack;
-        const int i0 = w * G;
-        if (i0 >= nitems) return;
-        shtb_dev::bf_r_items_few<NB, G, false>(items + i0, min(G, nitems - i0), v.lmax, v.nhalf, ints, dbl, ai,
-                                               nmaps, b0, ubuf0, ubuf1, depth_par, qt, lane);
-        return;
-    }
     if (w >= nitems) return;
     const BfRItem it = items[w];
     double *ubuf = depth_par[it.m * 2 + it.t] ? ubuf1 : ubuf0;
-    shtb_dev::bf_r_item<NB, false>(it, v.lmax, v.nhalf, ints, dbl, ai, nmaps, b0, ubuf, qt, lane);
+    shtb_dev::bf_r_item<NB, false>(it, v.lmax, v.nhalf, ints, words, ai, nmaps, b0, ubuf, qt, lane);
 }
 
 // RING: the launch is the plan's level 1, whose items all write q^t (no
 // other level's do), so each instantiation holds one output path.
 template <int NB, bool RING>
-__global__ void __launch_bounds__(32 * kBfWarps, NB <= 2 ? 6 : 8)
+__global__ void __launch_bounds__(32 * kBfWarps, 4)
 bf_level_kernel(const BfItem *__restrict__ items, int nitems, int L, int nhalf, int maxnc,
-                const int *__restrict__ ints, const double *__restrict__ dbl,
+                const int *__restrict__ ints, const uint2 *__restrict__ words,
                 const double *__restrict__ uin, double *__restrict__ uout, double *__restrict__ qt)
 {
-    extern __shared__ double sout[];     // [kBfWarps][level_scratch_doubles<NB>(maxnc)]
+    extern __shared__ __align__(16) double sout[];     // [kBfWarps][maxnc * 2 NB]
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     const int w = blockIdx.x * kBfWarps + wib;
-    double *scr = sout + (size_t)wib * level_scratch_doubles<NB>(maxnc);
-    if constexpr (NB <= 2) {
-        constexpr int G = kBfLevelPack;
-        const int i0 = w * G;
-        if (i0 >= nitems) return;
-        const int n = min(G, nitems - i0);
-        BfItem it[G];
-#pragma unroll
-        for (int q = 0; q < G; ++q) it[q] = items[i0 + min(q, n - 1)];
-        shtb_dev::bf_level_items_few<NB, G, false>(it, n, L, nhalf, ints, dbl, uin, uout, qt, scr, maxnc, lane);
-        return;
-    }
     if (w >= nitems) return;
-    shtb_dev::bf_level_item<NB, false, RING ? 1 : 0>(items[w], L, nhalf, ints, dbl, uin, uout, qt, scr, lane);
+    shtb_dev::bf_level_item<NB, false, RING ? 1 : 0>(items[w], L, nhalf, ints, words, uin, uout, qt,
+                                                     sout + (size_t)wib * maxnc * 2 * NB, lane);
 }
 
 // regenerated residual blocks (residual_recurrence plans), one per warp
@@ -194,9 +150,8 @@ int launch_r(const shtb_plan_s *p, const double2 *ai, int nmaps, int b0, double 
         ++p->launches;
         return SHTB_OK;
     }
-    const long long warps = (bf.n_ritems + items_per_warp_residual<NB>() - 1) / items_per_warp_residual<NB>();
-    const unsigned grid = (unsigned)((warps + kBfWarps - 1) / kBfWarps);
-    bf_r_kernel<NB><<<grid, 32 * kBfWarps, 0, st>>>(p->view, bf.ritems, bf.n_ritems, bf.ints, bf.dbl, ai,
+    const unsigned grid = (unsigned)((bf.n_ritems + kBfWarps - 1) / kBfWarps);
+    bf_r_kernel<NB><<<grid, 32 * kBfWarps, 0, st>>>(p->view, bf.ritems, bf.n_ritems, bf.ints, bf.words(), ai,
                                                     nmaps, b0, u0, u1, bf.depth_parity, qt);
     SHTB_CUDA_TRY(cudaGetLastError());
     ++p->launches;
@@ -213,14 +168,13 @@ int launch_levels(const shtb_plan_s *p, double *u0, double *u1, double *qt, cuda
         if (n == 0) continue;
         double *uin = (lev % 2) ? u1 : u0;
         double *uout = ((lev - 1) % 2) ? u1 : u0;
-        const int warps = (n + items_per_warp_level<NB>() - 1) / items_per_warp_level<NB>();
-        const unsigned grid = (unsigned)((warps + kBfWarps - 1) / kBfWarps);
+        const unsigned grid = (unsigned)((n + kBfWarps - 1) / kBfWarps);
         const int maxnc = bf.level_maxnc[lev - 1];
-        const size_t smem = sizeof(double) * kBfWarps * level_scratch_doubles<NB>(maxnc);
+        const size_t smem = sizeof(double) * kBfWarps * maxnc * 2 * NB;
         auto *kern = lev == 1 ? bf_level_kernel<NB, true> : bf_level_kernel<NB, false>;
         SHTB_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         kern<<<grid, 32 * kBfWarps, smem, st>>>(bf.level_items[lev - 1], n, p->lmax, p->nhalf, maxnc, bf.ints,
-                                                bf.dbl, uin, uout, qt);
+                                                bf.words(), uin, uout, qt);
         SHTB_CUDA_TRY(cudaGetLastError());
         ++p->launches;
     }
@@ -274,171 +228,177 @@ __global__ void bf_gather_kernel(PlanView v, const double2 *const *__restrict__ 
 // level 1, else the u of level l-1) and applies both children's T:
 // u_s = [I | T_s] v  (identity entries copy, dense rows are k x nd dots).
 
-// NR rows of child s per lane, rows q0 + dl + r LD (r < NR), component c
-template <int NB, int NR>
-__device__ __forceinline__ void adj_rows(const BfItem &it, int s, const int *__restrict__ ints,
-                                         const double *__restrict__ dbl, const double *in, int q0, int dl,
-                                         int c, double *__restrict__ uout)
-{
-    constexpr int C = 2 * NB, LD = shtb_dev::Lanes<C>::LD;
-    const int k = it.k[s], nd = it.nd[s];
-    const double *__restrict__ T = dbl + it.T_off[s];        // k x nd, row-major
-    const int *__restrict__ dpos = ints + it.dpos_off[s];
-    const int *__restrict__ ipos = ints + it.ipos_off[s];
-    double acc[NR];
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-        const int i = q0 + dl + r * LD;
-        acc[r] = i < k ? in[ipos[i] * C + c] : 0.0;
-    }
-#pragma unroll 2
-    for (int d = 0; d < nd; ++d) {
-        const double x = in[dpos[d] * C + c];
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            const int i = q0 + dl + r * LD;
-            const double t = i < k ? T[(size_t)i * nd + d] : 0.0;
-            acc[r] = fma(t, x, acc[r]);
-        }
-    }
-    double *dst = uout + (size_t)it.u_off[s] * C + c;
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-        const int i = q0 + dl + r * LD;
-        if (i < k) dst[(size_t)i * C] = acc[r];
-    }
-}
+// The contraction runs over T's dense columns, so their exponents go onto
+// the candidates' values (shift) and the outputs have none.
 
-template <int NB, int NR>
-__device__ __forceinline__ void adj_rows_dispatch(int nr, const BfItem &it, int s, const int *ints,
-                                                  const double *dbl, const double *in, int q0, int dl, int c,
-                                                  double *uout)
-{
-    if constexpr (NR > 1) {
-        if (nr < NR) {
-            adj_rows_dispatch<NB, NR - 1>(nr, it, s, ints, dbl, in, q0, dl, c, uout);
+// a level item's candidate vector in shared memory, dense column d at dpos[d]
+template <int C>
+struct AdjLevelVec {
+    const double *in;
+    const int *dpos;
+    const uint2 *T;                     // the child's words: row 0 carries each column's exponent
+    template <int W>
+    __device__ __forceinline__ void load(int d, int i, double (&x)[W]) const
+    {
+        shtb_dev::ld_comps<shtb_dev::Ld::kPlain>(in + __ldg(dpos + d) * C, i, x);
+    }
+    __device__ __forceinline__ int shift(int d) const
+    {
+        const uint2 w = __ldg(T + d);
+        return shtb::fix_word_exp(w.x, w.y);
+    }
+    __device__ __forceinline__ double value(int d, int c) const { return in[dpos[d] * C + c]; }
+};
+
+// u_i: the identity entry plus the dense product (later chunks on top)
+template <int C>
+struct AdjLevelOut {
+    const double *in;
+    const int *ipos;
+    double *dst;
+    // output i and its identity entry's position (both below 2^15)
+    __device__ __forceinline__ int key(int i) const { return i << 16 | __ldg(ipos + i); }
+    template <int W>
+    __device__ __forceinline__ void put(int key, bool add, int c, const double (&v)[W]) const
+    {
+        double *d = dst + (size_t)(key >> 16) * C;
+        if (add) {
+            shtb_dev::st_comps(d, c, v, true);
             return;
         }
+        double x[W];
+        shtb_dev::ld_comps<shtb_dev::Ld::kPlain>(in + (key & 0xffff) * C, c, x);
+#pragma unroll
+        for (int q = 0; q < W; ++q) x[q] += v[q];
+        shtb_dev::st_comps(d, c, x, false);
     }
-    adj_rows<NB, NR>(it, s, ints, dbl, in, q0, dl, c, uout);
-}
+};
+
 template <int NB>
-__global__ void __launch_bounds__(32 * kBfWarps)
-bf_adj_level_kernel(const BfItem *__restrict__ items, int nitems, const int *__restrict__ ints,
-                    const double *__restrict__ dbl, const double *__restrict__ uin,
+__global__ void __launch_bounds__(32 * kBfWarps, 4)
+bf_adj_level_kernel(const BfItem *__restrict__ items, int nitems, int maxnc, const int *__restrict__ ints,
+                    const uint2 *__restrict__ words, const double *__restrict__ uin,
                     const double2 *__restrict__ g, int nmaps, int b0, double *__restrict__ uout)
 {
     constexpr int C = 2 * NB;
-    extern __shared__ double sin_[];     // [kBfWarps][kMaxCand * C]
+    extern __shared__ __align__(16) double sin_[];     // [kBfWarps][maxnc * C]
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     const int w = blockIdx.x * kBfWarps + wib;
     if (w >= nitems) return;
     const BfItem it = items[w];
-    double *in = sin_ + (size_t)wib * shtb::kMaxCand * C;
+    double *in = sin_ + (size_t)wib * maxnc * C;
+    double2 *in2 = reinterpret_cast<double2 *>(in);
     if (it.to_rings) {
         const int *__restrict__ ent = ints + it.out_off;
         for (int i = lane; i < it.nc * NB; i += 32) {
             const int cpos = i / NB, b = i - cpos * NB;
-            const double2 x = g[(size_t)ent[cpos] * nmaps + b0 + b];
-            in[cpos * C + 2 * b] = x.x;
-            in[cpos * C + 2 * b + 1] = x.y;
+            in2[i] = g[(size_t)ent[cpos] * nmaps + b0 + b];
         }
     } else {
-        const double *src = uin + (size_t)it.out_off * C;
-        for (int i = lane; i < it.nc * C; i += 32) in[i] = src[i];
+        const double2 *src = reinterpret_cast<const double2 *>(uin + (size_t)it.out_off * C);
+        for (int i = lane; i < it.nc * NB; i += 32) in2[i] = src[i];
     }
     __syncwarp();
-    // each child in turn, its k rows over the lanes (one component per lane,
-    // an exact per-lane row count): identity entry plus a dot product of the
-    // row of T with the candidates' dense part
-    using shtb_dev::Lanes;
-    constexpr int LD = Lanes<C>::LD, NRMAX = Lanes<C>::NRMAX;
-    const int dl = lane % LD, c = lane / LD;
-#pragma unroll
+#pragma unroll 1
     for (int s = 0; s < 2; ++s) {
-        const int k = it.k[s];
-        for (int q0 = 0; q0 < k; q0 += LD * NRMAX) {
-            const int nr = min(NRMAX, (k - q0 + LD - 1) / LD);
-            adj_rows_dispatch<NB, NRMAX>(nr, it, s, ints, dbl, in, q0, dl, c, uout);
+        const int k = it.k[s], nd = it.nd[s];
+        if (k == 0) continue;
+        const uint2 *T = words + it.T_off[s];
+        const int *__restrict__ ipos = ints + it.ipos_off[s];
+        double *dst = uout + (size_t)it.u_off[s] * C;
+        if (nd == 0) {                  // identity entries alone
+            for (int i = lane; i < k * C; i += 32) dst[i] = in[ipos[i / C] * C + i % C];
+            continue;
         }
+        const AdjLevelVec<C> vec{in, ints + it.dpos_off[s], T};
+        const AdjLevelOut<C> out{in, ipos, dst};
+        shtb_dev::fix_product<C, false>(T, 1, nd, nd, k, vec, out, lane);
     }
 }
 
-// NR rows per lane of one (chain, row interval) group, rows j0 + dl + r LD
-// (r < NR), component c: a_j = sum over the group's residual blocks of
-// R[j, :] x, x the block's u (or g at depth 0)
-template <int NB, int NR>
-__device__ __forceinline__ void adj_r_rows(const BfRGroup &gr, const BfRItem *__restrict__ ritems,
-                                           const int *__restrict__ ints, const double *__restrict__ dbl,
-                                           const double *ubuf, const double *gd, int nmaps, int b0, int j0,
-                                           int dl, int c, double *ad, long long aoff)
-{
-    constexpr int C = 2 * NB, LD = shtb_dev::Lanes<C>::LD;
-    double acc[NR];
-#pragma unroll
-    for (int r = 0; r < NR; ++r) acc[r] = 0.0;
-    const int jend = min(gr.r1, j0 + NR * LD);
-    for (int q = 0; q < gr.nblk; ++q) {
-        const BfRItem it = ritems[ints[gr.blk_off + q]];
-        if (it.j0 >= jend || it.j0 + it.nrows <= j0) continue;       // no row of this pass
-        const double *__restrict__ R = dbl + it.data_off;
-        for (int s = 0; s < it.k; ++s) {
-            const double x = it.to_rings ? __ldg(gd + ((size_t)ints[it.out_off + s] * nmaps + b0) * 2 + c)
-                                         : __ldg(ubuf + (size_t)(it.out_off + s) * C + c);
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const int j = j0 + dl + r * LD;
-                const bool in_blk = j >= it.j0 && j < it.j0 + it.nrows;
-                const double t = in_blk ? R[(size_t)(j - it.j0) * it.k + s] : 0.0;
-                acc[r] = fma(t, x, acc[r]);
-            }
-        }
+// a residual block's u (or g at depth 0), column s of R
+template <int C>
+struct AdjResVec {
+    const double *u;                    // u entries, or null: g entries ent
+    const double *g;                    // component 0 of the group in g[entry][nmaps]
+    const int *ent;
+    int gstride;
+    const uint2 *R;                     // row 0 carries each column's exponent
+    __device__ __forceinline__ const double *at(int s) const
+    {
+        return u ? u + (size_t)s * C : g + (size_t)__ldg(ent + s) * gstride;
     }
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-        const int j = j0 + dl + r * LD;
-        if (j < gr.r1) ad[((size_t)(aoff + 2 * j) * nmaps + b0) * 2 + c] = acc[r];
+    template <int W>
+    __device__ __forceinline__ void load(int s, int i, double (&x)[W]) const
+    {
+        shtb_dev::ld_comps<shtb_dev::Ld::kGlobal>(at(s), i, x);
     }
-}
+    __device__ __forceinline__ int shift(int s) const
+    {
+        const uint2 w = __ldg(R + s);
+        return shtb::fix_word_exp(w.x, w.y);
+    }
+    __device__ __forceinline__ double value(int s, int c) const { return at(s)[c]; }
+};
 
-template <int NB, int NR>
-__device__ __forceinline__ void adj_r_dispatch(int nr, const BfRGroup &gr, const BfRItem *ritems,
-                                               const int *ints, const double *dbl, const double *ubuf,
-                                               const double *gd, int nmaps, int b0, int j0, int dl, int c,
-                                               double *ad, long long aoff)
-{
-    if constexpr (NR > 1) {
-        if (nr < NR) {
-            adj_r_dispatch<NB, NR - 1>(nr, gr, ritems, ints, dbl, ubuf, gd, nmaps, b0, j0, dl, c, ad, aoff);
-            return;
-        }
+template <int C>
+struct AdjResOut {
+    double *acc;
+    __device__ __forceinline__ int key(int n) const { return n; }
+    template <int W>
+    __device__ __forceinline__ void put(int n, bool, int i, const double (&v)[W]) const
+    {
+        shtb_dev::st_comps(acc + n * C, i, v, true);
     }
-    adj_r_rows<NB, NR>(gr, ritems, ints, dbl, ubuf, gd, nmaps, b0, j0, dl, c, ad, aoff);
-}
+};
 
-// a rows of one (chain, row interval): every row of the interval is written
-// (zero when no block reaches it), so each chain row has exactly one writer
+// a rows of one (chain, row interval), kAdjRows at a time in shared memory:
+// a_j = sum over the group's residual blocks of R[j, :] x.  Every row of the
+// interval is written (zero when no block reaches it), so each chain row has
+// exactly one writer.  32 rows hold most intervals (25 on average), and a
+// longer pass would cost resident warps their shared memory.
+constexpr int kAdjRows = 32;
+
 template <int NB>
-__global__ void __launch_bounds__(32 * kBfWarps)
+__global__ void __launch_bounds__(32 * kBfWarps, 4)
 bf_adj_r_kernel(PlanView v, const BfRGroup *__restrict__ groups, int ngroups,
                 const BfRItem *__restrict__ ritems, const int *__restrict__ ints,
-                const double *__restrict__ dbl, const double *__restrict__ u0,
+                const uint2 *__restrict__ words, const double *__restrict__ u0,
                 const double *__restrict__ u1, const int *__restrict__ depth_par,
                 const double2 *__restrict__ g, int nmaps, int b0, double2 *__restrict__ aacc)
 {
-    constexpr int C = 2 * NB, LD = shtb_dev::Lanes<C>::LD, NRMAX = shtb_dev::Lanes<C>::NRMAX;
+    constexpr int C = 2 * NB;
+    __shared__ __align__(16) double srow[kBfWarps][kAdjRows * C];
     const int lane = threadIdx.x & 31;
     const int w = blockIdx.x * kBfWarps + (threadIdx.x >> 5);
     if (w >= ngroups) return;
+    double *acc = srow[threadIdx.x >> 5];
+    double2 *acc2 = reinterpret_cast<double2 *>(acc);
     const BfRGroup gr = groups[w];
     const double *ubuf = depth_par[gr.m * 2 + gr.t] ? u1 : u0;
     const long long aoff = shtb_dev::alm_off(v.lmax, gr.m) + gr.t;
-    const int dl = lane % LD, c = lane / LD;
-    for (int j0 = gr.r0; j0 < gr.r1; j0 += LD * NRMAX) {
-        const int nr = min(NRMAX, (gr.r1 - j0 + LD - 1) / LD);
-        adj_r_dispatch<NB, NRMAX>(nr, gr, ritems, ints, dbl, ubuf, reinterpret_cast<const double *>(g), nmaps,
-                                  b0, j0, dl, c, reinterpret_cast<double *>(aacc), aoff);
+    for (int j0 = gr.r0; j0 < gr.r1; j0 += kAdjRows) {
+        const int nj = min(kAdjRows, gr.r1 - j0);
+        for (int i = lane; i < nj * NB; i += 32) acc2[i] = make_double2(0.0, 0.0);
+        __syncwarp();
+        for (int q = 0; q < gr.nblk; ++q) {
+            const BfRItem it = ritems[ints[gr.blk_off + q]];
+            const int ja = max(j0, it.j0), jb = min(j0 + nj, it.j0 + it.nrows);
+            if (ja >= jb) continue;                    // no row of this pass
+            const uint2 *R = words + it.data_off;
+            const AdjResVec<C> vec{it.to_rings ? nullptr : ubuf + (size_t)it.out_off * C,
+                                   reinterpret_cast<const double *>(g + b0), it.to_rings ? ints + it.out_off : nullptr,
+                                   2 * nmaps, R};
+            const AdjResOut<C> out{acc + (ja - j0) * C};
+            shtb_dev::fix_product<C, false>(R + (size_t)(ja - it.j0) * it.k, 1, it.k, it.k, jb - ja, vec, out, lane);
+            __syncwarp();
+        }
+        for (int i = lane; i < nj * NB; i += 32) {
+            const int j = i / NB, b = i - j * NB;
+            aacc[(size_t)(aoff + 2 * (j0 + j)) * nmaps + b0 + b] = acc2[i];
+        }
+        __syncwarp();
     }
 }
 
@@ -512,11 +472,12 @@ int run_adj_group(const shtb_plan_s *p, const double2 *g, int nmaps, int b0, dou
         const double *uin = ((lev - 1) % 2) ? u1 : u0;
         double *uout = (lev % 2) ? u1 : u0;
         const unsigned grid = (unsigned)((n + kBfWarps - 1) / kBfWarps);
-        const size_t smem = sizeof(double) * kBfWarps * shtb::kMaxCand * 2 * NB;
+        const int maxnc = bf.level_maxnc[lev - 1];
+        const size_t smem = sizeof(double) * kBfWarps * maxnc * 2 * NB;
         SHTB_CUDA_TRY(cudaFuncSetAttribute(bf_adj_level_kernel<NB>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        bf_adj_level_kernel<NB><<<grid, 32 * kBfWarps, smem, st>>>(bf.level_items[lev - 1], n, bf.ints,
-                                                                   bf.dbl, uin, g, nmaps, b0, uout);
+        bf_adj_level_kernel<NB><<<grid, 32 * kBfWarps, smem, st>>>(bf.level_items[lev - 1], n, maxnc, bf.ints,
+                                                                   bf.words(), uin, g, nmaps, b0, uout);
         SHTB_CUDA_TRY(cudaGetLastError());
         ++p->launches;
     }
@@ -533,7 +494,7 @@ int run_adj_group(const shtb_plan_s *p, const double2 *g, int nmaps, int b0, dou
     } else if (bf.n_rgroups > 0) {
         const unsigned grid = (unsigned)((bf.n_rgroups + kBfWarps - 1) / kBfWarps);
         bf_adj_r_kernel<NB><<<grid, 32 * kBfWarps, 0, st>>>(p->view, bf.rgroups, bf.n_rgroups, bf.ritems,
-                                                            bf.ints, bf.dbl, u0, u1, bf.depth_parity, g,
+                                                            bf.ints, bf.words(), u0, u1, bf.depth_parity, g,
                                                             nmaps, b0, aacc);
         SHTB_CUDA_TRY(cudaGetLastError());
         ++p->launches;
@@ -541,7 +502,77 @@ int run_adj_group(const shtb_plan_s *p, const double2 *g, int nmaps, int b0, dou
     return SHTB_OK;
 }
 
+// ------------------------------------------------ stored elements as words
+// One warp per block of rows x cols doubles (row-major), a lane per column:
+// the column's largest element sets its exponent, then every element becomes
+// its word (shtb_fix.h) in place.  Runs once, when a plan is built or read.
+__device__ __forceinline__ void pack_block(double *blk, int rows, int cols, int lane, int *err)
+{
+    for (int c = lane; c < cols; c += 32) {
+        double big = 0.0;
+        bool bad = false;
+        for (int r = 0; r < rows; ++r) {
+            const double v = fabs(blk[(size_t)r * cols + c]);
+            bad |= !(v < 1.8e308);
+            big = fmax(big, v);
+        }
+        int E = 0;
+        if (big > 0.0) frexp(big, &E);                 // 2^(E-1) <= big < 2^E
+        else E = -shtb::kFixExpBias;
+        if (bad || E > shtb::kFixExpMax) {
+            *err = 1;
+            continue;
+        }
+        E = max(E, -shtb::kFixExpBias);
+        const double scale = shtb::pow2(54 - E);
+        for (int r = 0; r < rows; ++r) {
+            double *p = blk + (size_t)r * cols + c;
+            const long long X = __double2ll_rn(*p * scale) * 16;
+            *p = __longlong_as_double((long long)shtb::fix_word(X, E + shtb::kFixExpBias));
+        }
+    }
+}
+
+__global__ void pack_r_kernel(const BfRItem *__restrict__ items, int n, double *dbl, int *err)
+{
+    const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (w < n) pack_block(dbl + items[w].data_off, items[w].nrows, items[w].k, threadIdx.x & 31, err);
+}
+
+__global__ void pack_level_kernel(const BfItem *__restrict__ items, int n, double *dbl, int *err)
+{
+    const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (w >= 2 * n) return;
+    const BfItem &it = items[w >> 1];
+    const int s = w & 1;
+    pack_block(dbl + it.T_off[s], it.k[s], it.nd[s], threadIdx.x & 31, err);
+}
+
 }  // namespace
+
+int bf_pack_operator(shtb_plan_s *p)
+{
+    const BfPlanDev &bf = *p->bf;
+    double *dbl = const_cast<double *>(bf.dbl);
+    int *err = nullptr, bad = 0;
+    SHTB_CUDA_TRY(cudaMalloc(&err, sizeof(int)));
+    cudaError_t e = cudaMemset(err, 0, sizeof(int));
+    if (e == cudaSuccess && !bf.rec && bf.n_ritems > 0) {
+        pack_r_kernel<<<(unsigned)((bf.n_ritems + 7) / 8), 256>>>(bf.ritems, bf.n_ritems, dbl, err);
+        e = cudaGetLastError();
+    }
+    for (int l = 0; l < bf.depth_max && e == cudaSuccess; ++l) {
+        const int n = bf.level_counts[l];
+        if (n == 0) continue;
+        pack_level_kernel<<<(unsigned)((2LL * n + 7) / 8), 256>>>(bf.level_items[l], n, dbl, err);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(&bad, err, sizeof(int), cudaMemcpyDeviceToHost);
+    cudaFree(err);
+    if (e != cudaSuccess) return shtb_fail(SHTB_ECUDA, std::string("packing the operator: ") + cudaGetErrorString(e));
+    if (bad) return shtb_fail(SHTB_ENOTSUP, "operator element not finite or above 2^64");
+    return SHTB_OK;
+}
 
 size_t bf_workspace_bytes(const shtb_plan_s *p)
 {

@@ -122,7 +122,8 @@ struct BfPlanDev {
     std::vector<int> level_counts;
     std::vector<int> level_maxnc;               // largest candidate list per level
     const int *ints = nullptr;
-    const double *dbl = nullptr;
+    const double *dbl = nullptr;         // R and T blocks: the words of shtb_fix.h, 8 bytes an element
+    const uint2 *words() const { return reinterpret_cast<const uint2 *>(dbl); }
     const int *depth_parity = nullptr;   // per chain (m*2 + t): depth % 2 (u buffer of its R output)
     const RecStart *rstart = nullptr;    // regenerated R: one per (block, column)
     bool rec = false;                    // R regenerated by the recurrence, not stored
@@ -139,3 +140,5 @@ RecStart block_column_start(int n, int t, int j0, int nrows, int ring, double x,
 
 // Builds the compressed operator of a plan (eps > 0) and uploads it.
 int shtb_build_butterfly(shtb_plan_s *p);
+// The uploaded R and T blocks from doubles to fixed-point words, in place.
+int bf_pack_operator(shtb_plan_s *p);

@@ -685,8 +685,8 @@ int shtb_build_butterfly(shtb_plan_s *p)
             if ((l == 0) != (it.to_rings != 0))
                 return shtb_fail(SHTB_ENOTSUP, "butterfly item writing q^t outside level 1");
     // longest items first within each launch, so that the last wave is
-    // short; items of similar shape end up adjacent, which is what the
-    // few-map kernels need when they pack consecutive items on one warp
+    // short; items of similar shape end up adjacent, so a block's warps
+    // finish together
     std::vector<int> rord(ritems.size());
     std::iota(rord.begin(), rord.end(), 0);
     std::stable_sort(rord.begin(), rord.end(), [&](int a, int b) {
@@ -725,8 +725,8 @@ int shtb_build_butterfly(shtb_plan_s *p)
         });
     }
     // level items: heaviest first (a short last wave), then within runs of
-    // 64 by longest child input and most dense rows, so that adjacent items
-    // (which the few-map kernels pack on one warp) have similar shapes
+    // 64 by longest child input and most dense rows, so that a block's warps
+    // have similar shapes
     for (auto &lv : litems) {
         std::stable_sort(lv.begin(), lv.end(), [](const BfItem &a, const BfItem &b) {
             return (long long)a.k[0] * a.nd[0] + (long long)a.k[1] * a.nd[1] >
@@ -778,6 +778,7 @@ int shtb_build_butterfly(shtb_plan_s *p)
         bf->level_items[l] = (const BfItem *)d;
         bf->level_counts[l] = (int)litems[l].size();
     }
+    if ((rc = bf_pack_operator(p))) return rc;
     p->stats.n_dense = n_dense;
     p->stats.n_rstored = n_r;
     p->stats.n_rgen = n_rgen;

@@ -203,7 +203,9 @@ void profile_end(shtb_plan_s *p, cudaStream_t st, int stage, int ev);
 // Fills every host-side table and uploads it; defined in shtb_plan_host.cpp.
 int shtb_build_dense_plan(shtb_plan_s *p);
 
-// Device allocation helper that registers the pointer with the plan.
+// Device allocation helper that registers the pointer with the plan; each
+// allocation has kPlanSlack bytes more than it is asked for.
+constexpr size_t kPlanSlack = 8 * 128 * 8;
 int plan_alloc_upload(shtb_plan_s *p, void **dst, const void *src, size_t bytes);
 
 // Plan cache files (shtb_plan_cache.cpp): write a built plan; fill a fresh

@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "shtb_butterfly.h"
+#include "shtb_fix.h"
 #include "shtb_internal.h"
 
 namespace {
@@ -155,6 +156,14 @@ bool write_payload(Writer &w, shtb_plan_s *p)
         w.val(n);
         buf.resize(n);
         if (cudaMemcpy(buf.data(), p->allocations[i], n, cudaMemcpyDeviceToHost) != cudaSuccess) return false;
+        if (p->bf && p->allocations[i] == (const void *)p->bf->dbl) {     // files hold the blocks as doubles
+            for (uint64_t k = 0; k + 8 <= n; k += 8) {
+                uint64_t word;
+                memcpy(&word, buf.data() + k, 8);
+                const double v = shtb::fix_unpack(word);
+                memcpy(buf.data() + k, &v, 8);
+            }
+        }
         w.raw(buf.data(), n);
     }
     // the plan's device pointers as allocation indices (0 = null)
@@ -298,6 +307,9 @@ int plan_load(shtb_plan_s *p, const char *path)
     fclose(f);
     if (!complete || r.sum.h != h.checksum)
         return shtb_fail(SHTB_ECORRUPT, std::string("plan file failed its size or checksum check: ") + path);
+    // the item lists are trusted from here on
+    if (p->bf && (rc = bf_pack_operator(p))) return rc;
+    if (p->partner && p->partner->bf && (rc = bf_pack_operator(p->partner))) return rc;
     return SHTB_OK;
 }
 

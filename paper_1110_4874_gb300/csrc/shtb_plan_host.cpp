@@ -487,7 +487,9 @@ int plan_alloc_upload(shtb_plan_s *p, void **dst, const void *src, size_t bytes)
 {
     void *d = nullptr;
     size_t nb = bytes ? bytes : 16;
-    cudaError_t e = cudaMalloc(&d, nb);
+    // the block products read up to 7 rows of at most 128 words past a block
+    // (against zero digits): the last block's are in this slack
+    cudaError_t e = cudaMalloc(&d, nb + kPlanSlack);
     if (e != cudaSuccess)
         return shtb_fail(SHTB_ENOMEM, std::string("cudaMalloc plan table: ") + cudaGetErrorString(e));
     p->allocations.push_back(d);
