@@ -119,7 +119,7 @@ __device__ void gather_item(const BatchDev &bd, const BatchWork &w, int lane)
 
 // one ring of one map of a map group, by the whole block, from the group's
 // parity halves (fused combine, as in phi_synth_qt_kernel)
-__device__ void ring_item(const BatchDev &bd, const BatchWork &w, double2 *sm)
+__device__ void ring_item(const BatchDev &bd, const BatchWork &w, shtb_dev::fx2 *sm)
 {
     const BatchGroupDev &G = bd.groups[w.g];
     const BatchMG &M = bd.mgs[w.mg];
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(256, 2) batch_kernel(BatchDev bd)
         __syncthreads();
         if (s_abort) return;
         if (P.block) {
-            ring_item(bd, bd.work[P.first], reinterpret_cast<double2 *>(bsm));
+            ring_item(bd, bd.work[P.first], reinterpret_cast<shtb_dev::fx2 *>(bsm));
         } else if (wib < P.count) {
             const BatchWork w = bd.work[P.first + wib];
             if (w.type == W_GATHER) {
@@ -460,7 +460,7 @@ int build_schedule(shtb_batch_s *b, int warps, int width, int lpt)
     b->ncounters = ncounters;
     b->stall_counter = 0;             // the first plan group's gather
     b->warps = warps;
-    b->smem = std::max(sizeof(double2) * ring_entries, sizeof(double) * (size_t)warps * b->dev.scratch);
+    b->smem = std::max((sizeof(shtb_dev::fx2) + sizeof(short)) * ring_entries + 16, sizeof(double) * (size_t)warps * b->dev.scratch);
     if (b->smem > 227 * 1024) return shtb_fail(SHTB_ENOTSUP, "batch kernel shared memory above 227 KB");
     SHTB_CUDA_TRY(cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem));
     int per_sm = 0, nsm = 0;

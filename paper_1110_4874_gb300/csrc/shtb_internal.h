@@ -199,6 +199,16 @@ struct shtb_plan_s {
 int profile_begin(shtb_plan_s *p, cudaStream_t st);
 void profile_end(shtb_plan_s *p, cudaStream_t st, int stage, int ev);
 
+// ------------------------------------------------- ring tables (shtb_phi.cu)
+// The complex tables that the device holds as fixed-point halves
+// (shtb_ring_fix.h), and their units; the uploaded doubles to halves, in place.
+struct RingTable {
+    const double2 *table;
+    int bits;
+};
+std::vector<RingTable> ring_tables(const shtb_plan_s *p);
+int ring_pack_tables(shtb_plan_s *p);
+
 // ------------------------------------------------------- host plan build
 // Fills every host-side table and uploads it; defined in shtb_plan_host.cpp.
 int shtb_build_dense_plan(shtb_plan_s *p);
@@ -231,8 +241,9 @@ int launch_adjoint_parity(const shtb_plan_s *p, const double2 *qadj, double2 *g,
 size_t legendre_adjoint_state_bytes(const shtb_plan_s *p);
 
 // shtb_phi.cu
+// one_stream: no side streams (the allocation-free call creates none)
 int launch_phi_synth(const shtb_plan_s *p, const double2 *q, double *map, int nmaps,
-                     cudaStream_t st);
+                     cudaStream_t st, bool one_stream = false);
 int launch_phi_adjoint(const shtb_plan_s *p, const double *map, double2 *q, int nmaps,
                        cudaStream_t st);
 int launch_phi_synth_qt(const shtb_plan_s *p, const double *qt, int nb, double *map, int b0,

@@ -88,5 +88,5 @@ extern "C" int shtb_synthesize_noalloc(shtb_plan p, const double *alm_dev, doubl
     cudaStream_t st = (cudaStream_t)stream;
     if ((rc = launch_alm_prescale(p, (const double2 *)alm_dev, ap, nmaps, st))) return rc;
     if ((rc = launch_legendre_synth(p, ap, q, nmaps, st))) return rc;
-    return launch_phi_synth(p, q, map_dev, nmaps, st);
+    return launch_phi_synth(p, q, map_dev, nmaps, st, true);
 }

@@ -10,13 +10,16 @@
 // of length K: Z_k = E_k + i e^{2 pi i k/J} O_k with E_k = g_k + g_{k+K},
 // O_k = g_k - g_{k+K}; then z_n = sum_k Z_k e^{2 pi i k n / K} holds the
 // pixels as f_{2n} + i f_{2n+1}.
-// One CTA per (ring, map); the ring's data live in shared memory.  K factoring
+// One CTA per (ring, map); the ring's data live in shared memory, as 64-bit
+// fixed-point numbers (shtb_phi_items.cuh).  K factoring
 // over 2, 3, 5, 7, 11, 13: in-place mixed-radix FFT (radices 4, 2, 3, 5, 7,
 // 11, 13) from position-order input.  Otherwise Bluestein's chirp transform
 // through a convolution of 7-smooth length M >= 2K-1 (decimation in
 // frequency, pointwise product with a precomputed filter in position order,
 // decimation in time), so no permutation pass is needed.
 #include <cuda_runtime.h>
+
+#include <vector>
 
 #include "shtb_internal.h"
 #include "shtb_phi_items.cuh"
@@ -27,30 +30,29 @@ using namespace shtb_dev;
 
 // threads per ring CTA: the Bluestein variant holds up to ~8.4k complex
 // values of shared memory per CTA (one CTA per SM at the longest rings), so
-// it runs twice the threads to keep the FP64 pipe fed
+// it runs twice the threads
 template <int KIND>
 constexpr int phi_threads()
 {
     return KIND == kBluestein ? 512 : 256;
 }
 
-// CTAs per SM the synthesis kernels are compiled for: the common mixed-radix
-// kind fits in 64 registers without spilling, so four share an SM wherever
-// their shared memory allows it (transforms of up to 3.5k points); the
-// radix-11/13 kind keeps two per SM (128 registers) and Bluestein one (512
-// threads).  The adjoint kernels need more registers and keep the default.
+// CTAs per SM the ring kernels are compiled for: four of the common
+// mixed-radix kind (64 registers; three, at 84, measured 1.20 against 1.14 ms
+// for the ring stage of 8 maps at Nside = 512), two of the radix-11/13 kind
+// and one of Bluestein's (128 registers)
 template <int KIND>
-constexpr int phi_synth_min_blocks()
+constexpr int phi_min_blocks()
 {
     return KIND == kDirect ? 4 : KIND == kDirectBig ? 2 : 1;
 }
 
 template <int KIND>
-__global__ void __launch_bounds__(phi_threads<KIND>(), phi_synth_min_blocks<KIND>())
+__global__ void __launch_bounds__(phi_threads<KIND>(), phi_min_blocks<KIND>())
 phi_synth_kernel(PlanView v, const int *__restrict__ rings, const double2 *__restrict__ q,
                  double *__restrict__ map)
 {
-    extern __shared__ double2 sm[];
+    extern __shared__ fx2 sm[];
     const int ring = rings[blockIdx.x];
     const int b = blockIdx.y;
     shtb_dev::phi_synth_ring<KIND, false>(v, ring, q + ((size_t)b * v.nrings + ring) * (v.lmax + 1),
@@ -66,11 +68,11 @@ struct MapOut {
 };
 
 template <int KIND>
-__global__ void __launch_bounds__(phi_threads<KIND>(), phi_synth_min_blocks<KIND>())
+__global__ void __launch_bounds__(phi_threads<KIND>(), phi_min_blocks<KIND>())
 phi_synth_qt_kernel(PlanView v, const int *__restrict__ rings, const double2 *__restrict__ qt,
                     MapOut mo, int b0)
 {
-    extern __shared__ double2 sm[];
+    extern __shared__ fx2 sm[];
     const int ring = rings[blockIdx.x];
     const int b = blockIdx.y;
     double *base = mo.table ? mo.table[b0 + b] : mo.map + (size_t)(b0 + b) * v.npix;
@@ -78,54 +80,15 @@ phi_synth_qt_kernel(PlanView v, const int *__restrict__ rings, const double2 *__
 }
 
 template <int KIND>
-__global__ void __launch_bounds__(phi_threads<KIND>())
+__global__ void __launch_bounds__(phi_threads<KIND>(), phi_min_blocks<KIND>())
 phi_adjoint_kernel(PlanView v, const int *__restrict__ rings, const double *__restrict__ map,
                    double2 *__restrict__ qa)
 {
-    constexpr bool BLUE = KIND == kBluestein;
-    extern __shared__ double2 sm[];
+    extern __shared__ fx2 sm[];
     const int ring = rings[blockIdx.x];
     const int b = blockIdx.y;
-    const int L = v.lmax;
-    const int J = v.ring_J[ring], K = J / 2, s = v.ring_s[ring];
-    const double2 *__restrict__ T = v.tw + v.ring_tw[ring];
-    const int *__restrict__ rl = v.rad + v.ring_rad[ring];
-
-    // z_n = f_{2n} + i f_{2n+1}; forward DFT Zf_k = sum_n z_n e^{-2 pi i k n/K}
-    const double2 *in = reinterpret_cast<const double2 *>(map + (size_t)b * v.npix + v.ring_start[ring]);
-    for (int n = threadIdx.x; n < K; n += blockDim.x) {
-        const double2 z = in[n];
-        sm[n] = BLUE ? cconj(z) : z;     // Bluestein: forward = conj(inverse(conj))
-    }
-    if (BLUE) {
-        __syncthreads();
-        bluestein_mx<true>(sm, K, v.ring_mx[ring], T, v.mfb + v.ring_mfb[ring], rl,
-                           TwTable{v.mtw + v.ring_mtw[ring]});
-        for (int n = threadIdx.x; n < K; n += blockDim.x) sm[n] = cconj(sm[n]);
-        __syncthreads();
-    } else {
-        constexpr bool BIG = KIND == kDirectBig;
-        RaderCtx rc;
-        const RaderCtx *rcp = BIG ? rader_ctx(v, ring, K, sm, rc) : nullptr;
-        fft_mx_dif<BIG, BIG>(sm, K, K, rl, TwRing{T, J}, rcp);   // position order
-    }
-
-    // F_r = E'_r + e^{-2 pi i r/J} O'_r with E' = (Zf_r + conj Zf_{K-r})/2,
-    // O' = (Zf_r - conj Zf_{K-r})/(2i), K-periodic; then
-    // q_adj[m] = e^{-i pi m s / J} F_{m mod J}.
-    double2 *outq = qa + ((size_t)b * v.nrings + ring) * (L + 1);
-    for (int m = threadIdx.x; m <= L; m += blockDim.x) {
-        const int r = m % J;
-        const int rho = r < K ? r : r - K;
-        const int rho2 = rho == 0 ? 0 : K - rho;
-        const double2 A = BLUE ? sm[rho] : sm[fft_pos(rho, K, rl)];
-        const double2 B = cconj(BLUE ? sm[rho2] : sm[fft_pos(rho2, K, rl)]);
-        const double2 Ep = make_double2(0.5 * (A.x + B.x), 0.5 * (A.y + B.y));
-        const double2 D = make_double2(0.5 * (A.x - B.x), 0.5 * (A.y - B.y));   // (A - B)/2
-        const double2 Op = make_double2(D.y, -D.x);                             // D / i
-        const double2 F = cadd(Ep, cmul_conj(Op, ring_root(T, J, 2LL * r)));
-        outq[m] = s ? cmul_conj(F, ring_root(T, J, (long long)m)) : F;
-    }
+    shtb_dev::phi_adjoint_ring<KIND>(v, ring, map + (size_t)b * v.npix + v.ring_start[ring],
+                                     qa + ((size_t)b * v.nrings + ring) * (v.lmax + 1), sm);
 }
 
 // one launch per ring kind: grid (rings of that kind) x maps, shared memory
@@ -135,6 +98,10 @@ phi_adjoint_kernel(PlanView v, const int *__restrict__ rings, const double *__re
 // threads with shared memory for their own longest transform, so that two
 // CTAs share an SM and one's barriers between FFT passes are covered by the
 // other's work.  Every body loops over blockDim.x.
+// shared memory of a transform of `len` entries: the points and, while a
+// spectrum is folded, a 16-bit exponent for each
+size_t ring_smem_bytes(int len) { return (sizeof(fx2) + sizeof(short)) * (size_t)len + 16; }
+
 struct RingSet {
     const int *rings;
     int n, len;
@@ -156,15 +123,15 @@ int launch_parts(const shtb_plan_s *p, const RingSet &rs, const void *kernel, La
 {
     if (rs.n == 0) return SHTB_OK;
     SHTB_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(sizeof(double2) * (size_t)rs.len)));
+                                       (int)ring_smem_bytes(rs.len)));
     if (rs.split > 0) {
-        launch(rs.rings, rs.split, phi_threads<KIND>(), sizeof(double2) * (size_t)rs.len);
+        launch(rs.rings, rs.split, phi_threads<KIND>(), ring_smem_bytes(rs.len));
         SHTB_CUDA_TRY(cudaGetLastError());
         ++p->launches;
     }
     if (rs.split < rs.n) {
         launch(rs.rings + rs.split, rs.n - rs.split, phi_threads<KIND>() / 2,
-               sizeof(double2) * (size_t)rs.len_small);
+               ring_smem_bytes(rs.len_small));
         SHTB_CUDA_TRY(cudaGetLastError());
         ++p->launches;
     }
@@ -214,8 +181,14 @@ int side_by_side(const shtb_plan_s *p, cudaStream_t st, Blue blue, Direct direct
 }
 
 int launch_set(const shtb_plan_s *p, bool synth, const void *in, void *out, int nmaps,
-               cudaStream_t st)
+               cudaStream_t st, bool one_stream)
 {
+    if (one_stream) {
+        int rc;
+        if ((rc = launch_kind<kBluestein>(p, synth, in, out, nmaps, st))) return rc;
+        if ((rc = launch_kind<kDirect>(p, synth, in, out, nmaps, st))) return rc;
+        return launch_kind<kDirectBig>(p, synth, in, out, nmaps, st);
+    }
     return side_by_side(
         p, st, [&](cudaStream_t s2) { return launch_kind<kBluestein>(p, synth, in, out, nmaps, s2); },
         [&](cudaStream_t s2) { return launch_kind<kDirect>(p, synth, in, out, nmaps, s2); },
@@ -257,6 +230,16 @@ int launch_qt_all(const shtb_plan_s *p, const double *qt, int nb, MapOut mo, int
     return launch_qt_kind<kDirectBig>(p, q2, nb, mo, b0, st);
 }
 
+// Tables from doubles to halves, in place
+__global__ void ring_pack_kernel(double2 *t, size_t n, int bits)
+{
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const double2 v = t[i];
+        const int2 re = shtb_dev::ring_half_pack(v.x, bits), im = shtb_dev::ring_half_pack(v.y, bits);
+        reinterpret_cast<int4 *>(t)[i] = make_int4(re.x, re.y, im.x, im.y);
+    }
+}
+
 }  // namespace
 
 int launch_phi_synth_qt(const shtb_plan_s *p, const double *qt, int nb, double *map, int b0,
@@ -288,13 +271,32 @@ int launch_phi_synth_qt_ptr(const shtb_plan_s *p, const double *qt, int nb, doub
     return launch_qt_all(p, qt, nb, MapOut{nullptr, map_of_map}, b0, st);
 }
 
-int launch_phi_synth(const shtb_plan_s *p, const double2 *q, double *map, int nmaps, cudaStream_t st)
+int launch_phi_synth(const shtb_plan_s *p, const double2 *q, double *map, int nmaps, cudaStream_t st, bool one_stream)
 {
-    return launch_set(p, true, q, map, nmaps, st);
+    return launch_set(p, true, q, map, nmaps, st, one_stream);
 }
 
 int launch_phi_adjoint(const shtb_plan_s *p, const double *map, double2 *q, int nmaps,
                        cudaStream_t st)
 {
-    return launch_set(p, false, map, q, nmaps, st);
+    return launch_set(p, false, map, q, nmaps, st, false);
+}
+
+std::vector<RingTable> ring_tables(const shtb_plan_s *p)
+{
+    const PlanView &v = p->view;
+    return {{v.tw, shtb::kRootBits}, {v.mtw, shtb::kRootBits}, {v.mfb, shtb::kRootBits},
+            {v.rdr_dbl, shtb::kRootBits}, {v.ab, shtb::kFoldBits}};
+}
+
+int ring_pack_tables(shtb_plan_s *p)
+{
+    for (const RingTable &t : ring_tables(p))
+        for (size_t i = 0; i < p->allocations.size(); ++i) {
+            if (p->allocations[i] != (const void *)t.table) continue;
+            ring_pack_kernel<<<152 * 4, 256>>>((double2 *)p->allocations[i], p->alloc_bytes[i] / sizeof(double2), t.bits);
+            SHTB_CUDA_TRY(cudaGetLastError());
+        }
+    SHTB_CUDA_TRY(cudaDeviceSynchronize());
+    return SHTB_OK;
 }

@@ -1,27 +1,35 @@
-// Device bodies of the ring stage (Eq. sh-baseline, Eq. tau): complex
-// helpers, the mixed-radix and Bluestein FFTs in shared memory and the
-// per-ring synthesis used by the ring kernels of shtb_phi.cu and by the
+// Device bodies of the ring stage (Eq. sh-baseline, Eq. tau): the fold of a
+// ring's spectrum, its mixed-radix, Rader or Bluestein FFT in shared memory,
+// and the adjoint, used by the ring kernels of shtb_phi.cu and by the
 // persistent batch kernel of shtb_batch.cu.
+//
+// The transforms run in 64-bit fixed point.  An SM does 2 FP64 instructions a
+// clock but 56 32 x 32 + 64-bit multiply-adds and 61 64-bit additions, so a
+// complex product (12 multiply-adds on balanced 32-bit halves) costs 6 clocks
+// a warp where its four FP64 instructions cost 64, and an addition 1 where
+// FP64 takes 16.  A ring's points share one power of two: every pass first
+// shifts them up so that the largest component has 61 bits (its size is known
+// from the pass before: one OR a component, one shared-memory OR a warp) and
+// then works without overflow, rounding its results to whole units.  A pass
+// so adds an error of a few 2^-58 of the largest point, below the last place
+// of the FP64 numbers the ring is made from and turned into at the end.
+// Measured (Nside = 512, L = 1024, 8 maps; FP64 transforms before): ring
+// synthesis 1.80 -> 1.14 ms, adjoint 2.42 -> 1.16 ms; Nside = 1024: 7.60 ->
+// 3.90 and 9.79 -> 4.12 ms.  What bounds them now is the issue of integer
+// instructions (55 to 68 % of the slots at the direct lengths).
+// Rings whose values hold an infinity or a NaN, or lie outside 1e-217 ..
+// 1e204, are summed directly in FP64 (ring_direct_*), as such values spread.
 #pragma once
 
 #include <cuda_runtime.h>
 
+#include "shtb_bf_fix.cuh"
 #include "shtb_internal.h"
+#include "shtb_ring_fix.h"
 
 namespace shtb_dev {
 
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
-__device__ __forceinline__ double2 cmul(double2 a, double2 b)
-{
-    return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
-}
-__device__ __forceinline__ double2 cmul_conj(double2 a, double2 b)   // a * conj(b)
-{
-    return make_double2(fma(a.x, b.x, a.y * b.y), fma(a.y, b.x, -a.x * b.y));
-}
-__device__ __forceinline__ double2 times_i(double2 a) { return make_double2(-a.y, a.x); }
 
 // sign flips as integer operations on the sign bit (no FP64 instruction)
 __device__ __forceinline__ double dneg_if(double x, int neg)
@@ -33,23 +41,6 @@ __device__ __forceinline__ double2 cneg_if(double2 a, int neg)
     return make_double2(dneg_if(a.x, neg), dneg_if(a.y, neg));
 }
 __device__ __forceinline__ double2 cconj_i(double2 a) { return make_double2(a.x, dneg_if(a.y, 1)); }
-
-// e^{i pi n / J} for any integer n >= 0 from the half-circle table T (n < J)
-__device__ __forceinline__ double2 ring_root(const double2 *__restrict__ T, int J, long long n)
-{
-    long long k = n % (2LL * J);
-    if (k < J) return __ldg(T + k);
-    double2 t = __ldg(T + (k - J));
-    return make_double2(-t.x, -t.y);
-}
-
-// ... for 0 <= n < 2^31, in 32-bit integer arithmetic
-__device__ __forceinline__ double2 ring_root32(const double2 *__restrict__ T, int J, int n)
-{
-    const int k = n % (2 * J);
-    if (k < J) return __ldg(T + k);
-    return cneg_if(__ldg(T + (k - J)), 1);
-}
 
 template <bool CG>
 __device__ __forceinline__ double2 ldq(const double2 *p)
@@ -83,6 +74,92 @@ __device__ __forceinline__ double2 fold_G(QAt qat, int L, int J, int s, int r)
     return acc;
 }
 
+// ------------------------------------------------ fixed-point complex numbers
+typedef longlong2 fx2;
+
+__device__ __forceinline__ fx2 fadd(fx2 a, fx2 b) { return make_longlong2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ fx2 fsub(fx2 a, fx2 b) { return make_longlong2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ fx2 fconj(fx2 a) { return make_longlong2(a.x, -a.y); }
+__device__ __forceinline__ fx2 ftimes_i(fx2 a) { return make_longlong2(-a.y, a.x); }
+__device__ __forceinline__ fx2 fshl(fx2 a, int s) { return make_longlong2(a.x << s, a.y << s); }
+
+// a / 2^n to nearest (n >= 1)
+__device__ __forceinline__ long long rshift(long long a, int n) { return (a + (1LL << (n - 1))) >> n; }
+__device__ __forceinline__ fx2 frshift(fx2 a, int n) { return make_longlong2(rshift(a.x, n), rshift(a.y, n)); }
+
+// balanced halves, a = h 2^32 + l with l signed
+__device__ __forceinline__ void halves(long long a, int &h, int &l)
+{
+    l = (int)a;
+    h = (int)(a >> 32) - (l >> 31);
+}
+
+// table entries: {low, high} balanced halves of the real and the imaginary
+// part in units of 2^-62 (fold weights 2^-61; shtb_ring_fix.h)
+__device__ __forceinline__ int4 wneg_if(int4 w, bool neg)
+{
+    return neg ? make_int4(-w.x, -w.y, -w.z, -w.w) : w;
+}
+
+// a w / 4 (CONJ: a conj(w) / 4) for |a| < 2^61.5: the products of the high
+// halves, and of high and low halves over 2^32, both exact in 64 bits; those
+// of the low halves are below a quarter of a unit
+template <bool CONJ = false>
+__device__ __forceinline__ fx2 fmul(fx2 a, int4 w)
+{
+    int ah, al, bh, bl;
+    halves(a.x, ah, al);
+    halves(a.y, bh, bl);
+    const int cl = w.x, ch = w.y;
+    const int dl = CONJ ? -w.z : w.z, dh = CONJ ? -w.w : w.w, nl = CONJ ? w.z : -w.z, nh = CONJ ? w.w : -w.w;
+    long long P = (long long)ah * ch + (long long)bh * nh;
+    long long M = (1LL << 31) + (long long)ah * cl;
+    M += (long long)al * ch;
+    M += (long long)bh * nl;
+    M += (long long)bl * nh;
+    long long Q = (long long)ah * dh + (long long)bh * ch;
+    long long N = (1LL << 31) + (long long)ah * dl;
+    N += (long long)al * dh;
+    N += (long long)bh * cl;
+    N += (long long)bl * ch;
+    return make_longlong2(P + (M >> 32), Q + (N >> 32));
+}
+
+// bits of the largest component so far: the OR of the components' upper words
+// without their signs
+__device__ __forceinline__ unsigned fmag(fx2 a)
+{
+    const int x = (int)(a.x >> 32), y = (int)(a.y >> 32);
+    return (unsigned)(x ^ (x >> 31)) | (unsigned)(y ^ (y >> 31));
+}
+
+// The common power of two of a block's points, true value = x 2^e, and the
+// shared-memory slots in which a pass leaves its results' size for the next:
+// slot i is read after the barrier that ends pass i, filled during pass i,
+// and cleared during pass i + 1's predecessor, three slots in turn.
+struct FxScale {
+    unsigned *slot;                    // 3 words of shared memory
+    int i, e;
+    // after a pass's results: every thread's OR
+    __device__ __forceinline__ void leave(unsigned mag)
+    {
+        mag = __reduce_or_sync(0xffffffffu, mag);
+        if ((threadIdx.x & 31) == 0 && mag) atomicOr(slot + (i + 1) % 3, mag);
+    }
+    // before a pass: the barrier, and the shift that brings the largest
+    // component to 61 bits
+    __device__ __forceinline__ int enter()
+    {
+        __syncthreads();
+        i = (i + 1) % 3;
+        const unsigned m = slot[i];
+        if (threadIdx.x == 0) slot[(i + 2) % 3] = 0;
+        const int s = max(0, 61 - (m ? 64 - __clz((int)m) : 32));
+        e -= s;
+        return s;
+    }
+};
+
 // ------------------------------------------------ mixed-radix ring FFTs
 // A transform of length N = r_0 r_1 ... r_{n-1} (radices 2, 3, 4, 5, 7, 11,
 // 13; list rl = {n, r_0, .., r_{n-1}}) runs in place in shared memory in n
@@ -97,9 +174,11 @@ __device__ __forceinline__ double2 fold_G(QAt qat, int L, int J, int s, int r)
 // the fold writes straight to pos(k), and a Bluestein filter is stored in
 // position order.
 
-// e^{2 pi i k / R} for the odd radices, k < R: R = 3, 5, 7, 11, 13 at offsets
-// 0, 3, 8, 15, 26
-static __constant__ double kRootCos[39] = {
+// cos and sin of 2 pi k / R for the odd radices, k < R: R = 3, 5, 7, 11, 13
+// at offsets 0, 3, 8, 15, 26, in units of 2^-59 as {low, high} halves
+__device__ __forceinline__ constexpr double root_cos(int k)
+{
+    constexpr double t[39] = {
     1.00000000000000000e+00, -5.00000000000000000e-01, -5.00000000000000000e-01,
     1.00000000000000000e+00, 3.09016994374947451e-01, -8.09016994374947451e-01, -8.09016994374947451e-01,
     3.09016994374947451e-01,
@@ -112,7 +191,11 @@ static __constant__ double kRootCos[39] = {
     -3.54604887042535621e-01, -7.48510748171101081e-01, -9.70941817426052012e-01, -9.70941817426052012e-01,
     -7.48510748171101081e-01, -3.54604887042535621e-01, 1.20536680255323048e-01, 5.68064746731155812e-01,
     8.85456025653209911e-01};
-static __constant__ double kRootSin[39] = {
+    return t[k];
+}
+__device__ __forceinline__ constexpr double root_sin(int k)
+{
+    constexpr double t[39] = {
     0.00000000000000000e+00, 8.66025403784438597e-01, -8.66025403784438597e-01,
     0.00000000000000000e+00, 9.51056516295153531e-01, 5.87785252292473137e-01, -5.87785252292473137e-01,
     -9.51056516295153531e-01,
@@ -125,6 +208,11 @@ static __constant__ double kRootSin[39] = {
     9.35016242685414833e-01, 6.63122658240795193e-01, 2.39315664287557767e-01, -2.39315664287557767e-01,
     -6.63122658240795193e-01, -9.35016242685414833e-01, -9.92708874098053973e-01, -8.22983865893656352e-01,
     -4.64723172043768562e-01};
+    return t[k];
+}
+__device__ __forceinline__ constexpr long long root_fix(double x) { return (long long)(x * 0x1p59); }
+__device__ __forceinline__ constexpr int root_low(long long v) { return (int)(unsigned)(v & 0xffffffffLL); }
+__device__ __forceinline__ constexpr int root_high(long long v) { return (int)((v - root_low(v)) / (1LL << 32)); }
 
 template <int R>
 __device__ __forceinline__ constexpr int root_off()
@@ -132,123 +220,133 @@ __device__ __forceinline__ constexpr int root_off()
     return R == 3 ? 0 : R == 5 ? 3 : R == 7 ? 8 : R == 11 ? 15 : 26;
 }
 
-// y_q = sum_p a_p e^{S 2 pi i p q / R}, in place (S = +1 or -1)
-template <int R, int S>
-__device__ __forceinline__ void dft_small(double2 (&a)[R])
+// bits by which dft_small scales down
+template <int R>
+__device__ __forceinline__ constexpr int dft_bits()
 {
-    if constexpr (R == 2) {
-        const double2 u = a[0];
-        a[0] = cadd(u, a[1]);
-        a[1] = csub(u, a[1]);
-    } else if constexpr (R == 4) {
-        const double2 s0 = cadd(a[0], a[2]), s1 = csub(a[0], a[2]);
-        const double2 s2 = cadd(a[1], a[3]), d = csub(a[1], a[3]);
-        const double2 s3 = S > 0 ? times_i(d) : make_double2(d.y, -d.x);   // S i (a1 - a3)
-        a[0] = cadd(s0, s2);
-        a[1] = cadd(s1, s3);
-        a[2] = csub(s0, s2);
-        a[3] = csub(s1, s3);
-    } else {
-        // odd R: pair p with R - p, y_q = A_q + S i B_q, y_{R-q} = A_q - S i B_q
-        constexpr int H = (R - 1) / 2, O = root_off<R>();
-        double2 sp[H], dp[H];
-#pragma unroll
-        for (int p = 1; p <= H; ++p) {
-            sp[p - 1] = cadd(a[p], a[R - p]);
-            dp[p - 1] = csub(a[p], a[R - p]);
-        }
-        const double2 a0 = a[0];
-        double2 y0 = a0;
-#pragma unroll
-        for (int p = 0; p < H; ++p) y0 = cadd(y0, sp[p]);
-#pragma unroll
-        for (int q = 1; q <= H; ++q) {
-            double2 A = a0, B = make_double2(0.0, 0.0);
-#pragma unroll
-            for (int p = 1; p <= H; ++p) {
-                const double c = kRootCos[O + (p * q) % R], sn = kRootSin[O + (p * q) % R];
-                A.x = fma(sp[p - 1].x, c, A.x);
-                A.y = fma(sp[p - 1].y, c, A.y);
-                B.x = fma(dp[p - 1].x, sn, B.x);
-                B.y = fma(dp[p - 1].y, sn, B.y);
-            }
-            const double2 iB = S > 0 ? make_double2(-B.y, B.x) : make_double2(B.y, -B.x);
-            a[q] = cadd(A, iB);
-            a[R - q] = csub(A, iB);
-        }
-        a[0] = y0;
-    }
+    return R == 2 || R == 4 ? 0 : 5;
 }
 
-// s = a + w b, d = a - w b as s and 2a - s: six FP64 instructions (four
-// fused multiply-adds, two for d) instead of a complex product and two sums
-__device__ __forceinline__ void bfly_fma(double2 a, double2 b, double2 w, double2 &s, double2 &d)
+// y_q = 2^-dft_bits sum_p a_p e^{S 2 pi i p q / R}, in place (S = +1 or -1),
+// |a| < 2^59.5
+template <int R, int S>
+__device__ __forceinline__ void dft_small(fx2 (&a)[R])
 {
-    s.x = fma(w.x, b.x, fma(-w.y, b.y, a.x));
-    s.y = fma(w.x, b.y, fma(w.y, b.x, a.y));
-    d.x = fma(2.0, a.x, -s.x);
-    d.y = fma(2.0, a.y, -s.y);
+    if constexpr (R == 2) {
+        const fx2 u = a[0];
+        a[0] = fadd(u, a[1]);
+        a[1] = fsub(u, a[1]);
+    } else if constexpr (R == 4) {
+        const fx2 s0 = fadd(a[0], a[2]), s1 = fsub(a[0], a[2]);
+        const fx2 s2 = fadd(a[1], a[3]), d = fsub(a[1], a[3]);
+        a[0] = fadd(s0, s2);
+        a[2] = fsub(s0, s2);
+        // s1 +- S i d
+        const fx2 p = make_longlong2(s1.x - d.y, s1.y + d.x), m = make_longlong2(s1.x + d.y, s1.y - d.x);
+        a[1] = S > 0 ? p : m;
+        a[3] = S > 0 ? m : p;
+    } else {
+        // odd R: pair p with R - p, y_q = A_q + S i B_q, y_{R-q} = A_q - S i
+        // B_q; A and B are sums of products with constants, each kept as the
+        // sum of the high halves' products and of the mixed ones (at most 6
+        // terms below 2^60.3)
+        constexpr int H = (R - 1) / 2, O = root_off<R>();
+        int sh[H][2], sl[H][2], dh[H][2], dl[H][2];
+        fx2 y0 = make_longlong2(a[0].x >> 1, a[0].y >> 1);
+#pragma unroll
+        for (int p = 1; p <= H; ++p) {
+            const fx2 sp = fadd(a[p], a[R - p]), dp = fsub(a[p], a[R - p]);
+            halves(sp.x, sh[p - 1][0], sl[p - 1][0]);
+            halves(sp.y, sh[p - 1][1], sl[p - 1][1]);
+            halves(dp.x, dh[p - 1][0], dl[p - 1][0]);
+            halves(dp.y, dh[p - 1][1], dl[p - 1][1]);
+            y0.x += sp.x >> 1;
+            y0.y += sp.y >> 1;
+        }
+        const fx2 a0 = frshift(a[0], 5);
+#pragma unroll
+        for (int q = 1; q <= H; ++q) {
+            long long A[2], B[2];
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                long long Ph = 0, Pm = 1LL << 31, Qh = 0, Qm = 1LL << 31;
+#pragma unroll
+                for (int p = 1; p <= H; ++p) {
+                    const long long cs = root_fix(root_cos(O + (p * q) % R)), sn = root_fix(root_sin(O + (p * q) % R));
+                    Ph += (long long)sh[p - 1][c] * root_high(cs);
+                    Pm += (long long)sh[p - 1][c] * root_low(cs);
+                    Pm += (long long)sl[p - 1][c] * root_high(cs);
+                    Qh += (long long)dh[p - 1][c] * root_high(sn);
+                    Qm += (long long)dh[p - 1][c] * root_low(sn);
+                    Qm += (long long)dl[p - 1][c] * root_high(sn);
+                }
+                A[c] = (c ? a0.y : a0.x) + Ph + (Pm >> 32);
+                B[c] = Qh + (Qm >> 32);
+            }
+            const fx2 iB = S > 0 ? make_longlong2(-B[1], B[0]) : make_longlong2(B[1], -B[0]);
+            a[q] = make_longlong2(A[0] + iB.x, A[1] + iB.y);
+            a[R - q] = make_longlong2(A[0] - iB.x, A[1] - iB.y);
+        }
+        a[0] = frshift(y0, 4);
+    }
 }
 
 // one pass of radix R over Ntot points: back-to-back sequences of Nseq
-// points (Nseq a multiple of B), in blocks of B; tw(t) = e^{2 pi i t / Nseq}
+// points (Nseq a multiple of B), in blocks of B; tw(t) = e^{2 pi i t / Nseq};
+// s: the shift of FxScale::enter.  Returns the results' size; scales down by
+// pass_bits.
+template <int R, bool INV>
+__device__ __forceinline__ int pass_bits(int Ns)
+{
+    return 2 + dft_bits<R>() + (!INV && Ns > 1 ? 2 : 0);
+}
+
 template <int R, bool INV, class TW>
-__device__ __forceinline__ void mx_pass(double2 *x, int Ntot, int Nseq, int B, const TW &tw)
+__device__ __forceinline__ unsigned mx_pass(fx2 *x, int Ntot, int Nseq, int B, const TW &tw, int s)
 {
     const int Ns = B / R, step = Nseq / B;
-    if constexpr (INV) {
-        if (Ns == 1) {
-            // the first pass of decimation in time: every twiddle is 1, so
-            // only the R-point DFT remains (16 adds for radix 4, not 24 FMAs)
-            for (int t = threadIdx.x; t < Ntot / R; t += blockDim.x) {
-                double2 a[R];
+    unsigned mag = 0;
+    if (Ns == 1) {
+        // the first pass of decimation in time, the last of decimation in
+        // frequency: every twiddle is 1
+        for (int t = threadIdx.x; t < Ntot / R; t += blockDim.x) {
+            fx2 a[R];
 #pragma unroll
-                for (int q = 0; q < R; ++q) a[q] = x[t * R + q];
-                dft_small<R, 1>(a);
+            for (int q = 0; q < R; ++q) a[q] = frshift(fshl(x[t * R + q], s), 2);
+            dft_small<R, INV ? 1 : -1>(a);
 #pragma unroll
-                for (int q = 0; q < R; ++q) x[t * R + q] = a[q];
+            for (int q = 0; q < R; ++q) {
+                x[t * R + q] = a[q];
+                mag |= fmag(a[q]);
             }
-            return;
         }
+        return mag;
     }
     for (int t = threadIdx.x; t < Ntot / R; t += blockDim.x) {
         const int j = t % Ns, base = (t - j) * R + j;
-        double2 a[R];
+        fx2 a[R];
 #pragma unroll
-        for (int q = 0; q < R; ++q) a[q] = x[base + q * Ns];
-        if constexpr (INV && R == 2) {
-            // y_0,1 = a_0 +- w a_1, w = w_B^j
-            double2 y0, y1;
-            bfly_fma(a[0], a[1], tw(j * step), y0, y1);
-            a[0] = y0;
-            a[1] = y1;
-        } else if constexpr (INV && R == 4) {
-            // twiddles w_B^{pj} then the 4-point DFT (exponent +1), as two
-            // layers of fused radix-2 butterflies: u0 = a0 +- w2 a2,
-            // u1 = a1 +- w2 a3 (w2 = w_B^{2j}), then y_0,2 = u0+ +- w1 u1+,
-            // y_1,3 = u0- +- i w1 u1- (w1 = w_B^j)
-            const double2 w1 = tw(j * step), w2 = tw(2 * j * step);
-            double2 u0p, u0m, u1p, u1m;
-            bfly_fma(a[0], a[2], w2, u0p, u0m);
-            bfly_fma(a[1], a[3], w2, u1p, u1m);
-            bfly_fma(u0p, u1p, w1, a[0], a[2]);
-            bfly_fma(u0m, u1m, make_double2(-w1.y, w1.x), a[1], a[3]);
-        } else if (INV) {
-            if (j) {
+        for (int q = 0; q < R; ++q) a[q] = fshl(x[base + q * Ns], s);
+        a[0] = frshift(a[0], 2);
+        if constexpr (INV) {
 #pragma unroll
-                for (int p = 1; p < R; ++p) a[p] = cmul(a[p], tw(p * j * step));
-            }
+            for (int p = 1; p < R; ++p) a[p] = fmul(a[p], tw(p * j * step));
             dft_small<R, 1>(a);
         } else {
-            dft_small<R, -1>(a);
-            if (j) {
 #pragma unroll
-                for (int p = 1; p < R; ++p) a[p] = cmul_conj(a[p], tw(p * j * step));
-            }
+            for (int p = 1; p < R; ++p) a[p] = frshift(a[p], 2);
+            dft_small<R, -1>(a);
+            a[0] = frshift(a[0], 2);
+#pragma unroll
+            for (int p = 1; p < R; ++p) a[p] = fmul<true>(a[p], tw(p * j * step));
         }
 #pragma unroll
-        for (int q = 0; q < R; ++q) x[base + q * Ns] = a[q];
+        for (int q = 0; q < R; ++q) {
+            x[base + q * Ns] = a[q];
+            mag |= fmag(a[q]);
+        }
     }
+    return mag;
 }
 
 // Rader pass context: the ring's prime tables, and shared-memory scratch
@@ -257,67 +355,73 @@ struct RaderCtx {
     const RaderInfo *ri;
     const int *rad;
     const int *ints;
-    const double2 *dbl;
-    double2 *scratch;
+    const int4 *tab;
+    fx2 *scratch;
 };
 
 template <bool CONJ>
-__device__ void rader_pass(double2 *x, int N, const RaderCtx &c);
+__device__ void rader_pass(fx2 *x, int N, const RaderCtx &c, FxScale &sc);
 
-// BIG: the radix-11 and radix-13 butterflies are compiled in (they need many
-// more registers; only lengths with those factors are run with BIG); RADER:
-// a radix above 13 is a prime done by Rader's algorithm (BIG kernels only)
+// One pass, its barrier before it included.  BIG: the radix-11 and radix-13
+// butterflies are compiled in (they need many more registers; only lengths
+// with those factors are run with BIG); RADER: a radix above 13 is a prime
+// done by Rader's algorithm (BIG kernels only)
 template <bool INV, bool BIG, bool RADER, class TW>
-__device__ __forceinline__ void mx_pass_any(int r, double2 *x, int Ntot, int Nseq, int B, const TW &tw,
+__device__ __forceinline__ void mx_pass_any(int r, fx2 *x, int Ntot, int Nseq, int B, const TW &tw, FxScale &sc,
                                             const RaderCtx *rc)
 {
+    if constexpr (RADER)
+        if (r > 13) {
+            rader_pass<!INV>(x, Ntot, *rc, sc);
+            return;
+        }
+    const int s = sc.enter(), Ns = B / r;
+    unsigned mag = 0;
     switch (r) {
-    case 4: mx_pass<4, INV>(x, Ntot, Nseq, B, tw); break;
-    case 2: mx_pass<2, INV>(x, Ntot, Nseq, B, tw); break;
-    case 3: mx_pass<3, INV>(x, Ntot, Nseq, B, tw); break;
-    case 5: mx_pass<5, INV>(x, Ntot, Nseq, B, tw); break;
-    case 7: mx_pass<7, INV>(x, Ntot, Nseq, B, tw); break;
+    case 4: mag = mx_pass<4, INV>(x, Ntot, Nseq, B, tw, s); sc.e += pass_bits<4, INV>(Ns); break;
+    case 2: mag = mx_pass<2, INV>(x, Ntot, Nseq, B, tw, s); sc.e += pass_bits<2, INV>(Ns); break;
+    case 3: mag = mx_pass<3, INV>(x, Ntot, Nseq, B, tw, s); sc.e += pass_bits<3, INV>(Ns); break;
+    case 5: mag = mx_pass<5, INV>(x, Ntot, Nseq, B, tw, s); sc.e += pass_bits<5, INV>(Ns); break;
+    case 7: mag = mx_pass<7, INV>(x, Ntot, Nseq, B, tw, s); sc.e += pass_bits<7, INV>(Ns); break;
     default:
         if constexpr (BIG) {
-            if (r == 11) mx_pass<11, INV>(x, Ntot, Nseq, B, tw);
-            else if (r == 13) mx_pass<13, INV>(x, Ntot, Nseq, B, tw);
-            else if constexpr (RADER) rader_pass<!INV>(x, Ntot, *rc);
+            if (r == 11) mag = mx_pass<11, INV>(x, Ntot, Nseq, B, tw, s);
+            else mag = mx_pass<13, INV>(x, Ntot, Nseq, B, tw, s);
+            sc.e += pass_bits<13, INV>(Ns);
         }
         break;
     }
+    sc.leave(mag);
 }
 
-// natural order in, position order out, exponent -1; Ntot / Nseq
-// sequences of Nseq points transformed side by side
+// natural order in, position order out, exponent -1; Ntot / Nseq sequences
+// of Nseq points transformed side by side.  The results' size is left for
+// the caller's FxScale::enter, which is also the barrier after the last pass.
 template <bool BIG, bool RADER, class TW>
-__device__ void fft_mx_dif(double2 *x, int Ntot, int Nseq, const int *__restrict__ rl, const TW &tw,
-                           const RaderCtx *rc = nullptr)
+__device__ __forceinline__ void fft_mx_dif(fx2 *x, int Ntot, int Nseq, const int *__restrict__ rl, const TW &tw,
+                                           FxScale &sc, const RaderCtx *rc = nullptr)
 {
     const int n = rl[0];
     int B = Nseq;
     for (int i = 0; i < n; ++i) {
         const int r = rl[1 + i];
-        __syncthreads();
-        mx_pass_any<false, BIG, RADER>(r, x, Ntot, Nseq, B, tw, rc);
+        mx_pass_any<false, BIG, RADER>(r, x, Ntot, Nseq, B, tw, sc, rc);
         B /= r;
     }
-    __syncthreads();
 }
 
 // position order in, natural order out, exponent +1 (unnormalised)
 template <bool BIG, bool RADER, class TW>
-__device__ void fft_mx_dit(double2 *x, int Ntot, int Nseq, const int *__restrict__ rl, const TW &tw,
-                           const RaderCtx *rc = nullptr)
+__device__ __forceinline__ void fft_mx_dit(fx2 *x, int Ntot, int Nseq, const int *__restrict__ rl, const TW &tw,
+                                           FxScale &sc, const RaderCtx *rc = nullptr)
 {
     const int n = rl[0];
     int B = 1;
     for (int i = n - 1; i >= 0; --i) {
         const int r = rl[1 + i];
         B *= r;
-        __syncthreads();
-        mx_pass_any<true, BIG, RADER>(r, x, Ntot, Nseq, B, tw, rc);
+        mx_pass_any<true, BIG, RADER>(r, x, Ntot, Nseq, B, tw, sc, rc);
     }
-    __syncthreads();
 }
 
 // ring transform kinds: direct mixed radix over 2, 3, 4, 5, 7; Bluestein
@@ -339,46 +443,59 @@ __device__ __forceinline__ int fft_pos(int k, int N, const int *__restrict__ rl)
     return pos;
 }
 
+// e^{i pi n / J}, n >= 0, from the ring's half-circle table (n < J)
+__device__ __forceinline__ int4 ring_root(const int4 *__restrict__ T, int J, int n)
+{
+    const int k = n % (2 * J);
+    return wneg_if(__ldg(T + (k < J ? k : k - J)), k >= J);
+}
+
 // e^{2 pi i t / K} (t < K) from the ring's half-circle table of J = 2K roots
 struct TwRing {
-    const double2 *T;
+    const int4 *T;
     int J;
-    __device__ __forceinline__ double2 operator()(int t) const
+    __device__ __forceinline__ int4 operator()(int t) const
     {
         const int n = 4 * t;             // e^{2 pi i t / K} = e^{i pi 4t / J}, 4t < 2J
-        if (n < J) return __ldg(T + n);
-        const double2 u = __ldg(T + (n - J));
-        return make_double2(-u.x, -u.y);
+        return wneg_if(__ldg(T + (n < J ? n : n - J)), n >= J);
     }
 };
 
 // e^{2 pi i t / M} (t < M) from a table of M roots
 struct TwTable {
-    const double2 *R;
-    __device__ __forceinline__ double2 operator()(int t) const { return __ldg(R + t); }
+    const int4 *R;
+    __device__ __forceinline__ int4 operator()(int t) const { return __ldg(R + t); }
 };
 
-// x[0..K) holds the input; computes x[n] = sum_k x_k e^{2 pi i k n / K} in
-// place for n < K through Bluestein's chirp transform: a cyclic convolution
-// of length M (smooth, >= 2K - 1) with the chirp filter, stored transformed
-// in position order and scaled by 1/M.  x must hold M entries.  T is the
-// ring's e^{i pi n/J} table (J = 2K): the chirp c_j = e^{i pi j^2 / K} is
-// the root of index 2 j^2 mod 2J.  PRECHIRP = false: the input already
-// carries its chirp c_k (the synthesis fold weights include it).
-template <bool PRECHIRP>
-__device__ void bluestein_mx(double2 *x, int K, int M, const double2 *__restrict__ T,
-                             const double2 *__restrict__ fb, const int *__restrict__ rl, const TwTable &tw)
+// x[0..K) holds the input, zeros follow up to M; computes x[n] =
+// sum_k x_k e^{2 pi i k n / K} for n < K through Bluestein's chirp transform:
+// a cyclic convolution of length M (smooth, >= 2K - 1) with the chirp filter,
+// stored transformed in position order and scaled by 1/M.  The input already
+// carries its chirp c_k = e^{i pi k^2 / K} and the results do not: the caller
+// multiplies them by c_n as it reads them.
+__device__ __forceinline__ void bluestein_mx(fx2 *x, int M, const int4 *__restrict__ fb, const int *__restrict__ rl,
+                                             const TwTable &tw, FxScale &sc)
 {
-    const int J = 2 * K;
+    fft_mx_dif<false, false>(x, M, M, rl, tw, sc);
+    const int s = sc.enter();
+    unsigned mag = 0;
     for (int k = threadIdx.x; k < M; k += blockDim.x) {
-        if (k >= K) x[k] = make_double2(0.0, 0.0);
-        else if (PRECHIRP) x[k] = cmul(x[k], ring_root32(T, J, 2 * k * k));
+        const fx2 y = fmul(fshl(x[k], s), __ldg(fb + k));
+        x[k] = y;
+        mag |= fmag(y);
     }
-    fft_mx_dif<false, false>(x, M, M, rl, tw);
-    for (int k = threadIdx.x; k < M; k += blockDim.x) x[k] = cmul(x[k], __ldg(fb + k));
-    fft_mx_dit<false, false>(x, M, M, rl, tw);
-    for (int n = threadIdx.x; n < K; n += blockDim.x) x[n] = cmul(x[n], ring_root32(T, J, 2 * n * n));
-    __syncthreads();
+    sc.e += 2;
+    sc.leave(mag);
+    fft_mx_dit<false, false>(x, M, M, rl, tw, sc);
+}
+
+// x true = x 2^from in units of 2^to, to nearest
+__device__ __forceinline__ fx2 frescale(fx2 a, int from, int to)
+{
+    const int n = to - from;
+    if (n == 0) return a;
+    if (n < 0) return fshl(a, -n);
+    return n > 62 ? make_longlong2(0, 0) : frshift(a, n);
 }
 
 // Rader's algorithm for the p-point DFTs of one pass over N points (blocks
@@ -391,99 +508,213 @@ __device__ void bluestein_mx(double2 *x, int K, int M, const double2 *__restrict
 // side for the N / p blocks in the scratch.  a_0 joins every output through
 // the product's zero frequency, and y_0 = a_0 + (sum of alpha) is that
 // frequency before the product.  Exponent +1; CONJ = true gives exponent -1
-// as conj(DFT(conj a)).  Barriers: the transform's passes sync before they
-// start and after they end; the caller syncs before the next pass.
+// as conj(DFT(conj a)).  The a_0 stay in the units they have when the pass
+// begins; at the end all points are in the convolution's units.
 template <bool CONJ>
-__device__ void rader_pass(double2 *x, int N, const RaderCtx &c)
+__device__ void rader_pass(fx2 *x, int N, const RaderCtx &c, FxScale &sc)
 {
     const RaderInfo ri = *c.ri;
     const int p = ri.p, n = ri.n, tot = (N / p) * n;
     const int *__restrict__ ga = c.ints + ri.ga;
     const int *__restrict__ gi = c.ints + ri.gi;
-    const double2 *__restrict__ G = c.dbl + ri.G;
+    const int4 *__restrict__ G = c.tab + ri.G;
     const int *__restrict__ rl = c.rad + ri.rl;
-    const TwTable tw{c.dbl + ri.tw};
-    double2 *S = c.scratch;
+    const TwTable tw{c.tab + ri.tw};
+    fx2 *S = c.scratch;
+    const int s0 = sc.enter();
+    const int e0 = sc.e + s0;                          // units of the a_0 left in x
+    unsigned mag = 0;
     for (int e = threadIdx.x; e < tot; e += blockDim.x) {
         const int b = e / n, v = e - b * n;
-        const double2 a = x[b * p + __ldg(gi + v)];
-        S[e] = CONJ ? cconj_i(a) : a;
+        fx2 a = fshl(x[b * p + __ldg(gi + v)], s0);
+        if (CONJ) a = fconj(a);
+        S[e] = a;
+        mag |= fmag(a);
     }
-    fft_mx_dif<true, false>(S, tot, n, rl, tw);
+    sc.leave(mag);
+    fft_mx_dif<true, false>(S, tot, n, rl, tw, sc);
+    // y_0 (and a_0 with the product) may need as many more bits as a_0 has
+    // above the rest: both sides at a quarter of their size, in the larger units
+    const int s1 = sc.enter(), e1 = max(sc.e, e0) + 2;
+    mag = 0;
     for (int e = threadIdx.x; e < tot; e += blockDim.x) {
         const int b = e / n, v = e - b * n;
-        const double2 A = S[e];
-        double2 C = cmul(A, __ldg(G + v));
+        const fx2 A = frescale(fshl(S[e], s1), sc.e, e1);
+        fx2 C = fmul(A, __ldg(G + v));                 // e1 + 2
         if (v == 0) {
-            const double2 a0 = CONJ ? cconj_i(x[b * p]) : x[b * p];
-            const double2 y0 = cadd(a0, A);
-            x[b * p] = CONJ ? cconj_i(y0) : y0;
-            C = cadd(C, a0);
+            fx2 a0 = frescale(CONJ ? fconj(x[b * p]) : x[b * p], e0, e1);
+            fx2 y0 = fadd(a0, A);
+            if (CONJ) y0 = fconj(y0);
+            x[b * p] = y0;                             // in units of 2^e1
+            mag |= fmag(frshift(y0, 2));
+            C = fadd(C, frshift(a0, 2));
         }
         S[e] = C;
+        mag |= fmag(C);
     }
-    fft_mx_dit<true, false>(S, tot, n, rl, tw);
+    sc.e = e1 + 2;
+    sc.leave(mag);
+    fft_mx_dit<true, false>(S, tot, n, rl, tw, sc);
+    const int s2 = sc.enter(), e2 = max(sc.e, e1) + 1;
+    mag = 0;
     for (int e = threadIdx.x; e < tot; e += blockDim.x) {
         const int b = e / n, w = e - b * n;
-        const double2 y = S[e];
-        x[b * p + __ldg(ga + w)] = CONJ ? cconj_i(y) : y;
+        fx2 y = frescale(fshl(S[e], s2), sc.e, e2);
+        if (CONJ) y = fconj(y);
+        x[b * p + __ldg(ga + w)] = y;
+        mag |= fmag(y);
+        if (w == 0) {
+            const fx2 y0 = frescale(x[b * p], e1, e2);
+            x[b * p] = y0;
+            mag |= fmag(y0);
+        }
     }
+    sc.e = e2;
+    sc.leave(mag);
 }
 
 // The Rader context of a ring of a BIG kernel (nullptr for other rings):
 // its scratch follows the ring's K points in shared memory.
-__device__ __forceinline__ const RaderCtx *rader_ctx(const PlanView &v, int ring, int K, double2 *sm, RaderCtx &rc)
+__device__ __forceinline__ const RaderCtx *rader_ctx(const PlanView &v, int ring, int K, fx2 *sm, RaderCtx &rc)
 {
     const int ri = v.ring_rdr[ring];
     if (ri < 0) return nullptr;
-    rc = RaderCtx{v.rdr + ri, v.rad, v.rdr_int, v.rdr_dbl, sm + K};
+    rc = RaderCtx{v.rdr + ri, v.rad, v.rdr_int, ring_table(v.rdr_dbl), sm + K};
     return &rc;
+}
+
+// v = a whole number of 2^(ex - 1083) below 2^61, toward zero; sh = 3 + ex - v's exponent
+__device__ __forceinline__ long long ring_fix(double v, int sh)
+{
+    const int hi = __double2hiint(v), lo = __double2loint(v);
+    const unsigned mh = __funnelshift_l((unsigned)lo, (unsigned)hi, 11) | 0x80000000u;
+    unsigned long long X;
+    asm("shr.u64 %0, %1, %2;" : "=l"(X) : "l"((unsigned long long)mh << 32 | ((unsigned)lo << 11)), "r"(sh));
+    const unsigned long long s = (unsigned long long)(long long)(hi >> 31);
+    return (long long)((X ^ s) - s);
+}
+
+__device__ __forceinline__ int exp_field(double v) { return __double2hiint(v) & 0x7ff00000; }
+__device__ __forceinline__ unsigned nonzero_bits(double v)
+{
+    return (unsigned)__double2hiint(v) << 1 | (unsigned)__double2loint(v);
+}
+
+// Shared words of a ring's block: the three size slots of FxScale, the
+// largest exponent, whether any value is not zero
+struct RingAux {
+    unsigned slot[3];
+    int emax;
+    unsigned any;
+};
+
+// Range of the block exponent that the fixed-point path takes
+constexpr int kRingExpLo = 300, kRingExpHi = 1700;
+
+// the ring's direct sum in FP64, for values the fixed-point path does not take
+template <class QAt>
+__device__ __noinline__ void ring_direct_synth(const int4 *T, int J, int s, int L, QAt qat, double *out)
+{
+    for (int j = threadIdx.x; j < J; j += blockDim.x) {
+        double f = qat(0).x;
+        for (int m = 1; m <= L; ++m) {
+            const int k = (int)(((long long)m * (2 * j + s)) % (2 * J));
+            const double2 w = ring_unfix(T[k < J ? k : k - J], k >= J), q = qat(m);
+            f += 2.0 * (q.x * w.x - q.y * w.y);
+        }
+        out[j] = f;
+    }
 }
 
 // Pixels of one ring from its q_m (m = 0..L): fold (Eq. tau) and pack the
 // Hermitian spectrum into a half-length complex FFT in one step,
-// Z_k = G_k A_k + G_{k+K} B_k (8 FP64 instructions per k; the plan's fold
-// weights A, B hold the phi_0 phase, the packing twiddle and, on Bluestein
-// rings, the chirp), transform, and write f_{2n}, f_{2n+1} as the real and
-// imaginary parts of z_n.  All threads of the block take part; sm holds K
-// (direct), K plus the Rader scratch, or M (Bluestein) entries.
+// Z_k = G_k A_k + G_{k+K} B_k (the plan's fold weights A, B hold the phi_0
+// phase, the packing twiddle and, on Bluestein rings, the chirp), transform,
+// and write f_{2n}, f_{2n+1} as the real and imaginary parts of z_n.  The
+// fold's sums are FP64; each Z_k is formed in fixed point with its own
+// exponent, and once the largest is known all are brought to it.  All threads
+// of the block take part; sm holds the transform's entries (K direct, K plus
+// the Rader scratch, M Bluestein) and K 16-bit exponents after them.
 template <int KIND, class QAt>
-__device__ void phi_synth_ring_at(const PlanView &v, int ring, QAt qat, double *out_ring, double2 *sm)
+__device__ __forceinline__ void phi_synth_ring_at(const PlanView &v, int ring, QAt qat, double *out_ring, fx2 *sm)
 {
     constexpr bool BLUE = KIND == kBluestein, BIG = KIND == kDirectBig;
+    __shared__ RingAux aux;
     const int L = v.lmax;
     const int J = v.ring_J[ring], K = J / 2, s = v.ring_s[ring];
-    const double2 *__restrict__ T = v.tw + v.ring_tw[ring];
-    const double2 *__restrict__ AB = v.ab + v.ring_ab[ring];
+    const int4 *__restrict__ T = ring_table(v.tw) + v.ring_tw[ring];
+    const int4 *__restrict__ AB = ring_table(v.ab) + v.ring_ab[ring];
     const int *__restrict__ rl = v.rad + v.ring_rad[ring];
+    RaderCtx rc;
+    const RaderCtx *rcp = BIG ? rader_ctx(v, ring, K, sm, rc) : nullptr;
+    const int M = BLUE ? v.ring_mx[ring] : 0;
+    const int entries = BLUE ? M : BIG && rcp ? K + (K / rcp->ri->p) * rcp->ri->n : K;
+    short *ex = reinterpret_cast<short *>(sm + entries);
+    if (threadIdx.x == 0) aux = RingAux{{0, 0, 0}, 0, 0};
+    __syncthreads();
+    int emax = 0;
+    unsigned any = 0;
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
         const double2 G0 = fold_G(qat, L, J, s, k);
         const double2 G1 = fold_G(qat, L, J, s, k + K);
-        const double2 A = __ldg(AB + 2 * k), B = __ldg(AB + 2 * k + 1);
-        double2 Z;
-        Z.x = fma(G0.x, A.x, fma(-G0.y, A.y, fma(G1.x, B.x, -(G1.y * B.y))));
-        Z.y = fma(G0.x, A.y, fma(G0.y, A.x, fma(G1.x, B.y, G1.y * B.x)));
-        if (BLUE) sm[k] = Z;
-        else sm[fft_pos(k, K, rl)] = Z;
+        const int f = max(max(exp_field(G0.x), exp_field(G0.y)), max(exp_field(G1.x), exp_field(G1.y)));
+        any |= nonzero_bits(G0.x) | nonzero_bits(G0.y) | nonzero_bits(G1.x) | nonzero_bits(G1.y);
+        const int f3 = f + (3 << 20);
+        const fx2 X0 = make_longlong2(ring_fix(G0.x, (f3 - exp_field(G0.x)) >> 20),
+                                      ring_fix(G0.y, (f3 - exp_field(G0.y)) >> 20));
+        const fx2 X1 = make_longlong2(ring_fix(G1.x, (f3 - exp_field(G1.x)) >> 20),
+                                      ring_fix(G1.y, (f3 - exp_field(G1.y)) >> 20));
+        const int pos = BLUE ? k : fft_pos(k, K, rl);
+        sm[pos] = fadd(fmul(X0, __ldg(AB + 2 * k)), fmul(X1, __ldg(AB + 2 * k + 1)));    // units 2^(f - 1080)
+        ex[pos] = (short)(f >> 20);
+        emax = max(emax, f >> 20);
     }
-    if constexpr (BLUE) {
-        __syncthreads();
-        bluestein_mx<false>(sm, K, v.ring_mx[ring], T, v.mfb + v.ring_mfb[ring], rl,
-                            TwTable{v.mtw + v.ring_mtw[ring]});
-    } else {
-        RaderCtx rc;
-        const RaderCtx *rcp = BIG ? rader_ctx(v, ring, K, sm, rc) : nullptr;
-        fft_mx_dit<BIG, BIG>(sm, K, K, rl, TwRing{T, J}, rcp);
+    emax = (int)__reduce_max_sync(0xffffffffu, (unsigned)emax);
+    any = __reduce_or_sync(0xffffffffu, any);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&aux.emax, emax);
+        atomicOr(&aux.any, any);
     }
+    __syncthreads();
+    emax = aux.emax;
     double2 *out = reinterpret_cast<double2 *>(out_ring);
-    for (int n = threadIdx.x; n < K; n += blockDim.x) out[n] = sm[n];
+    if (emax < kRingExpLo || emax > kRingExpHi) {
+        if (!aux.any) {
+            for (int n = threadIdx.x; n < K; n += blockDim.x) out[n] = make_double2(0.0, 0.0);
+        } else {
+            ring_direct_synth(T, J, s, L, qat, out_ring);
+        }
+        __syncthreads();
+        return;
+    }
+    FxScale sc{aux.slot, 0, emax - 1080};
+    unsigned mag = 0;
+    for (int p = threadIdx.x; p < (BLUE ? M : K); p += blockDim.x) {
+        if (BLUE && p >= K) {
+            sm[p] = make_longlong2(0, 0);
+            continue;
+        }
+        const int n = min(63, emax - ex[p]);
+        const fx2 z = make_longlong2(sm[p].x >> n, sm[p].y >> n);
+        sm[p] = z;
+        mag |= fmag(z);
+    }
+    sc.leave(mag);
+    if constexpr (BLUE) bluestein_mx(sm, M, ring_table(v.mfb) + v.ring_mfb[ring], rl, TwTable{ring_table(v.mtw) + v.ring_mtw[ring]}, sc);
+    else fft_mx_dit<BIG, BIG>(sm, K, K, rl, TwRing{T, J}, sc, rcp);
+    const int sh = sc.enter();
+    const int be = sc.e + (BLUE ? 2 : 0) + 1054;
+    for (int n = threadIdx.x; n < K; n += blockDim.x) {
+        fx2 z = fshl(sm[n], sh);
+        if (BLUE) z = fmul(z, ring_root(T, J, 2 * n * n));
+        out[n] = make_double2(fix_to_double(z.x, be), fix_to_double(z.y, be));
+    }
     __syncthreads();
 }
 
 // ... with q_m read from a ring-major array qr[m]
 template <int KIND, bool CG>
-__device__ void phi_synth_ring(const PlanView &v, int ring, const double2 *qr, double *out_ring,
-                               double2 *sm)
+__device__ __forceinline__ void phi_synth_ring(const PlanView &v, int ring, const double2 *qr, double *out_ring, fx2 *sm)
 {
     phi_synth_ring_at<KIND>(v, ring, [qr](int m) { return ldq<CG>(qr + m); }, out_ring, sm);
 }
@@ -492,8 +723,8 @@ __device__ void phi_synth_ring(const PlanView &v, int ring, const double2 *qr, d
 // stored map-major: qt[((b * 2 + t) * nhalf + r) * (L + 1) + m] (complex);
 // north rings (ring < nhalf) take q^0 + q^1, their mirrors q^0 - q^1.
 template <int KIND, bool CG>
-__device__ void phi_synth_ring_qt(const PlanView &v, int ring, const double2 *qt, int b,
-                                  double *out_ring, double2 *sm)
+__device__ __forceinline__ void phi_synth_ring_qt(const PlanView &v, int ring, const double2 *qt, int b,
+                                                  double *out_ring, fx2 *sm)
 {
     const int Z = v.nhalf, L = v.lmax;
     const bool north = ring < Z;
@@ -506,6 +737,114 @@ __device__ void phi_synth_ring_qt(const PlanView &v, int ring, const double2 *qt
         return cadd(x0, cneg_if(ldq<CG>(q1 + m), !north));
     };
     phi_synth_ring_at<KIND>(v, ring, qat, out_ring, sm);
+}
+
+static __device__ __noinline__ void ring_direct_adjoint(const int4 *T, int J, int s, int L, const double *f, double2 *outq);
+
+// Adjoint of one ring: q_adj[m] = sum_j f_j e^{-i m phi_j}, m = 0..L, from
+// z_n = f_{2n} + i f_{2n+1}, Zf = DFT(z) with exponent -1 (position order, or
+// natural order on Bluestein rings), F_r = E'_r + e^{-2 pi i r/J} O'_r with
+// E' = (Zf_r + conj Zf_{K-r})/2, O' = (Zf_r - conj Zf_{K-r})/(2i), K-periodic,
+// and q_adj[m] = e^{-i pi m s / J} F_{m mod J}.
+template <int KIND>
+__device__ __forceinline__ void phi_adjoint_ring(const PlanView &v, int ring, const double *f_ring, double2 *outq, fx2 *sm)
+{
+    constexpr bool BLUE = KIND == kBluestein, BIG = KIND == kDirectBig;
+    __shared__ RingAux aux;
+    const int L = v.lmax;
+    const int J = v.ring_J[ring], K = J / 2, s = v.ring_s[ring];
+    const int4 *__restrict__ T = ring_table(v.tw) + v.ring_tw[ring];
+    const int *__restrict__ rl = v.rad + v.ring_rad[ring];
+    RaderCtx rc;
+    const RaderCtx *rcp = BIG ? rader_ctx(v, ring, K, sm, rc) : nullptr;
+    const int M = BLUE ? v.ring_mx[ring] : 0;
+    if (threadIdx.x == 0) aux = RingAux{{0, 0, 0}, 0, 0};
+    __syncthreads();
+    const double2 *in = reinterpret_cast<const double2 *>(f_ring);
+    int emax = 0;
+    unsigned any = 0;
+    for (int n = threadIdx.x; n < K; n += blockDim.x) {
+        const double2 z = __ldg(in + n);
+        emax = max(emax, max(exp_field(z.x), exp_field(z.y)));
+        any |= nonzero_bits(z.x) | nonzero_bits(z.y);
+    }
+    emax = (int)__reduce_max_sync(0xffffffffu, (unsigned)emax);
+    any = __reduce_or_sync(0xffffffffu, any);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&aux.emax, emax);
+        atomicOr(&aux.any, any);
+    }
+    __syncthreads();
+    emax = aux.emax;
+    if (emax < kRingExpLo << 20 || emax > kRingExpHi << 20) {
+        if (!aux.any) {
+            for (int m = threadIdx.x; m <= L; m += blockDim.x) outq[m] = make_double2(0.0, 0.0);
+        } else {
+            ring_direct_adjoint(T, J, s, L, f_ring, outq);
+        }
+        __syncthreads();
+        return;
+    }
+    FxScale sc{aux.slot, 0, (emax >> 20) - 1083};
+    const int e3 = emax + (3 << 20);
+    unsigned mag = 0;
+    for (int n = threadIdx.x; n < (BLUE ? M : K); n += blockDim.x) {
+        if (BLUE && n >= K) {
+            sm[n] = make_longlong2(0, 0);
+            continue;
+        }
+        const double2 zd = __ldg(in + n);
+        fx2 z = make_longlong2(ring_fix(zd.x, (e3 - exp_field(zd.x)) >> 20), ring_fix(zd.y, (e3 - exp_field(zd.y)) >> 20));
+        if (BLUE) z = fmul(fconj(z), ring_root(T, J, 2 * n * n));    // forward = conj(inverse(conj))
+        sm[n] = z;
+        mag |= fmag(z);
+    }
+    if (BLUE) sc.e += 2;
+    sc.leave(mag);
+    if constexpr (BLUE) {
+        bluestein_mx(sm, M, ring_table(v.mfb) + v.ring_mfb[ring], rl, TwTable{ring_table(v.mtw) + v.ring_mtw[ring]}, sc);
+        const int sh = sc.enter();
+        mag = 0;
+        for (int n = threadIdx.x; n < K; n += blockDim.x) {
+            const fx2 z = fconj(fmul(fshl(sm[n], sh), ring_root(T, J, 2 * n * n)));
+            sm[n] = z;
+            mag |= fmag(z);
+        }
+        sc.e += 2;
+        sc.leave(mag);
+    } else {
+        fft_mx_dif<BIG, BIG>(sm, K, K, rl, TwRing{T, J}, sc, rcp);
+    }
+    const int sh = sc.enter();
+    const int be = sc.e + 1 + (s ? 4 : 2) + 1054;
+    for (int m = threadIdx.x; m <= L; m += blockDim.x) {
+        const int r = m % J;
+        const int rho = r < K ? r : r - K;
+        const int rho2 = rho == 0 ? 0 : K - rho;
+        // halves of A and conj B, so that their sum and difference have room
+        const fx2 A = frshift(fshl(BLUE ? sm[rho] : sm[fft_pos(rho, K, rl)], sh), 2);
+        const fx2 B = fconj(frshift(fshl(BLUE ? sm[rho2] : sm[fft_pos(rho2, K, rl)], sh), 2));
+        const fx2 D = fsub(A, B);
+        const fx2 Op = make_longlong2(D.y, -D.x);                              // D / i
+        fx2 F = fadd(frshift(fadd(A, B), 2), fmul<true>(Op, ring_root(T, J, 2 * r)));
+        if (s) F = fmul<true>(F, ring_root(T, J, m));
+        outq[m] = make_double2(fix_to_double(F.x, be), fix_to_double(F.y, be));
+    }
+    __syncthreads();
+}
+
+static __device__ __noinline__ void ring_direct_adjoint(const int4 *T, int J, int s, int L, const double *f, double2 *outq)
+{
+    for (int m = threadIdx.x; m <= L; m += blockDim.x) {
+        double2 q = make_double2(0.0, 0.0);
+        for (int j = 0; j < J; ++j) {
+            const int k = (int)(((long long)m * (2 * j + s)) % (2 * J));
+            const double2 w = ring_unfix(T[k < J ? k : k - J], k >= J);
+            q.x += f[j] * w.x;
+            q.y -= f[j] * w.y;
+        }
+        outq[m] = q;
+    }
 }
 
 }  // namespace shtb_dev

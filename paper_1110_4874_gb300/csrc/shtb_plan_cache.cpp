@@ -20,6 +20,7 @@
 #include "shtb_butterfly.h"
 #include "shtb_fix.h"
 #include "shtb_internal.h"
+#include "shtb_ring_fix.h"
 
 namespace {
 
@@ -156,7 +157,16 @@ bool write_payload(Writer &w, shtb_plan_s *p)
         w.val(n);
         buf.resize(n);
         if (cudaMemcpy(buf.data(), p->allocations[i], n, cudaMemcpyDeviceToHost) != cudaSuccess) return false;
-        if (p->bf && p->allocations[i] == (const void *)p->bf->dbl) {     // files hold the blocks as doubles
+        for (const RingTable &t : ring_tables(p)) {                       // files hold the tables as doubles
+            if (p->allocations[i] != (const void *)t.table) continue;
+            for (uint64_t k = 0; k + 8 <= n; k += 8) {
+                int half[2];
+                memcpy(half, buf.data() + k, 8);
+                const double v = shtb::ring_half_unpack(half[0], half[1], t.bits);
+                memcpy(buf.data() + k, &v, 8);
+            }
+        }
+        if (p->bf && p->allocations[i] == (const void *)p->bf->dbl) {     // ... and the blocks
             for (uint64_t k = 0; k + 8 <= n; k += 8) {
                 uint64_t word;
                 memcpy(&word, buf.data() + k, 8);
@@ -307,9 +317,12 @@ int plan_load(shtb_plan_s *p, const char *path)
     fclose(f);
     if (!complete || r.sum.h != h.checksum)
         return shtb_fail(SHTB_ECORRUPT, std::string("plan file failed its size or checksum check: ") + path);
-    // the item lists are trusted from here on
-    if (p->bf && (rc = bf_pack_operator(p))) return rc;
-    if (p->partner && p->partner->bf && (rc = bf_pack_operator(p->partner))) return rc;
+    // the lists and sizes are trusted from here on
+    for (shtb_plan_s *q : {p, p->partner}) {
+        if (!q) continue;
+        if ((rc = ring_pack_tables(q))) return rc;
+        if (q->bf && (rc = bf_pack_operator(q))) return rc;
+    }
     return SHTB_OK;
 }
 

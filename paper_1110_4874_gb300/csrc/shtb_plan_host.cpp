@@ -900,6 +900,7 @@ int shtb_build_dense_plan(shtb_plan_s *p)
     rc = plan_alloc_upload(p, &d, chunk_list.data(), sizeof(int) * chunk_list.size());
     if (rc) return rc;
     p->d_chunk_list = (int *)d;
+    if ((rc = ring_pack_tables(p))) return rc;
 
     // bytes one call reads from the plan (Legendre tables + start values)
     p->stats.plan_read_bytes = (long long)(sizeof(RecCoef) * coef.size() + sizeof(int) * jstart.size() +
