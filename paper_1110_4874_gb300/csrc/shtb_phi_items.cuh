@@ -74,6 +74,18 @@ __device__ __forceinline__ double2 fold_G(QAt qat, int L, int J, int s, int r)
     return acc;
 }
 
+// The terms of fold_G number part, part + parts, .. of both signs
+template <class QAt>
+__device__ __forceinline__ double2 fold_part(QAt qat, int L, int J, int s, int r, int part, int parts)
+{
+    double2 acc = make_double2(0.0, 0.0);
+    int t = part;
+    for (int m = r + part * J; m <= L; m += parts * J, t += parts) acc = cadd(acc, cneg_if(qat(m), s & t));
+    t = part + 1;
+    for (int mp = t * J - r; mp <= L; mp += parts * J, t += parts) acc = cadd(acc, cneg_if(cconj_i(qat(mp)), s & t));
+    return acc;
+}
+
 // ------------------------------------------------ fixed-point complex numbers
 typedef longlong2 fx2;
 
@@ -654,9 +666,7 @@ __device__ __forceinline__ void phi_synth_ring_at(const PlanView &v, int ring, Q
     __syncthreads();
     int emax = 0;
     unsigned any = 0;
-    for (int k = threadIdx.x; k < K; k += blockDim.x) {
-        const double2 G0 = fold_G(qat, L, J, s, k);
-        const double2 G1 = fold_G(qat, L, J, s, k + K);
+    auto pack = [&](int k, double2 G0, double2 G1) {
         const int f = max(max(exp_field(G0.x), exp_field(G0.y)), max(exp_field(G1.x), exp_field(G1.y)));
         any |= nonzero_bits(G0.x) | nonzero_bits(G0.y) | nonzero_bits(G1.x) | nonzero_bits(G1.y);
         const int f3 = f + (3 << 20);
@@ -668,6 +678,27 @@ __device__ __forceinline__ void phi_synth_ring_at(const PlanView &v, int ring, Q
         sm[pos] = fadd(fmul(X0, __ldg(AB + 2 * k)), fmul(X1, __ldg(AB + 2 * k + 1)));    // units 2^(f - 1080)
         ex[pos] = (short)(f >> 20);
         emax = max(emax, f >> 20);
+    };
+    // A short ring folds many terms onto few k (J = 4: L / 2 each): up to 32
+    // neighbouring threads then share one k's terms
+    int parts = 1;
+    while (parts < 32 && 2 * parts * K <= (int)blockDim.x) parts *= 2;
+    if (parts == 1) {
+        for (int k = threadIdx.x; k < K; k += blockDim.x) pack(k, fold_G(qat, L, J, s, k), fold_G(qat, L, J, s, k + K));
+    } else {
+        const int k = threadIdx.x / parts, part = threadIdx.x & (parts - 1);
+        double2 G0 = make_double2(0.0, 0.0), G1 = G0;
+        if (k < K) {
+            G0 = fold_part(qat, L, J, s, k, part, parts);
+            G1 = fold_part(qat, L, J, s, k + K, part, parts);
+        }
+        for (int o = 1; o < parts; o *= 2) {
+            G0.x += __shfl_xor_sync(0xffffffffu, G0.x, o);
+            G0.y += __shfl_xor_sync(0xffffffffu, G0.y, o);
+            G1.x += __shfl_xor_sync(0xffffffffu, G1.x, o);
+            G1.y += __shfl_xor_sync(0xffffffffu, G1.y, o);
+        }
+        if (k < K && part == 0) pack(k, G0, G1);
     }
     emax = (int)__reduce_max_sync(0xffffffffu, (unsigned)emax);
     any = __reduce_or_sync(0xffffffffu, any);
