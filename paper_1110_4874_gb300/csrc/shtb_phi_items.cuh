@@ -188,7 +188,7 @@ struct FxScale {
 
 // cos and sin of 2 pi k / R for the odd radices, k < R: R = 3, 5, 7, 11, 13
 // at offsets 0, 3, 8, 15, 26, in units of 2^-59 as {low, high} halves
-__device__ __forceinline__ constexpr double root_cos(int k)
+__host__ __device__ constexpr double root_cos(int k)
 {
     constexpr double t[39] = {
     1.00000000000000000e+00, -5.00000000000000000e-01, -5.00000000000000000e-01,
@@ -205,7 +205,7 @@ __device__ __forceinline__ constexpr double root_cos(int k)
     8.85456025653209911e-01};
     return t[k];
 }
-__device__ __forceinline__ constexpr double root_sin(int k)
+__host__ __device__ constexpr double root_sin(int k)
 {
     constexpr double t[39] = {
     0.00000000000000000e+00, 8.66025403784438597e-01, -8.66025403784438597e-01,
@@ -222,9 +222,9 @@ __device__ __forceinline__ constexpr double root_sin(int k)
     -4.64723172043768562e-01};
     return t[k];
 }
-__device__ __forceinline__ constexpr long long root_fix(double x) { return (long long)(x * 0x1p59); }
-__device__ __forceinline__ constexpr int root_low(long long v) { return (int)(unsigned)(v & 0xffffffffLL); }
-__device__ __forceinline__ constexpr int root_high(long long v) { return (int)((v - root_low(v)) / (1LL << 32)); }
+__host__ __device__ constexpr long long root_fix(double x) { return (long long)(x * 0x1p59); }
+__host__ __device__ constexpr int root_low(long long v) { return (int)(unsigned)(v & 0xffffffffLL); }
+__host__ __device__ constexpr int root_high(long long v) { return (int)((v - root_low(v)) / (1LL << 32)); }
 
 template <int R>
 __device__ __forceinline__ constexpr int root_off()
@@ -361,6 +361,101 @@ __device__ __forceinline__ unsigned mx_pass(fx2 *x, int Ntot, int Nseq, int B, c
     return mag;
 }
 
+// cos and sin of 2 pi k / R in units of 2^-59 as halves {low, high, low,
+// high}, k < R, for R = 11 and 13 at root_off<R>() - 15
+struct RootTable {
+    int4 v[24];
+};
+constexpr RootTable make_root_table()
+{
+    RootTable t{};
+    for (int i = 0; i < 24; ++i) {
+        const long long c = root_fix(root_cos(15 + i)), n = root_fix(root_sin(15 + i));
+        t.v[i].x = root_low(c);
+        t.v[i].y = root_high(c);
+        t.v[i].z = root_low(n);
+        t.v[i].w = root_high(n);
+    }
+    return t;
+}
+static __constant__ RootTable kRoots = make_root_table();
+
+// mx_pass for the radices 11 and 13, with dft_small written out around the
+// loads and stores: the inputs are taken pair by pair and each pair of
+// outputs is stored as soon as it is made, in a rolled loop over the outputs.
+// Unrolled, with inputs and outputs in registers, the radix-13 pass spilled
+// at 128 registers and the kernel's code overflowed the instruction cache
+// (ring stage of 8 maps at Nside = 512 1.058 -> 1.021 ms, adjoint 1.158 ->
+// 1.125; radix 7 the same way measured 1.034 and 1.117).
+template <int R, bool INV, class TW>
+__device__ __forceinline__ unsigned mx_pass_odd(fx2 *x, int Ntot, int Nseq, int B, const TW &tw, int s)
+{
+    constexpr int H = (R - 1) / 2, O = root_off<R>() - 15;
+    const int Ns = B / R, step = Nseq / B;
+    const bool twiddled = Ns > 1;
+    unsigned mag = 0;
+    for (int t = threadIdx.x; t < Ntot / R; t += blockDim.x) {
+        const int j = t % Ns, base = (t - j) * R + j;
+        int sh[H][2], sl[H][2], dh[H][2], dl[H][2];
+        const fx2 a0 = frshift(fshl(x[base], s), 2);
+        fx2 y0 = make_longlong2(a0.x >> 1, a0.y >> 1);
+#pragma unroll
+        for (int p = 1; p <= H; ++p) {
+            fx2 a = fshl(x[base + p * Ns], s), b = fshl(x[base + (R - p) * Ns], s);
+            if (INV && twiddled) {
+                a = fmul(a, tw(p * j * step));
+                b = fmul(b, tw((R - p) * j * step));
+            } else {
+                a = frshift(a, 2);
+                b = frshift(b, 2);
+            }
+            const fx2 sp = fadd(a, b), dp = fsub(a, b);
+            halves(sp.x, sh[p - 1][0], sl[p - 1][0]);
+            halves(sp.y, sh[p - 1][1], sl[p - 1][1]);
+            halves(dp.x, dh[p - 1][0], dl[p - 1][0]);
+            halves(dp.y, dh[p - 1][1], dl[p - 1][1]);
+            y0.x += sp.x >> 1;
+            y0.y += sp.y >> 1;
+        }
+        y0 = frshift(y0, !INV && twiddled ? 6 : 4);
+        x[base] = y0;
+        mag |= fmag(y0);
+        const fx2 a05 = frshift(a0, 5);
+#pragma unroll 1
+        for (int q = 1; q <= H; ++q) {
+            long long Ph[2] = {0, 0}, Pm[2] = {1LL << 31, 1LL << 31}, Qh[2] = {0, 0}, Qm[2] = {1LL << 31, 1LL << 31};
+            int idx = 0;
+#pragma unroll
+            for (int p = 0; p < H; ++p) {
+                idx += q;
+                if (idx >= R) idx -= R;
+                const int4 w = kRoots.v[O + idx];
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    Ph[c] += (long long)sh[p][c] * w.y;
+                    Pm[c] += (long long)sh[p][c] * w.x;
+                    Pm[c] += (long long)sl[p][c] * w.y;
+                    Qh[c] += (long long)dh[p][c] * w.w;
+                    Qm[c] += (long long)dh[p][c] * w.z;
+                    Qm[c] += (long long)dl[p][c] * w.w;
+                }
+            }
+            const fx2 A = make_longlong2(a05.x + Ph[0] + (Pm[0] >> 32), a05.y + Ph[1] + (Pm[1] >> 32));
+            const fx2 Bv = make_longlong2(Qh[0] + (Qm[0] >> 32), Qh[1] + (Qm[1] >> 32));
+            const fx2 iB = INV ? ftimes_i(Bv) : make_longlong2(Bv.y, -Bv.x);
+            fx2 y = fadd(A, iB), z = fsub(A, iB);
+            if (!INV && twiddled) {
+                y = fmul<true>(y, tw(q * j * step));
+                z = fmul<true>(z, tw((R - q) * j * step));
+            }
+            x[base + q * Ns] = y;
+            x[base + (R - q) * Ns] = z;
+            mag |= fmag(y) | fmag(z);
+        }
+    }
+    return mag;
+}
+
 // Rader pass context: the ring's prime tables, and shared-memory scratch
 // for its convolutions ((N / p) (p - 1) points after the N of the ring)
 struct RaderCtx {
@@ -397,8 +492,8 @@ __device__ __forceinline__ void mx_pass_any(int r, fx2 *x, int Ntot, int Nseq, i
     case 7: mag = mx_pass<7, INV>(x, Ntot, Nseq, B, tw, s); sc.e += pass_bits<7, INV>(Ns); break;
     default:
         if constexpr (BIG) {
-            if (r == 11) mag = mx_pass<11, INV>(x, Ntot, Nseq, B, tw, s);
-            else mag = mx_pass<13, INV>(x, Ntot, Nseq, B, tw, s);
+            if (r == 11) mag = mx_pass_odd<11, INV>(x, Ntot, Nseq, B, tw, s);
+            else mag = mx_pass_odd<13, INV>(x, Ntot, Nseq, B, tw, s);
             sc.e += pass_bits<13, INV>(Ns);
         }
         break;
