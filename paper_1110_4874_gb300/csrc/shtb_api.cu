@@ -20,11 +20,11 @@ size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct Workspace {
     // synthesis
-    double2 *ap = nullptr;      // [nalm][nmaps]
+    double2 *ap = nullptr;      // [nalm][padded_maps]
     double2 *q = nullptr;       // [nmaps][nrings][L+1]  (also the adjoint's q_adj)
     // adjoint
     void *adj = nullptr;        // g + recurrence state
-    double2 *aacc = nullptr;    // [nalm][nmaps]
+    double2 *aacc = nullptr;    // [nalm][padded_maps]
     // host-buffer variants
     double2 *alm = nullptr;     // [nmaps][nalm]
     double *map = nullptr;      // [nmaps][npix]
@@ -41,13 +41,13 @@ size_t alm_bytes(const shtb_plan_s *p, int nmaps) { return sizeof(double2) * (si
 
 size_t adj_bytes(const shtb_plan_s *p, int nmaps)
 {
-    return sizeof(double2) * (size_t)(p->lmax + 1) * 2 * p->nhalf * nmaps +
+    return sizeof(double2) * (size_t)(p->lmax + 1) * 2 * p->nhalf * padded_maps(nmaps) +
            legendre_adjoint_state_bytes(p);
 }
 
 size_t ws_total(const shtb_plan_s *p, int nmaps)
 {
-    return align256(alm_bytes(p, nmaps)) * 2 + align256(q_bytes(p, nmaps)) +
+    return align256(alm_bytes(p, padded_maps(nmaps))) * 2 + align256(q_bytes(p, nmaps)) +
            align256(adj_bytes(p, nmaps)) + align256(alm_bytes(p, nmaps)) +
            align256(sizeof(double) * (size_t)nmaps * p->npix) + align256(bf_workspace_bytes(p));
 }
@@ -56,10 +56,10 @@ Workspace carve(shtb_plan_s *p, int nmaps)
 {
     Workspace w;
     char *c = (char *)p->ws;
-    w.ap = (double2 *)c;    c += align256(alm_bytes(p, nmaps));
+    w.ap = (double2 *)c;    c += align256(alm_bytes(p, padded_maps(nmaps)));
     w.q = (double2 *)c;     c += align256(q_bytes(p, nmaps));
     w.adj = c;              c += align256(adj_bytes(p, nmaps));
-    w.aacc = (double2 *)c;  c += align256(alm_bytes(p, nmaps));
+    w.aacc = (double2 *)c;  c += align256(alm_bytes(p, padded_maps(nmaps)));
     w.alm = (double2 *)c;   c += align256(alm_bytes(p, nmaps));
     w.map = (double *)c;    c += align256(sizeof(double) * (size_t)nmaps * p->npix);
     w.bf = c;
@@ -163,8 +163,9 @@ int run_adjoint(shtb_plan_s *p, const double *map, double2 *alm, int nmaps, cuda
         // transposed butterfly (compressed plans)
         StageTimer t(p, st, 3);
         double2 *g = (double2 *)w.adj;
-        if ((rc = launch_adjoint_parity(p, w.q, g, nmaps, st))) return rc;
-        if ((rc = launch_bf_adjoint(p, g, w.aacc, w.bf, alm, nmaps, st))) return rc;
+        const int columns = padded_maps(nmaps);
+        if ((rc = launch_adjoint_parity(p, w.q, g, nmaps, columns, st))) return rc;
+        if ((rc = launch_bf_adjoint(p, g, w.aacc, w.bf, alm, nmaps, columns, st))) return rc;
         return SHTB_OK;
     }
     {
@@ -513,9 +514,10 @@ int run_adjoint_spin(shtb_plan_s *p, const double *map, double2 *alm, int npairs
     Workspace wp = carve(p, nm), wq = carve(q, nm);
     double2 *g_plus = (double2 *)wp.adj, *g_minus = (double2 *)wq.adj;
     if ((rc = launch_phi_adjoint(p, map, wp.q, nm, st))) return rc;      // ring sums of Q and U
-    if ((rc = launch_spin_uncombine(p, wp.q, g_plus, g_minus, npairs, st))) return rc;
-    if ((rc = launch_bf_adjoint(p, g_plus, wp.aacc, wp.bf, alm, nm, st))) return rc;
-    if ((rc = launch_bf_adjoint(q, g_minus, wq.aacc, wq.bf, wq.alm, nm, st))) return rc;
+    const int columns = padded_maps(nm);
+    if ((rc = launch_spin_uncombine(p, wp.q, g_plus, g_minus, npairs, columns, st))) return rc;
+    if ((rc = launch_bf_adjoint(p, g_plus, wp.aacc, wp.bf, alm, nm, columns, st))) return rc;
+    if ((rc = launch_bf_adjoint(q, g_minus, wq.aacc, wq.bf, wq.alm, nm, columns, st))) return rc;
     return launch_alm_add(p, alm, wq.alm, (size_t)nm * p->nalm, st);
 }
 
@@ -698,7 +700,7 @@ int shtb_test_butterfly(shtb_plan p, const double *alm_dev, double *qt_dev, int 
     cudaStream_t st = (cudaStream_t)stream;
     // the (m = L, t = 1) chain is empty: its entries stay zero
     SHTB_CUDA_TRY(cudaMemsetAsync(qt_dev, 0, sizeof(double2) * 2 * (size_t)nmaps * p->nhalf * (p->lmax + 1), st));
-    return launch_bf_synth(p, (const double2 *)alm_dev, w.ap, w.bf, nullptr, nmaps, st, qt_dev);
+    return launch_bf_synth(p, (const double2 *)alm_dev, w.ap, w.bf, nullptr, nmaps, st, qt_dev, false);
 }
 
 int shtb_test_phi(shtb_plan p, const double *q_dev, double *map_dev, int nmaps, void *stream)

@@ -65,9 +65,9 @@ struct BatchGroupDev {
     const int *ints;
     const uint2 *words;
     const int *depth_parity;
-    double2 *ai;                      // [nalm][nmaps]
-    int nmaps;
-    const double2 *const *alm_of_map; // request a_lm of each merged map
+    double2 *ai;                      // [nalm][columns]
+    int columns;                      // merged maps, padded to a sum of group widths
+    const double2 *const *alm_of_map; // request a_lm of each column (padding repeats the last map)
     double *const *map_of_map;        // request output map of each merged map
 };
 
@@ -92,7 +92,7 @@ __device__ void warp_item(const BatchDev &bd, const BatchWork &w, double *wsm, i
     if (w.type == W_RES) {
         const BfRItem it = G.ritems[w.idx];
         double *ubuf = G.depth_parity[it.m * 2 + it.t] ? M.u1 : M.u0;
-        shtb_dev::bf_r_item<NB, true>(it, G.v.lmax, G.v.nhalf, G.ints, G.words, G.ai, G.nmaps, M.b0, ubuf, M.qt,
+        shtb_dev::bf_r_item<NB, true>(it, G.v.lmax, G.v.nhalf, G.ints, G.words, G.ai, G.columns, M.b0, ubuf, M.qt,
                                       lane);
     } else {
         const double *uin = (w.aux % 2) ? M.u1 : M.u0;
@@ -109,11 +109,11 @@ __device__ void gather_item(const BatchDev &bd, const BatchWork &w, int lane)
     const int m = w.idx, L = G.v.lmax;
     const long long off = shtb_dev::alm_off(L, m);
     const int n = L - m + 1;
-    for (int i = lane; i < n * G.nmaps; i += 32) {
+    for (int i = lane; i < n * G.columns; i += 32) {
         const int b = i / n, dl = i - b * n;
         const long long idx = off + dl;
         const double2 a = G.alm_of_map[b][idx];
-        G.ai[(size_t)idx * G.nmaps + b] = make_double2(a.x, m == 0 ? 0.0 : a.y);
+        G.ai[(size_t)idx * G.columns + b] = make_double2(a.x, m == 0 ? 0.0 : a.y);
     }
 }
 
@@ -219,13 +219,13 @@ struct shtb_batch_s {
     int mode = 0;                     // 0 persistent kernel, 1 stage-kernel graph
     int nstreams = 1;
     struct GMapGroup {
-        int b0, nb, stream;
+        int b0, nb, real, stream;     // columns of the group, and its maps
         double *u0, *u1, *qt;
         double cost;
     };
     struct GPlanGroup {
         shtb_plan_s *plan;
-        int nmaps;
+        int columns;
         double2 *ai;
         const double2 *const *alm_tab;
         double *const *map_tab;
@@ -278,6 +278,26 @@ long long ring_cost(const shtb_plan_s *p, int kind, int r)
     return kind == shtb_dev::kBluestein ? 8 * K * (lg + 1) : K * lg;
 }
 
+// Columns and group widths of a plan's merged maps: groups of the largest
+// power of two up to `width`, the rest padded to a group of its own
+// (padded_maps).  Widths above 8 are not padded, so that a batch that fills
+// one is refused by the width check.
+struct MapGroups {
+    int width, nmaps, columns;
+    MapGroups(int w, int n) : width(1), nmaps(n)
+    {
+        while (2 * width <= w) width *= 2;
+        columns = width > 8 ? n : padded_maps(n, width);
+    }
+    int next(int b0) const                 // width of the group at column b0
+    {
+        if (width <= 8) return std::min(width, group_width(columns - b0));
+        int nb = 1;
+        while (nb * 2 <= std::min(nmaps - b0, width)) nb *= 2;
+        return nb;
+    }
+};
+
 // Builds the work list, packs and device tables for `warps` warps per block
 // and map groups of at most `width` maps; work inside a phase in decreasing
 // size (lpt = 1) or in plan order (lpt = 0).
@@ -316,11 +336,15 @@ int build_schedule(shtb_batch_s *b, int warps, int width, int lpt)
         D.ints = bf.ints;
         D.words = bf.words();
         D.depth_parity = bf.depth_parity;
-        D.nmaps = G.nmaps;
+        const MapGroups groups(width, G.nmaps);
+        const int columns = groups.columns;
+        std::vector<const double2 *> alm_of_col = G.alm_of_map;
+        alm_of_col.resize(columns, G.alm_of_map.back());
+        D.columns = columns;
         void *d;
-        if ((rc = balloc(b->sched_allocs, &d, sizeof(double2) * (size_t)p->nalm * G.nmaps))) return rc;
+        if ((rc = balloc(b->sched_allocs, &d, sizeof(double2) * (size_t)p->nalm * columns))) return rc;
         D.ai = (double2 *)d;
-        if ((rc = balloc(b->sched_allocs, &d, sizeof(void *) * G.nmaps, G.alm_of_map.data()))) return rc;
+        if ((rc = balloc(b->sched_allocs, &d, sizeof(void *) * columns, alm_of_col.data()))) return rc;
         D.alm_of_map = (const double2 *const *)d;
         if ((rc = balloc(b->sched_allocs, &d, sizeof(void *) * G.nmaps, G.map_of_map.data()))) return rc;
         D.map_of_map = (double *const *)d;
@@ -334,7 +358,7 @@ int build_schedule(shtb_batch_s *b, int warps, int width, int lpt)
         const int gather_cnt = ug.cnt;
         for (int m = 0; m <= p->lmax; ++m) {
             ug.items.push_back({W_GATHER, (int)g, 0, m, 0, 0});
-            ug.cost.push_back((long long)(p->lmax - m + 1) * G.nmaps);
+            ug.cost.push_back((long long)(p->lmax - m + 1) * columns);
         }
         const int gather_total = (int)ug.items.size();
         units.push_back(std::move(ug));
@@ -350,10 +374,8 @@ int build_schedule(shtb_batch_s *b, int warps, int width, int lpt)
                                          cudaMemcpyDeviceToHost));
         }
         // ---- map groups of power-of-two widths up to `width`
-        for (int b0 = 0; b0 < G.nmaps;) {
-            const int left = G.nmaps - b0;
-            int nb = 1;
-            while (nb * 2 <= std::min(left, width)) nb *= 2;
+        for (int b0 = 0; b0 < columns;) {
+            const int nb = groups.next(b0), real = std::min(nb, G.nmaps - b0);
             cmax = std::max(cmax, 2 * nb);
             BatchMG M{};
             M.b0 = b0;
@@ -392,7 +414,7 @@ int build_schedule(shtb_batch_s *b, int warps, int width, int lpt)
                 units.push_back(std::move(u));
             }
             Unit ur{2 + dmax, dep, need, ncounters++, 1, {}, {}};
-            for (int bl = 0; bl < nb; ++bl)
+            for (int bl = 0; bl < real; ++bl)
                 for (int r = 0; r < p->nrings; ++r) {
                     ur.items.push_back({W_PHI, (int)g, mg, r, bl, kind[r]});
                     ur.cost.push_back(ring_cost(p, kind[r], r));
@@ -489,22 +511,24 @@ int build_graph_schedule(shtb_batch_s *b, int width, int nstreams)
         const BfPlanDev &bf = *p->bf;
         shtb_batch_s::GPlanGroup P{};
         P.plan = p;
-        P.nmaps = G.nmaps;
-        if ((rc = balloc(b->sched_allocs, &d, sizeof(double2) * (size_t)p->nalm * G.nmaps))) return rc;
+        const MapGroups groups(width, G.nmaps);
+        P.columns = groups.columns;
+        std::vector<const double2 *> alm_of_col = G.alm_of_map;
+        alm_of_col.resize(P.columns, G.alm_of_map.back());
+        if ((rc = balloc(b->sched_allocs, &d, sizeof(double2) * (size_t)p->nalm * P.columns))) return rc;
         P.ai = (double2 *)d;
-        if ((rc = balloc(b->sched_allocs, &d, sizeof(void *) * G.nmaps, G.alm_of_map.data()))) return rc;
+        if ((rc = balloc(b->sched_allocs, &d, sizeof(void *) * P.columns, alm_of_col.data()))) return rc;
         P.alm_tab = (const double2 *const *)d;
         if ((rc = balloc(b->sched_allocs, &d, sizeof(void *) * G.nmaps, G.map_of_map.data()))) return rc;
         P.map_tab = (double *const *)d;
         const double per_map = 4.0 * (double)(bf.n_dense + bf.n_r) + 2.0 * (double)bf.n_ident +
                                p->stats.phi_flops_per_map;
-        for (int b0 = 0; b0 < G.nmaps;) {
-            const int left = G.nmaps - b0;
-            int nb = 1;
-            while (nb * 2 <= std::min(left, width)) nb *= 2;
+        for (int b0 = 0; b0 < P.columns;) {
+            const int nb = groups.next(b0);
             shtb_batch_s::GMapGroup M{};
             M.b0 = b0;
             M.nb = nb;
+            M.real = std::min(nb, G.nmaps - b0);
             M.cost = per_map * nb;
             const size_t entry = sizeof(double) * 2 * nb;
             if ((rc = balloc(b->sched_allocs, &d, entry * (size_t)bf.u_entries))) return rc;
@@ -546,16 +570,16 @@ int enqueue_graph(shtb_batch_s *b, cudaStream_t st)
 {
     int rc;
     for (auto &P : b->gg)
-        if ((rc = launch_bf_gather(P.plan, P.alm_tab, P.ai, P.nmaps, st))) return rc;
+        if ((rc = launch_bf_gather(P.plan, P.alm_tab, P.ai, P.columns, st))) return rc;
     // fork: every side stream starts after the gathers
     SHTB_CUDA_TRY(cudaEventRecord(b->fork_join[0], st));
     for (int s = 1; s < b->nstreams; ++s) SHTB_CUDA_TRY(cudaStreamWaitEvent(b->side[s - 1], b->fork_join[0], 0));
     for (auto &P : b->gg) {
         for (auto &M : P.mgs) {
             cudaStream_t ss = M.stream == 0 ? st : b->side[M.stream - 1];
-            if ((rc = launch_bf_legendre_group(P.plan, P.ai, P.nmaps, M.b0, M.nb, M.u0, M.u1, M.qt, ss)))
+            if ((rc = launch_bf_legendre_group(P.plan, P.ai, P.columns, M.b0, M.nb, M.u0, M.u1, M.qt, ss)))
                 return rc;
-            if ((rc = launch_phi_synth_qt_ptr(P.plan, M.qt, M.nb, P.map_tab, M.b0, ss))) return rc;
+            if ((rc = launch_phi_synth_qt_ptr(P.plan, M.qt, M.real, P.map_tab, M.b0, ss))) return rc;
         }
     }
     // join

@@ -49,30 +49,31 @@ __device__ __forceinline__ double2 staged(double2 a, long long i, long long L, c
     return sig ? make_double2(a.x * s, i <= L ? 0.0 : a.y * s) : make_double2(a.x, i <= L ? 0.0 : a.y);
 }
 
+// ai has `columns` >= nmaps columns, those past nmaps repeating the last map
 __global__ void __launch_bounds__(256) bf_interleave_kernel(PlanView v, const double2 *__restrict__ alm,
-                                                            double2 *__restrict__ ai, int nmaps,
+                                                            double2 *__restrict__ ai, int nmaps, int columns,
                                                             const RecCoef *__restrict__ sig)
 {
     __shared__ double2 tile[2 * kStageTile];
     const long long nalm = v.nalm, L = v.lmax;
-    if (nmaps == 1) {
+    if (columns == 1) {
         for (long long i = blockIdx.x * 256LL + threadIdx.x; i < nalm; i += 256LL * gridDim.x)
             ai[i] = staged(alm[i], i, L, sig);
         return;
     }
-    const StageTile st(nmaps);
+    const StageTile st(columns);
     for (long long i0 = (long long)blockIdx.x * st.T; i0 < nalm; i0 += (long long)st.T * gridDim.x) {
         const int nt = (int)min((long long)st.T, nalm - i0);
-        for (int b0 = 0; b0 < nmaps; b0 += st.MB) {
-            const int mb = min(st.MB, nmaps - b0);
+        for (int b0 = 0; b0 < columns; b0 += st.MB) {
+            const int mb = min(st.MB, columns - b0);
             for (int e = threadIdx.x; e < nt * mb; e += blockDim.x) {
                 const int b = e / nt, t = e - b * nt;
-                tile[b * (st.T + 1) + t] = alm[(size_t)(b0 + b) * nalm + i0 + t];
+                tile[b * (st.T + 1) + t] = alm[(size_t)min(b0 + b, nmaps - 1) * nalm + i0 + t];
             }
             __syncthreads();
             for (int e = threadIdx.x; e < nt * mb; e += blockDim.x) {
                 const int t = e / mb, b = e - t * mb;
-                ai[(size_t)(i0 + t) * nmaps + b0 + b] = staged(tile[b * (st.T + 1) + t], i0 + t, L, sig);
+                ai[(size_t)(i0 + t) * columns + b0 + b] = staged(tile[b * (st.T + 1) + t], i0 + t, L, sig);
             }
             __syncthreads();
         }
@@ -182,16 +183,16 @@ int launch_levels(const shtb_plan_s *p, double *u0, double *u1, double *qt, cuda
 }
 
 // One map group: residual blocks, butterfly levels, then (map != nullptr)
-// the ring stage.  With map == nullptr the group's q^t is the caller's
-// array (the Legendre stage alone).
+// the ring stage of the group's first `real` maps.  With map == nullptr the
+// group's q^t is the caller's array (the Legendre stage alone).
 template <int NB>
-int run_group(const shtb_plan_s *p, const double2 *ai, int nmaps, int b0, double *u0, double *u1,
+int run_group(const shtb_plan_s *p, const double2 *ai, int columns, int b0, int real, double *u0, double *u1,
               double *qt, double *map, cudaStream_t st)
 {
     shtb_plan_s *pp = const_cast<shtb_plan_s *>(p);
     const int ev_leg = profile_begin(pp, st);
     int ev = profile_begin(pp, st);
-    int rc = launch_r<NB>(p, ai, nmaps, b0, u0, u1, qt, st);
+    int rc = launch_r<NB>(p, ai, columns, b0, u0, u1, qt, st);
     if (rc) return rc;
     profile_end(pp, st, 5, ev);
     ev = profile_begin(pp, st);
@@ -201,7 +202,7 @@ int run_group(const shtb_plan_s *p, const double2 *ai, int nmaps, int b0, double
     if (!map) return SHTB_OK;
     // ring stage of this group straight from q^0, q^1 (parity combine fused)
     ev = profile_begin(pp, st);
-    rc = launch_phi_synth_qt(p, qt, NB, map, b0, st);
+    rc = launch_phi_synth_qt(p, qt, real, map, b0, st);
     profile_end(pp, st, 1, ev);
     return rc;
 }
@@ -427,7 +428,7 @@ bf_adj_r_rec_kernel(PlanView v, const BfRGroup *__restrict__ groups, int ngroups
 // non-null (plans that regenerate R: the residual adjoint sums V, not
 // Ptilde = sigma V)
 __global__ void __launch_bounds__(256) bf_finish_kernel(PlanView v, const double2 *__restrict__ aacc,
-                                                        double2 *__restrict__ alm, int nmaps,
+                                                        double2 *__restrict__ alm, int nmaps, int columns,
                                                         const RecCoef *__restrict__ sig)
 {
     __shared__ double2 tile[2 * kStageTile];
@@ -437,7 +438,7 @@ __global__ void __launch_bounds__(256) bf_finish_kernel(PlanView v, const double
         return idx <= L ? make_double2(sig ? a.x * cs : a.x, 0.0)
                         : make_double2(sig ? cs * a.x : 2.0 * a.x, sig ? cs * a.y : 2.0 * a.y);
     };
-    if (nmaps == 1) {
+    if (columns == 1) {
         for (long long i = blockIdx.x * 256LL + threadIdx.x; i < nalm; i += 256LL * gridDim.x)
             alm[i] = scaled(aacc[i], i);
         return;
@@ -449,7 +450,7 @@ __global__ void __launch_bounds__(256) bf_finish_kernel(PlanView v, const double
             const int mb = min(st.MB, nmaps - b0);
             for (int e = threadIdx.x; e < nt * mb; e += blockDim.x) {
                 const int t = e / mb, b = e - t * mb;
-                tile[b * (st.T + 1) + t] = aacc[(size_t)(i0 + t) * nmaps + b0 + b];
+                tile[b * (st.T + 1) + t] = aacc[(size_t)(i0 + t) * columns + b0 + b];
             }
             __syncthreads();
             for (int e = threadIdx.x; e < nt * mb; e += blockDim.x) {
@@ -582,31 +583,34 @@ size_t bf_workspace_bytes(const shtb_plan_s *p)
 }
 
 int launch_bf_synth(const shtb_plan_s *p, const double2 *alm, double2 *ai, void *ws, double *map,
-                    int nmaps, cudaStream_t st, double *qt_out)
+                    int nmaps, cudaStream_t st, double *qt_out, bool padded)
 {
     const BfPlanDev &bf = *p->bf;
     const size_t entry = 16;
     double *u0 = (double *)ws;
     double *u1 = u0 + (size_t)bf.u_entries * entry;
     double *qt_ws = u1 + (size_t)bf.u_entries * entry;
-    // q^t of map b in the caller's [nmaps][2][nhalf][L+1] array (Legendre stage alone)
+    const int columns = padded ? padded_maps(nmaps) : nmaps;
+    // q^t of map b in the caller's [columns][2][nhalf][L+1] array (Legendre stage alone)
     const size_t qt_map = (size_t)4 * p->nhalf * (p->lmax + 1);
-    auto qt_of = [&](int b0) { return qt_out ? qt_out + (size_t)b0 * qt_map : qt_ws; };
     const int ev = profile_begin(const_cast<shtb_plan_s *>(p), st);
-    bf_interleave_kernel<<<stage_grid(p, nmaps), 256, 0, st>>>(p->view, alm, ai, nmaps,
-                                                               p->bf->rec ? p->view.coef : nullptr);
+    bf_interleave_kernel<<<stage_grid(p, columns), 256, 0, st>>>(p->view, alm, ai, nmaps, columns,
+                                                                 p->bf->rec ? p->view.coef : nullptr);
     SHTB_CUDA_TRY(cudaGetLastError());
     ++p->launches;
     profile_end(const_cast<shtb_plan_s *>(p), st, 4, ev);
-    for (int b0 = 0; b0 < nmaps;) {
-        const int left = nmaps - b0;
+    for (int b0 = 0; b0 < columns;) {
+        const int nb = group_width(columns - b0), real = std::min(nb, nmaps - b0);
+        double *qt = qt_out ? qt_out + (size_t)b0 * qt_map : qt_ws;
         int rc;
-        double *qt = qt_of(b0);
-        if (left >= 8) { rc = run_group<8>(p, ai, nmaps, b0, u0, u1, qt, map, st); b0 += 8; }
-        else if (left >= 4) { rc = run_group<4>(p, ai, nmaps, b0, u0, u1, qt, map, st); b0 += 4; }
-        else if (left >= 2) { rc = run_group<2>(p, ai, nmaps, b0, u0, u1, qt, map, st); b0 += 2; }
-        else { rc = run_group<1>(p, ai, nmaps, b0, u0, u1, qt, map, st); b0 += 1; }
+        switch (nb) {
+        case 8: rc = run_group<8>(p, ai, columns, b0, real, u0, u1, qt, map, st); break;
+        case 4: rc = run_group<4>(p, ai, columns, b0, real, u0, u1, qt, map, st); break;
+        case 2: rc = run_group<2>(p, ai, columns, b0, real, u0, u1, qt, map, st); break;
+        default: rc = run_group<1>(p, ai, columns, b0, real, u0, u1, qt, map, st); break;
+        }
         if (rc) return rc;
+        b0 += nb;
     }
     return SHTB_OK;
 }
@@ -624,24 +628,24 @@ int launch_bf_synth_to_host(shtb_plan_s *p, const double2 *alm, double2 *ai, voi
     double *u0 = (double *)ws;
     double *u1 = u0 + (size_t)bf.u_entries * entry;
     double *qt = u1 + (size_t)bf.u_entries * entry;
-    bf_interleave_kernel<<<stage_grid(p, nmaps), 256, 0, st>>>(p->view, alm, ai, nmaps,
-                                                               p->bf->rec ? p->view.coef : nullptr);
+    const int columns = padded_maps(nmaps);
+    bf_interleave_kernel<<<stage_grid(p, columns), 256, 0, st>>>(p->view, alm, ai, nmaps, columns,
+                                                                 p->bf->rec ? p->view.coef : nullptr);
     SHTB_CUDA_TRY(cudaGetLastError());
     ++p->launches;
-    for (int b0 = 0; b0 < nmaps;) {
-        const int left = nmaps - b0;
-        const int nb = left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
-        int rc = launch_bf_legendre_group(p, ai, nmaps, b0, nb, u0, u1, qt, st);
+    for (int b0 = 0; b0 < columns;) {
+        const int nb = group_width(columns - b0), real = std::min(nb, nmaps - b0);
+        int rc = launch_bf_legendre_group(p, ai, columns, b0, nb, u0, u1, qt, st);
         if (rc) return rc;
         // ring stage chunk by chunk; each chunk's pixels go back while the
         // next chunk (or the next map group) computes
         for (int c = 0; c < NCH; ++c) {
-            if ((rc = launch_phi_synth_qt_chunk(p, qt, nb, map, b0, c, st))) return rc;
+            if ((rc = launch_phi_synth_qt_chunk(p, qt, real, map, b0, c, st))) return rc;
             const long long p0 = p->chunk_pix[c], p1 = p->chunk_pix[c + 1];
             if (p1 == p0) continue;
             SHTB_CUDA_TRY(cudaEventRecord(p->chunk_ev[c], st));
             SHTB_CUDA_TRY(cudaStreamWaitEvent(p->copy_stream, p->chunk_ev[c], 0));
-            for (int b = b0; b < b0 + nb; ++b)
+            for (int b = b0; b < b0 + real; ++b)
                 SHTB_CUDA_TRY(cudaMemcpyAsync(map_host + (size_t)b * p->npix + p0, map + (size_t)b * p->npix + p0,
                                               sizeof(double) * (size_t)(p1 - p0), cudaMemcpyDeviceToHost,
                                               p->copy_stream));
@@ -655,22 +659,25 @@ int launch_bf_synth_to_host(shtb_plan_s *p, const double2 *alm, double2 *ai, voi
 }
 
 int launch_bf_adjoint(const shtb_plan_s *p, const double2 *g, double2 *aacc, void *ws, double2 *alm,
-                      int nmaps, cudaStream_t st)
+                      int nmaps, int columns, cudaStream_t st)
 {
     const BfPlanDev &bf = *p->bf;
     const size_t entry = 16;
     double *u0 = (double *)ws;
     double *u1 = u0 + (size_t)bf.u_entries * entry;
-    for (int b0 = 0; b0 < nmaps;) {
-        const int left = nmaps - b0;
+    for (int b0 = 0; b0 < columns;) {
+        const int nb = group_width(columns - b0);
         int rc;
-        if (left >= 8) { rc = run_adj_group<8>(p, g, nmaps, b0, u0, u1, aacc, st); b0 += 8; }
-        else if (left >= 4) { rc = run_adj_group<4>(p, g, nmaps, b0, u0, u1, aacc, st); b0 += 4; }
-        else if (left >= 2) { rc = run_adj_group<2>(p, g, nmaps, b0, u0, u1, aacc, st); b0 += 2; }
-        else { rc = run_adj_group<1>(p, g, nmaps, b0, u0, u1, aacc, st); b0 += 1; }
+        switch (nb) {
+        case 8: rc = run_adj_group<8>(p, g, columns, b0, u0, u1, aacc, st); break;
+        case 4: rc = run_adj_group<4>(p, g, columns, b0, u0, u1, aacc, st); break;
+        case 2: rc = run_adj_group<2>(p, g, columns, b0, u0, u1, aacc, st); break;
+        default: rc = run_adj_group<1>(p, g, columns, b0, u0, u1, aacc, st); break;
+        }
         if (rc) return rc;
+        b0 += nb;
     }
-    bf_finish_kernel<<<stage_grid(p, nmaps), 256, 0, st>>>(p->view, aacc, alm, nmaps,
+    bf_finish_kernel<<<stage_grid(p, nmaps), 256, 0, st>>>(p->view, aacc, alm, nmaps, columns,
                                                            p->bf->rec ? p->view.coef : nullptr);
     SHTB_CUDA_TRY(cudaGetLastError());
     ++p->launches;

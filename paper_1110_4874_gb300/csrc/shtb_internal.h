@@ -236,7 +236,8 @@ int launch_legendre_adjoint(const shtb_plan_s *p, const double2 *qadj, double2 *
                             int nmaps, void *state_ws, cudaStream_t st);
 int launch_alm_finish(const shtb_plan_s *p, const double2 *aacc, double2 *alm, int nmaps,
                       cudaStream_t st);
-int launch_adjoint_parity(const shtb_plan_s *p, const double2 *qadj, double2 *g, int nmaps,
+// g has `columns` >= nmaps columns, those past nmaps repeating the last map
+int launch_adjoint_parity(const shtb_plan_s *p, const double2 *qadj, double2 *g, int nmaps, int columns,
                           cudaStream_t st);
 size_t legendre_adjoint_state_bytes(const shtb_plan_s *p);
 
@@ -263,7 +264,7 @@ int launch_spin_combine(const shtb_plan_s *p, const double *qt_plus, const doubl
 // ... and its transpose: ring sums of Q, U -> entry-major parity gradients of
 // the F+ and F- butterflies; alm += add over n complex entries
 int launch_spin_uncombine(const shtb_plan_s *p, const double2 *G, double2 *g_plus, double2 *g_minus, int npairs,
-                          cudaStream_t st);
+                          int columns, cudaStream_t st);
 int launch_alm_add(const shtb_plan_s *p, double2 *alm, const double2 *add, size_t n, cudaStream_t st);
 
 // analysis (shtb_analysis.cu): quadrature weighting of a map or a residual,
@@ -273,11 +274,28 @@ int launch_ring_weight(const shtb_plan_s *p, const double *f, const double *y, c
 int launch_alm_quadrature_add(const shtb_plan_s *p, const double2 *g, double2 *alm, int nmaps,
                               bool first, cudaStream_t st);
 
+// Map groups.  The butterfly carries 8, 4, 2 or 1 maps an entry, and a group
+// of 4 costs little more than one of 1 (block products at Nside = 512: 0.80,
+// 0.95, 1.23 and 1.57 ms for 1, 2, 4 and 8 maps), so the maps left after the
+// eights are padded to the next of these widths and run as one group, in
+// place of several.  The a_lm-sided arrays [idx][maps] have padded_maps
+// columns; the padding repeats the last map and is never returned.
+inline int padded_maps(int nmaps, int width = 8)
+{
+    const int rest = nmaps % width;
+    int pad = 1;
+    while (pad < rest) pad *= 2;
+    return nmaps - rest + (rest ? pad : 0);
+}
+// width of the group that starts `left` padded columns before the end
+inline int group_width(int left) { return left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1; }
+
 size_t bf_workspace_bytes(const shtb_plan_s *p);
 // map != nullptr: the whole synthesis; map == nullptr: the Legendre stage
 // alone, q^t of map b written to qt_out + b [2][nhalf][L+1] complex
+// (padded: ai and qt_out have padded_maps(nmaps) columns and maps)
 int launch_bf_synth(const shtb_plan_s *p, const double2 *alm, double2 *ai, void *ws, double *map,
-                    int nmaps, cudaStream_t st, double *qt_out = nullptr);
+                    int nmaps, cudaStream_t st, double *qt_out = nullptr, bool padded = true);
 // whole synthesis with the maps copied back to host memory as the ring
 // stage finishes each chunk of rings (the copies overlap the rest)
 int launch_bf_synth_to_host(shtb_plan_s *p, const double2 *alm, double2 *ai, void *ws, double *map,
@@ -290,8 +308,9 @@ int launch_bf_gather(const shtb_plan_s *p, const double2 *const *alm_of_map, dou
                      cudaStream_t st);
 int launch_bf_legendre_group(const shtb_plan_s *p, const double2 *ai, int nmaps, int b0, int nb, double *u0,
                              double *u1, double *qt, cudaStream_t st);
+// g and aacc with `columns` columns (a sum of group widths)
 int launch_bf_adjoint(const shtb_plan_s *p, const double2 *g, double2 *aacc, void *ws, double2 *alm,
-                      int nmaps, cudaStream_t st);
+                      int nmaps, int columns, cudaStream_t st);
 
 // shtb_util.cu
 int measure_fp64_peak(int device, double *dfma, double *dmma);

@@ -175,18 +175,18 @@ legendre_synth_kernel(PlanView v, const double2 *__restrict__ ap, double2 *__res
 constexpr int kParityM = 64, kParityMaps = 16;
 
 __global__ void __launch_bounds__(256) adjoint_parity_kernel(PlanView v, const double2 *__restrict__ qa,
-                                                             double2 *__restrict__ g, int nmaps)
+                                                             double2 *__restrict__ g, int nmaps, int columns)
 {
     __shared__ double2 tile[2][kParityMaps][kParityM];     // north, south
     const int r = blockIdx.x, m0 = blockIdx.y * kParityM;
     const int Z = v.nhalf, L = v.lmax;
     const int nm = min(kParityM, L + 1 - m0);
     const bool equator = r == Z - 1;
-    for (int b0 = 0; b0 < nmaps; b0 += kParityMaps) {
-        const int nb = min(kParityMaps, nmaps - b0);
+    for (int b0 = 0; b0 < columns; b0 += kParityMaps) {
+        const int nb = min(kParityMaps, columns - b0);
         for (int i = threadIdx.x; i < nb * nm; i += blockDim.x) {
             const int b = i / nm, ml = i - b * nm;
-            const size_t row = (size_t)(b0 + b) * v.nrings;
+            const size_t row = (size_t)min(b0 + b, nmaps - 1) * v.nrings;
             tile[0][b][ml] = qa[(row + r) * (L + 1) + m0 + ml];
             tile[1][b][ml] = equator ? make_double2(0.0, 0.0) : qa[(row + (v.nrings - 1 - r)) * (L + 1) + m0 + ml];
         }
@@ -195,8 +195,8 @@ __global__ void __launch_bounds__(256) adjoint_parity_kernel(PlanView v, const d
             const int ml = i / nb, b = i - ml * nb;
             const double2 a = tile[0][b][ml], c = tile[1][b][ml];
             const size_t m = (size_t)(m0 + ml);
-            g[((m * 2 + 0) * Z + r) * nmaps + b0 + b] = make_double2(a.x + c.x, a.y + c.y);
-            g[((m * 2 + 1) * Z + r) * nmaps + b0 + b] = make_double2(a.x - c.x, a.y - c.y);
+            g[((m * 2 + 0) * Z + r) * columns + b0 + b] = make_double2(a.x + c.x, a.y + c.y);
+            g[((m * 2 + 1) * Z + r) * columns + b0 + b] = make_double2(a.x - c.x, a.y - c.y);
         }
         __syncthreads();
     }
@@ -421,11 +421,11 @@ size_t legendre_adjoint_state_bytes(const shtb_plan_s *p)
     return sizeof(RecState) * (size_t)(p->lmax + 1) * p->nhalf;
 }
 
-int launch_adjoint_parity(const shtb_plan_s *p, const double2 *qadj, double2 *g, int nmaps,
+int launch_adjoint_parity(const shtb_plan_s *p, const double2 *qadj, double2 *g, int nmaps, int columns,
                           cudaStream_t st)
 {
     adjoint_parity_kernel<<<dim3(p->nhalf, (p->lmax + kParityM) / kParityM), 256, 0, st>>>(p->view, qadj, g,
-                                                                                           nmaps);
+                                                                                           nmaps, columns);
     ++p->launches;
     SHTB_CUDA_TRY(cudaGetLastError());
     return SHTB_OK;
@@ -437,7 +437,7 @@ int launch_legendre_adjoint(const shtb_plan_s *p, const double2 *qadj, double2 *
     // ws: [g: (L+1)*2*Z*nmaps double2][state: (L+1)*Z RecState]
     double2 *g = (double2 *)ws;
     RecState *state = (RecState *)(g + (size_t)(p->lmax + 1) * 2 * p->nhalf * nmaps);
-    int rc0 = launch_adjoint_parity(p, qadj, g, nmaps, st);
+    int rc0 = launch_adjoint_parity(p, qadj, g, nmaps, nmaps, st);
     if (rc0) return rc0;
     for (int b0 = 0; b0 < nmaps;) {
         const int left = nmaps - b0;

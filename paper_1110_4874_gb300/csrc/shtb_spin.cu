@@ -48,20 +48,21 @@ __global__ void spin_combine_kernel(int L, int nhalf, int nrings, const double2 
 // folded onto the half-rings by the transposed mirror (F+: g^0 = g_N + g_S,
 // g^1 = g_N - g_S; F-: g^0 = g_N - g_S, g^1 = g_N + g_S; the equator has no
 // mirror), in the entry-major layout of the adjoint butterflies,
-// g[((m * 2 + t) * nhalf + r) * nmaps + b] with b = 2 pair (E), 2 pair + 1 (B).
+// g[((m * 2 + t) * nhalf + r) * columns + b] with b = 2 pair (E), 2 pair + 1 (B),
+// the columns past the last pair repeating it.
 // One CTA per (half-ring, block of kSpinM orders); threads run over
 // (order, input) with the input fastest, so the stores are contiguous.
 constexpr int kSpinM = 32;
 
-__global__ void spin_uncombine_kernel(int L, int nhalf, int nrings, int npairs, const double2 *__restrict__ G,
+__global__ void spin_uncombine_kernel(int L, int nhalf, int nrings, int npairs, int columns, const double2 *__restrict__ G,
                                       double2 *__restrict__ gp, double2 *__restrict__ gm)
 {
     const int r = blockIdx.x, m0 = blockIdx.y * kSpinM;
-    const int nm = min(kSpinM, L + 1 - m0), nb = 2 * npairs;
+    const int nm = min(kSpinM, L + 1 - m0), nb = columns;
     const bool equator = r == nhalf - 1;
     const int south = nrings - 1 - r;
     for (int i = threadIdx.x; i < nm * nb; i += blockDim.x) {
-        const int ml = i / nb, b = i - ml * nb, pair = b >> 1;
+        const int ml = i / nb, b = i - ml * nb, pair = min(b >> 1, npairs - 1);
         const size_t m = (size_t)(m0 + ml);
         const double2 *gq = G + (size_t)(2 * pair) * nrings * (L + 1) + m;
         const double2 *gu = gq + (size_t)nrings * (L + 1);
@@ -102,10 +103,10 @@ __global__ void alm_add_kernel(double2 *__restrict__ alm, const double2 *__restr
 }  // namespace
 
 int launch_spin_uncombine(const shtb_plan_s *p, const double2 *G, double2 *g_plus, double2 *g_minus, int npairs,
-                          cudaStream_t st)
+                          int columns, cudaStream_t st)
 {
     spin_uncombine_kernel<<<dim3((unsigned)p->nhalf, (unsigned)((p->lmax + kSpinM) / kSpinM)), 256, 0, st>>>(
-        p->lmax, p->nhalf, p->nrings, npairs, G, g_plus, g_minus);
+        p->lmax, p->nhalf, p->nrings, npairs, columns, G, g_plus, g_minus);
     ++p->launches;
     SHTB_CUDA_TRY(cudaGetLastError());
     return SHTB_OK;
