@@ -5,10 +5,10 @@
 // Synthesis: for every order m and half-ring r (z_r >= 0)
 //   q^t_m(z_r) = sum_j a_{m+t+2j, m} Ptilde_{m+t+2j}^m(z_r),  t = 0 (even), 1 (odd),
 // then q_m(+z_r) = q^0 + q^1 and q_m(-z_r) = q^0 - q^1 (the mirror ring).
-// A warp owns 32 consecutive half-rings of one m, each lane runs both parity
-// chains of its ring in registers and accumulates all maps of the batch, so
-// the per-l constants and a_lm are warp-uniform (broadcast) loads.  Each
-// chain starts at its own crop point (first |Ptilde| >= 1e-30, Appendix) with
+// A warp owns 32 consecutive half-rings of one m and one parity; each lane
+// runs the chain of its ring in registers and accumulates all maps of the
+// batch, so the per-l constants and a_lm are warp-uniform (broadcast) loads.
+// Each chain starts at its own crop point (first |Ptilde| >= 1e-30, Appendix) with
 // two precomputed values and advances by two FMAs per step:
 //   w_j = mu_j x_r + C_j,   V_{j+1} = w_j V_j - V_{j-1},   Ptilde = sigma V,
 // the scale sigma being folded into a_lm by the prescale kernel.
@@ -16,11 +16,29 @@
 // Adjoint: a^t_{m+t+2j} = sum_r V_j(r) g^t_r with g^0 = F(+z) + F(-z) and
 // g^1 = F(+z) - F(-z).  The sum runs across the rings, i.e. across lanes, so
 // each warp writes a 32 (j) x 32 (ring) tile of V to shared memory and then
-// lets lane = j accumulate over the tile's rings with FMAs; the partial sums
-// of a block's warps are added in shared memory and written once.
+// lets lane = j sum over the tile's rings.
+//
+// The recurrence runs in FP64; the sums over the maps, 2 NB of them a value
+// of V, are integer (LegSums): V and the a or g of a chain are cut to limbs
+// at common exponents, and a product is three 32-bit multiply-adds.  The FP64
+// pipe, which takes a warp's DFMA in 16 clocks of an SM against half a clock
+// for an integer multiply-add, held these kernels with both done in FP64.
+// Legendre stage, FP64 sums -> this (ms):
+//   nside 64, lmax 128, 1 map      synthesis  .047 -> .028  adjoint  .054 -> .037
+//   nside 100, lmax 255, 1 map                .095 -> .051           .140 -> .085
+//   nside 256, lmax 512, 4 maps               .996 -> .418          1.385 -> .555
+//   nside 256, lmax 512, 8 maps              1.730 -> .711          2.416 -> .931
+//   nside 512, lmax 1024, 8 maps             12.22 -> 4.89          13.94 -> 5.48
+// What bounds them now is issue (48 % of the slots with 8 maps, the FP64 pipe
+// at 31 %) and, with few maps, the chain of dependent FMAs of the recurrence.
+// The sums keep 55 bits of a or g below the largest of a chain and 58 of V,
+// and end no further from the exact transform than sums of FMAs: over nside
+// 32..1024 both are 9.5e-16 .. 2.8e-14 of the result's norm away, which is the
+// recurrence's own rounding.
 #include <cuda_runtime.h>
 
 #include "shtb_internal.h"
+#include "shtb_limbs.cuh"
 
 namespace {
 
@@ -59,107 +77,268 @@ __global__ void alm_prescale_kernel(PlanView v, const double2 *__restrict__ alm,
     }
 }
 
+// Range of effective exponents the integer sums take, for the a of a chain
+// (per component) and for the V of a ring (the recurrence starts at 1e-30)
+constexpr int kLegExpLo = 300, kLegExpHi = 1700;
+
+// Bits of V, so that sums of n products of 55-bit a and V fit: between two
+// carries 32 products of 27-bit by 30-bit high limbs stay below 2^62, and the
+// words carried out, n 2^57 2^-40 in all, below 2^31 up to chains of 8192.
+__device__ __forceinline__ int v_bits(int n)
+{
+    return 58 - max(0, 32 - __clz(n) - 13);
+}
+
+// The values of one chain that a warp's sums weight: `count` entries of C
+// components, entry i at src + i stride (doubles).  scan: the largest
+// exponent of each component over all of them, kept by lanes b < NB for
+// components 2b, 2b + 1 (0: zero; -1: take the component in FP64).
 template <int NB>
-__global__ void __launch_bounds__(32 * kWarpsPerBlock)
+__device__ __forceinline__ int2 scan_chain(const double *src, size_t stride, int count, int lane)
+{
+    constexpr int STEP = 32 / NB;
+    const int b = lane % NB, r = lane / NB;
+    int e0 = 0, e1 = 0;
+    unsigned nz0 = 0, nz1 = 0;
+#pragma unroll 4
+    for (int i = r; i < count; i += STEP) {
+        const double2 x = __ldg(reinterpret_cast<const double2 *>(src + (size_t)i * stride) + b);
+        e0 = max(e0, shtb_dev::exp_bits(x.x));
+        e1 = max(e1, shtb_dev::exp_bits(x.y));
+        nz0 |= (unsigned)__double2hiint(x.x) << 1 | (unsigned)__double2loint(x.x);
+        nz1 |= (unsigned)__double2hiint(x.y) << 1 | (unsigned)__double2loint(x.y);
+    }
+#pragma unroll
+    for (int o = NB; o < 32; o *= 2) {
+        e0 = max(e0, __shfl_xor_sync(0xffffffffu, e0, o));
+        e1 = max(e1, __shfl_xor_sync(0xffffffffu, e1, o));
+        nz0 |= __shfl_xor_sync(0xffffffffu, nz0, o);
+        nz1 |= __shfl_xor_sync(0xffffffffu, nz1, o);
+    }
+    if (e0 < kLegExpLo || e0 > kLegExpHi) e0 = nz0 ? -1 : 0;
+    if (e1 < kLegExpLo || e1 > kLegExpHi) e1 = nz1 ? -1 : 0;
+    return make_int2(e0, e1);
+}
+
+// ... and entries [0, count) of them (at most 32) as limbs of 55 bits in lim
+template <int NB>
+__device__ __forceinline__ void chain_limbs(const double *src, size_t stride, int count, int2 e, int2 *lim, int lane)
+{
+    constexpr int STEP = 32 / NB;
+    const int b = lane % NB, r = lane / NB;
+    int4 *lim4 = reinterpret_cast<int4 *>(lim);
+#pragma unroll 2
+    for (int i = r; i < count; i += STEP) {
+        const double2 x = __ldg(reinterpret_cast<const double2 *>(src + (size_t)i * stride) + b);
+        const int2 l0 = e.x > 0 ? shtb_dev::to_limbs(x.x, 9 + e.x - shtb_dev::exp_bits(x.x)) : make_int2(0, 0);
+        const int2 l1 = e.y > 0 ? shtb_dev::to_limbs(x.y, 9 + e.y - shtb_dev::exp_bits(x.y)) : make_int2(0, 0);
+        lim4[i * NB + b] = make_int4(l0.x, l0.y, l1.x, l1.y);
+    }
+}
+
+// A warp's 32 running sums (one a lane) per component, on a common exponent E
+// of the V seen so far (0: none yet) with up to kHead bits to spare, so that a
+// growing V raises it only now and then: value (H 2^68 + P 2^28 + M) 2^28 2^(e_a + E - ..)
+constexpr int kHead = 3;
+// chain steps between two looks at E (one for every map count: the same bits)
+constexpr int kStep = 4;
+
+template <int C>
+struct LegSums {
+    long long P[C], M[C];
+    int H[C];
+    int E, vb, base;                     // exponent of V, bits of V, limb shift at exponent 0
+    __device__ __forceinline__ void clear(int n)
+    {
+        E = 0;
+        vb = v_bits(n);
+        base = 4096;                     // every V (a zero) shifted out
+#pragma unroll
+        for (int c = 0; c < C; ++c) P[c] = M[c] = H[c] = 0;
+    }
+    // before adding V of exponents up to e
+    __device__ __forceinline__ void raise(int e)
+    {
+        if (!__any_sync(0xffffffffu, e > E)) return;
+        int s = e > E ? e + kHead - E : 0;
+        if (s > 0) {
+            if (E == 0) s = 0;           // nothing summed yet
+            E = e + kHead;
+            base = 64 - vb + E;
+        }
+#pragma unroll 1
+        while (__any_sync(0xffffffffu, s > 0)) {
+            const int k = min(s, 20);
+            const unsigned mask = (1u << k) - 1;
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                M[c] = (M[c] + ((long long)((unsigned)P[c] & mask) << 28)) >> k;
+                P[c] = (P[c] + ((long long)((unsigned)H[c] & mask) << 40)) >> k;
+                H[c] >>= k;
+            }
+            s -= k;
+        }
+    }
+    __device__ __forceinline__ void add(double v, const int2 *lim)
+    {
+        const int2 w = shtb_dev::to_limbs(v, base - shtb_dev::exp_bits(v));
+#pragma unroll
+        for (int c = 0; c < C; c += 2) {
+            const int4 a = *reinterpret_cast<const int4 *>(lim + c);
+            P[c] = shtb_dev::mad_wide(a.y, w.y, P[c]);
+            M[c] = shtb_dev::mad_wide(a.y, w.x, M[c]);
+            M[c] = shtb_dev::mad_wide(a.x, w.y, M[c]);
+            P[c + 1] = shtb_dev::mad_wide(a.w, w.y, P[c + 1]);
+            M[c + 1] = shtb_dev::mad_wide(a.w, w.x, M[c + 1]);
+            M[c + 1] = shtb_dev::mad_wide(a.z, w.y, M[c + 1]);
+        }
+    }
+    // every 32 products, so that none overflows
+    __device__ __forceinline__ void carry()
+    {
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            P[c] += M[c] >> 28;
+            M[c] &= (1LL << 28) - 1;
+            H[c] += (int)(P[c] >> 40);
+            P[c] &= (1LL << 40) - 1;
+        }
+    }
+    // after a carry; a = X_a 2^(e_a - 1077), V = X_V 2^(E - 1022 - vb)
+    __device__ __forceinline__ double value(int c, int ea) const
+    {
+        const long long p = (long long)H[c] << 30 | P[c] >> 10, l = ((long long)P[c] & 1023) << 18 | M[c] >> 10;
+        return ea > 0 && E > 0 ? shtb_dev::limbs_to_double(p, l, 10 + 28 + 1054 + ea - 1077 + 28 + E - 1022 - vb) : 0.0;
+    }
+};
+
+// One ring's chain of one parity, advanced step by step: value V_j at `cur`
+struct Chain {
+    double x, cur, prev;
+    double2 start;
+    int js;
+    bool sform;
+    __device__ __forceinline__ void begin(int j)
+    {
+        cur = js == j ? start.x : 0.0;
+        prev = 0.0;
+    }
+    __device__ __forceinline__ void step(int j, const RecCoef &c)
+    {
+        const double w = fma(c.mu, x, sform ? c.cs : c.cz);
+        double nxt = fma(w, cur, -prev);
+        if (j == js) nxt = start.y;
+        if (j + 1 == js) nxt = start.x;
+        prev = cur;
+        cur = nxt;
+    }
+};
+
+// The sum of one component by FP64 FMAs along the recurrence, for chains
+// whose a hold an infinity, a NaN or extreme magnitudes
+__device__ __noinline__ double plain_chain_sum(const RecCoef *cf, const double *a, size_t stride, int jlo, int n,
+                                               Chain ch)
+{
+    double s = 0.0;
+    ch.begin(jlo);
+    for (int j = jlo; j < n; ++j) {
+        s = fma(a[(size_t)j * stride], ch.cur, s);
+        ch.step(j, cf[2 * j]);
+    }
+    return s;
+}
+
+// One warp per (m, 32 half-rings, parity); the two parities of a (m, rings)
+// are neighbouring warps and trade their sums through shared memory.  With 8
+// maps 3 CTAs an SM spare the spills of 4 (.711 against .744 ms, nside 256).
+template <int NB>
+__global__ void __launch_bounds__(32 * kWarpsPerBlock, NB == 8 ? 3 : 4)
 legendre_synth_kernel(PlanView v, const double2 *__restrict__ ap, double2 *__restrict__ q,
                       int nmaps, int b0)
 {
+    constexpr int C = 2 * NB;
+    __shared__ __align__(16) int2 slim[kWarpsPerBlock][32 * C];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int Z = v.nhalf, L = v.lmax;
     const int nchunk = (Z + 31) >> 5;
-    const long long item = (long long)blockIdx.x * kWarpsPerBlock + warp;
-    if (item >= (long long)(L + 1) * nchunk) return;
-    const int m = (int)(item / nchunk);
-    const int chunk = (int)(item - (long long)m * nchunk);
+    const long long item = ((long long)blockIdx.x * kWarpsPerBlock + warp) >> 1;
+    const int t = warp & 1;
+    const bool there = item < (long long)(L + 1) * nchunk;
+    const int m = there ? (int)(item / nchunk) : 0;
+    const int chunk = there ? (int)(item - (long long)m * nchunk) : 0;
     const int r = chunk * 32 + lane;
-    const bool valid = r < Z;
+    const bool valid = there && r < Z;
     const int rr = valid ? r : Z - 1;
-    const int n0 = dchain_len(L, m, 0), n1 = dchain_len(L, m, 1);
+    const int n = there ? dchain_len(L, m, t) : 0;
+    int2 *lim = slim[warp];
 
-    const double x = v.xarg[rr];
-    const bool sform = v.xform[rr] != 0;
-    const size_t base0 = ((size_t)m * 2) * Z + rr, base1 = base0 + Z;
-    const int js0 = valid ? v.jstart[base0] : n0;
-    const int js1 = valid ? v.jstart[base1] : n1;
-    const double2 s0 = v.vstart[base0], s1 = v.vstart[base1];
-
-    int lo = n0;
-    if (js0 < n0) lo = js0;
-    if (js1 < n1) lo = min(lo, js1);
-    const int jlo = warp_min(lo);
-    if (jlo >= n0) {
-        // nothing above the crop for any lane: q is zero for these rings
-        if (valid) {
-            for (int b = 0; b < NB; ++b) {
-                double2 *qb = q + (size_t)(b0 + b) * v.nrings * (L + 1);
-                qb[(size_t)r * (L + 1) + m] = make_double2(0.0, 0.0);
-                if (r < Z - 1) qb[(size_t)(v.nrings - 1 - r) * (L + 1) + m] = make_double2(0.0, 0.0);
+    double acc[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) acc[c] = 0.0;
+    Chain ch;
+    ch.x = v.xarg[rr];
+    ch.sform = v.xform[rr] != 0;
+    const size_t base = ((size_t)m * 2 + t) * Z + rr;
+    ch.js = valid ? v.jstart[base] : n;
+    ch.start = v.vstart[base];
+    const int jlo = warp_min(ch.js < n ? ch.js : n);
+    if (jlo < n) {
+        const long long off = dalm_index(L, m, m) + t;
+        const RecCoef *__restrict__ cf = v.coef + off;                // step j at cf[2 j]
+        const double *a = reinterpret_cast<const double *>(ap + (size_t)off * nmaps + b0);
+        const size_t stride = (size_t)4 * nmaps;                      // doubles between chain entries
+        const int2 ea = scan_chain<NB>(a + (size_t)jlo * stride, stride, n - jlo, lane);
+        LegSums<C> sums;
+        sums.clear(n);
+        ch.begin(jlo);
+        for (int jb = jlo; jb < n; jb += 32) {
+            const int nj = min(32, n - jb);
+            __syncwarp();
+            chain_limbs<NB>(a + (size_t)jb * stride, stride, nj, ea, lim, lane);
+            __syncwarp();
+            for (int i0 = 0; i0 < nj; i0 += kStep) {
+                double V[kStep];
+                int e = 0;
+#pragma unroll
+                for (int i = 0; i < kStep; ++i) {
+                    V[i] = 0.0;
+                    if (i0 + i < nj) {
+                        V[i] = ch.cur;
+                        e = max(e, shtb_dev::exp_bits(ch.cur));
+                        ch.step(jb + i0 + i, cf[2 * (jb + i0 + i)]);
+                    }
+                }
+                sums.raise(e);
+#pragma unroll
+                for (int i = 0; i < kStep; ++i)
+                    if (i0 + i < nj) sums.add(V[i], lim + (i0 + i) * C);
             }
+            sums.carry();
         }
-        return;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const int e = __shfl_sync(0xffffffffu, c & 1 ? ea.y : ea.x, c >> 1);
+            acc[c] = sums.value(c, e);
+            if (e < 0) acc[c] = plain_chain_sum(cf, a + c, stride, jlo, n, ch);
+        }
     }
 
-    double2 acc0[NB], acc1[NB];
+    // q(+z) = q^0 + q^1 by the even warp, q(-z) = q^0 - q^1 by the odd one
+    __syncthreads();
+    double *trade = reinterpret_cast<double *>(lim);                   // [C][32]
+#pragma unroll
+    for (int c = 0; c < C; ++c) trade[c * 32 + lane] = acc[c];
+    __syncthreads();
+    if (!valid || (t == 1 && r == Z - 1)) return;                      // the equator ring has no mirror
+    const double *other = reinterpret_cast<const double *>(slim[warp ^ 1]);
+    const int ring = t == 0 ? r : v.nrings - 1 - r;
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
-        acc0[b] = make_double2(0.0, 0.0);
-        acc1[b] = make_double2(0.0, 0.0);
-    }
-    double cur0 = (js0 == jlo) ? s0.x : 0.0, prev0 = 0.0;
-    double cur1 = (js1 == jlo) ? s1.x : 0.0, prev1 = 0.0;
-
-    const long long off = dalm_index(L, m, m);
-    const RecCoef *__restrict__ cf = v.coef + off;
-    const double2 *__restrict__ a = ap + (size_t)off * nmaps + b0;
-
-    for (int j = jlo; j < n0; ++j) {
-        // ---- even chain, l = m + 2j
-        {
-            const int dl = 2 * j;
-            const double2 *aj = a + (size_t)dl * nmaps;
-#pragma unroll
-            for (int b = 0; b < NB; ++b) {
-                const double2 av = __ldg(aj + b);
-                acc0[b].x = fma(av.x, cur0, acc0[b].x);
-                acc0[b].y = fma(av.y, cur0, acc0[b].y);
-            }
-            const RecCoef c = cf[dl];
-            const double w = fma(c.mu, x, sform ? c.cs : c.cz);
-            double nxt = fma(w, cur0, -prev0);
-            if (j == js0) nxt = s0.y;
-            if (j + 1 == js0) nxt = s0.x;
-            prev0 = cur0;
-            cur0 = nxt;
-        }
-        // ---- odd chain, l = m + 1 + 2j
-        if (j < n1) {
-            const int dl = 2 * j + 1;
-            const double2 *aj = a + (size_t)dl * nmaps;
-#pragma unroll
-            for (int b = 0; b < NB; ++b) {
-                const double2 av = __ldg(aj + b);
-                acc1[b].x = fma(av.x, cur1, acc1[b].x);
-                acc1[b].y = fma(av.y, cur1, acc1[b].y);
-            }
-            const RecCoef c = cf[dl];
-            const double w = fma(c.mu, x, sform ? c.cs : c.cz);
-            double nxt = fma(w, cur1, -prev1);
-            if (j == js1) nxt = s1.y;
-            if (j + 1 == js1) nxt = s1.x;
-            prev1 = cur1;
-            cur1 = nxt;
-        }
-    }
-
-    if (!valid) return;
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        double2 *qb = q + (size_t)(b0 + b) * v.nrings * (L + 1);
-        qb[(size_t)r * (L + 1) + m] = make_double2(acc0[b].x + acc1[b].x, acc0[b].y + acc1[b].y);
-        if (r < Z - 1)   // the equator ring (r = Z-1) has no mirror
-            qb[(size_t)(v.nrings - 1 - r) * (L + 1) + m] =
-                make_double2(acc0[b].x - acc1[b].x, acc0[b].y - acc1[b].y);
+        const double ox = other[2 * b * 32 + lane], oy = other[(2 * b + 1) * 32 + lane];
+        q[((size_t)(b0 + b) * v.nrings + ring) * (L + 1) + m] =
+            t == 0 ? make_double2(acc[2 * b] + ox, acc[2 * b + 1] + oy)
+                   : make_double2(ox - acc[2 * b], oy - acc[2 * b + 1]);
     }
 }
 
@@ -202,147 +381,143 @@ __global__ void __launch_bounds__(256) adjoint_parity_kernel(PlanView v, const d
     }
 }
 
-constexpr int kAdjWarps = 4;
+// Warps of a CTA: an order's chains are as long as its tiles are many, and
+// orders are too few to fill the chip by themselves.  4, 8, 16 warps: .786,
+// .542, .682 ms at nside 256 with 4 maps, 1.31, .89, 1.06 with 8, .51, .35, .38 with 1.
+constexpr int kAdjWarps = 8;
 constexpr int kTilePad = 33;   // row stride (doubles) of the 32x32 tile: no bank conflicts
 
+// per warp: the tile of V and the limbs of 32 rings' g (the sums' trade later)
 template <int NB>
 __host__ __device__ constexpr size_t adjoint_warp_smem_doubles()
 {
-    return 2 * 32 * kTilePad + 2 * 32 * NB * 2;
+    return 32 * kTilePad + 32 * 2 * NB;
 }
 
+// One component's a_j = sum_r V_j(r) g_r of a chain in FP64, by one warp
+// (lane = ring), for chains whose g hold an infinity, a NaN or extreme
+// magnitudes.  dst: the component in aacc, entry j at dst + j dstride.
+__device__ __noinline__ void plain_chain_adjoint(const PlanView &v, int m, int t, const double *gc, size_t gstride,
+                                                 double *dst, size_t dstride, int lane)
+{
+    const int Z = v.nhalf, n = dchain_len(v.lmax, m, t);
+    const RecCoef *cf = v.coef + dalm_index(v.lmax, m, m) + t;
+    for (int c0 = 0; c0 < Z; c0 += 32) {
+        const int r = c0 + lane, rr = min(r, Z - 1);
+        const size_t base = ((size_t)m * 2 + t) * Z + rr;
+        Chain ch;
+        ch.x = v.xarg[rr];
+        ch.sform = v.xform[rr] != 0;
+        ch.js = r < Z ? v.jstart[base] : n;
+        ch.start = v.vstart[base];
+        const double gv = r < Z ? gc[(size_t)rr * gstride] : 0.0;
+        ch.begin(0);
+        for (int j = 0; j < n; ++j) {
+            double s = r < Z && j >= ch.js ? ch.cur * gv : 0.0;
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) dst[(size_t)j * dstride] = c0 ? dst[(size_t)j * dstride] + s : s;
+            ch.step(j, cf[2 * j]);
+        }
+    }
+}
+
+// One CTA per m: the even warps take the even chain, the odd ones the odd
+// chain, each its share of the chunks of 32 rings.
 template <int NB>
-__global__ void __launch_bounds__(32 * kAdjWarps)
+__global__ void __launch_bounds__(32 * kAdjWarps, 16 / kAdjWarps)
 legendre_adjoint_kernel(PlanView v, const double2 *__restrict__ g, double2 *__restrict__ aacc,
                         RecState *__restrict__ state, int nmaps, int b0)
 {
-    extern __shared__ double smd[];
+    constexpr int C = 2 * NB;
+    extern __shared__ __align__(16) double smd[];
     const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
+    const int warp = threadIdx.x >> 5, t = warp & 1, set = warp >> 1;
     const int Z = v.nhalf, L = v.lmax;
     const int m = blockIdx.x;
-    const int n0 = dchain_len(L, m, 0), n1 = dchain_len(L, m, 1);
+    const int n = dchain_len(L, m, t), n0 = dchain_len(L, m, 0);
     const int nchunk = (Z + 31) >> 5;
     const long long off = dalm_index(L, m, m);
-    const RecCoef *__restrict__ cf = v.coef + off;
-    double *tile = smd + (size_t)warp * adjoint_warp_smem_doubles<NB>();   // [2][32][kTilePad]
-    double2 *gs = reinterpret_cast<double2 *>(tile + 2 * 32 * kTilePad);    // [2][32][NB]
-    RecState *st = state + (size_t)blockIdx.x * Z;
+    const RecCoef *__restrict__ cf = v.coef + off + t;                // step j at cf[2 j]
+    double *tile = smd + (size_t)warp * adjoint_warp_smem_doubles<NB>();   // [32][kTilePad]
+    int2 *lim = reinterpret_cast<int2 *>(tile + 32 * kTilePad);            // [32][C]
+    double2 *st = reinterpret_cast<double2 *>(state + (size_t)blockIdx.x * Z) + t;   // ring r at st[2 r]
+    const double *gm = reinterpret_cast<const double *>(g + ((size_t)m * 2 + t) * Z * nmaps + b0);
+    const size_t gstride = (size_t)2 * nmaps;                         // doubles between rings
+    const int2 eg = scan_chain<NB>(gm, gstride, Z, lane);
     const int ntiles = (n0 + 31) >> 5;
 
     for (int ti = 0; ti < ntiles; ++ti) {
         const int jt = ti * 32;
-        double2 acc0[NB], acc1[NB];
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            acc0[b] = make_double2(0.0, 0.0);
-            acc1[b] = make_double2(0.0, 0.0);
-        }
-        for (int c = warp; c < nchunk; c += kAdjWarps) {
+        LegSums<C> sums;
+        sums.clear(Z);
+        for (int c = set; c < nchunk && jt < n; c += kAdjWarps / 2) {
             const int r = c * 32 + lane;
             const bool valid = r < Z;
             const int rr = valid ? r : Z - 1;
-            const size_t base0 = ((size_t)m * 2) * Z + rr, base1 = base0 + Z;
-            const int js0 = valid ? v.jstart[base0] : n0;
-            const int js1 = valid ? v.jstart[base1] : n1;
-            int lo = n0;
-            if (js0 < n0) lo = js0;
-            if (js1 < n1) lo = min(lo, js1);
-            const int clo = warp_min(lo);
-            if (clo >= n0 || jt + 32 <= clo) continue;   // chunk is zero in this tile
-            const double2 s0 = v.vstart[base0], s1 = v.vstart[base1];
-            const double x = v.xarg[rr];
-            const bool sform = v.xform[rr] != 0;
-            double cur0, prev0, cur1, prev1;
-            if (ti == (clo >> 5)) {
-                cur0 = (js0 == jt) ? s0.x : 0.0;
-                cur1 = (js1 == jt) ? s1.x : 0.0;
-                prev0 = prev1 = 0.0;
-            } else {
-                const RecState sv = st[rr];
-                cur0 = sv.cur0; prev0 = sv.prev0; cur1 = sv.cur1; prev1 = sv.prev1;
+            const size_t base = ((size_t)m * 2 + t) * Z + rr;
+            Chain ch;
+            ch.js = valid ? v.jstart[base] : n;
+            const int clo = warp_min(ch.js < n ? ch.js : n);
+            if (clo >= n || jt + 32 <= clo) continue;   // chunk is zero in this tile
+            ch.start = v.vstart[base];
+            ch.x = v.xarg[rr];
+            ch.sform = v.xform[rr] != 0;
+            ch.begin(jt);
+            if (ti != (clo >> 5) && valid) {       // lanes past the last ring keep V = 0
+                const double2 sv = st[2 * rr];
+                ch.cur = sv.x;
+                ch.prev = sv.y;
             }
-            // phase 1: lane = ring; V_j for the tile's 32 chain steps
+            // lane = ring: V_j for the tile's 32 chain steps
             for (int jj = 0; jj < 32; ++jj) {
                 const int j = jt + jj;
-                double e0 = 0.0, e1 = 0.0;
-                if (j < n0) {
-                    e0 = cur0;
-                    const RecCoef cc = cf[2 * j];
-                    const double w = fma(cc.mu, x, sform ? cc.cs : cc.cz);
-                    double nxt = fma(w, cur0, -prev0);
-                    if (j == js0) nxt = s0.y;
-                    if (j + 1 == js0) nxt = s0.x;
-                    prev0 = cur0;
-                    cur0 = nxt;
-                }
-                if (j < n1) {
-                    e1 = cur1;
-                    const RecCoef cc = cf[2 * j + 1];
-                    const double w = fma(cc.mu, x, sform ? cc.cs : cc.cz);
-                    double nxt = fma(w, cur1, -prev1);
-                    if (j == js1) nxt = s1.y;
-                    if (j + 1 == js1) nxt = s1.x;
-                    prev1 = cur1;
-                    cur1 = nxt;
-                }
-                tile[jj * kTilePad + lane] = e0;
-                tile[(32 + jj) * kTilePad + lane] = e1;
+                tile[jj * kTilePad + lane] = j < n ? ch.cur : 0.0;
+                if (j < n) ch.step(j, cf[2 * j]);
             }
-            if (valid) {
-                RecState sv;
-                sv.cur0 = cur0; sv.prev0 = prev0; sv.cur1 = cur1; sv.prev1 = prev1;
-                st[r] = sv;
-            }
-            for (int i = lane; i < 2 * 32 * NB; i += 32) {
-                const int t = i / (32 * NB), rem = i - t * 32 * NB;
-                const int r2 = rem / NB, b = rem - r2 * NB;
-                const int ring = c * 32 + r2;
-                gs[i] = ring < Z ? g[(((size_t)m * 2 + t) * Z + ring) * nmaps + b0 + b]
-                                 : make_double2(0.0, 0.0);
-            }
+            if (valid) st[2 * r] = make_double2(ch.cur, ch.prev);
+            chain_limbs<NB>(gm + (size_t)c * 32 * gstride, gstride, min(32, Z - c * 32), eg, lim, lane);
             __syncwarp();
-            // phase 2: lane = chain step jj, sum over the tile's 32 rings
-            const double *row0 = tile + lane * kTilePad;
-            const double *row1 = tile + (32 + lane) * kTilePad;
-            for (int r2 = 0; r2 < 32; ++r2) {
-                const double V0 = row0[r2], V1 = row1[r2];
-                const double2 *g0 = gs + r2 * NB, *g1 = gs + (32 + r2) * NB;
-#pragma unroll
-                for (int b = 0; b < NB; ++b) {
-                    const double2 ga = g0[b], gb = g1[b];
-                    acc0[b].x = fma(V0, ga.x, acc0[b].x);
-                    acc0[b].y = fma(V0, ga.y, acc0[b].y);
-                    acc1[b].x = fma(V1, gb.x, acc1[b].x);
-                    acc1[b].y = fma(V1, gb.y, acc1[b].y);
-                }
-            }
+            // lane = chain step: sum over the tile's 32 rings (those past the last have V = 0)
+            const double *row = tile + lane * kTilePad;
+            int e = 0;
+#pragma unroll 8
+            for (int r2 = 0; r2 < 32; ++r2) e = max(e, shtb_dev::exp_bits(row[r2]));
+            sums.raise(e);
+#pragma unroll 4
+            for (int r2 = 0; r2 < 32; ++r2) sums.add(row[r2], lim + r2 * C);
+            sums.carry();
             __syncwarp();
         }
-        // add the warps' partial sums for this tile and store them
-        __syncthreads();
-        double2 *red = reinterpret_cast<double2 *>(smd);   // [warp][t][jj][b]
+        // add the warps' partial sums of each parity and store them
+        double *mine = tile;                            // [C][32], rows of 33
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            red[((warp * 2 + 0) * 32 + lane) * NB + b] = acc0[b];
-            red[((warp * 2 + 1) * 32 + lane) * NB + b] = acc1[b];
+        for (int c = 0; c < C; ++c) {
+            const int e = __shfl_sync(0xffffffffu, c & 1 ? eg.y : eg.x, c >> 1);
+            mine[c * kTilePad + lane] = sums.value(c, e);
         }
         __syncthreads();
         for (int i = threadIdx.x; i < 2 * 32 * NB; i += blockDim.x) {
-            const int t = i / (32 * NB), rem = i - t * 32 * NB;
+            const int tt = i / (32 * NB), rem = i - tt * 32 * NB;
             const int jj = rem / NB, b = rem - jj * NB;
             const int j = jt + jj;
-            if (j >= (t == 0 ? n0 : n1)) continue;
+            if (j >= (tt == 0 ? n0 : dchain_len(L, m, 1))) continue;
             double2 sum = make_double2(0.0, 0.0);
-            for (int w = 0; w < kAdjWarps; ++w) {
-                const double2 pv = red[((w * 2 + t) * 32 + jj) * NB + b];
-                sum.x += pv.x;
-                sum.y += pv.y;
+#pragma unroll
+            for (int w = tt; w < kAdjWarps; w += 2) {
+                const double *p = smd + (size_t)w * adjoint_warp_smem_doubles<NB>() + 2 * b * kTilePad + jj;
+                sum.x += p[0];
+                sum.y += p[kTilePad];
             }
-            aacc[(size_t)(off + t + 2 * j) * nmaps + b0 + b] = sum;
+            aacc[(size_t)(off + tt + 2 * j) * nmaps + b0 + b] = sum;
         }
         __syncthreads();
     }
+    if (set == 0 && n > 0)
+        for (int c = 0; c < C; ++c)
+            if (__shfl_sync(0xffffffffu, c & 1 ? eg.y : eg.x, c >> 1) < 0)
+                plain_chain_adjoint(v, m, t, gm + c, gstride,
+                                    reinterpret_cast<double *>(aacc + (size_t)(off + t) * nmaps + b0) + c,
+                                    (size_t)4 * nmaps, lane);
 }
 
 // alm[b][idx] = c_m sigma_idx aacc[idx][b], c_0 = 1 (Im a_l0 = 0), c_m = 2
@@ -392,7 +567,7 @@ int launch_legendre_synth(const shtb_plan_s *p, const double2 *ap, double2 *q, i
                           cudaStream_t st)
 {
     const int nchunk = (p->nhalf + 31) / 32;
-    const long long items = (long long)(p->lmax + 1) * nchunk;
+    const long long items = (long long)(p->lmax + 1) * nchunk * 2;     // warps: both parities
     const unsigned grid = (unsigned)((items + kWarpsPerBlock - 1) / kWarpsPerBlock);
     const dim3 block(32 * kWarpsPerBlock);
     for (int b0 = 0; b0 < nmaps;) {
