@@ -497,7 +497,7 @@ int run_synthesis_spin(shtb_plan_s *p, const double2 *alm, double *map, int npai
     int rc;
     if ((rc = ensure_ws(p, nm)) || (rc = ensure_ws(q, nm))) return rc;
     Workspace wp = carve(p, nm), wq = carve(q, nm);
-    double *qt_plus = (double *)wp.adj, *qt_minus = (double *)wq.adj;   // parity halves, map-major
+    double *qt_plus = (double *)wp.adj, *qt_minus = (double *)wq.adj;   // parity halves, in packs of two
     if ((rc = launch_bf_synth(p, alm, wp.ap, wp.bf, nullptr, nm, st, qt_plus))) return rc;
     if ((rc = launch_bf_synth(q, alm, wq.ap, wq.bf, nullptr, nm, st, qt_minus))) return rc;
     if ((rc = launch_spin_combine(p, qt_plus, qt_minus, wp.q, npairs, st))) return rc;

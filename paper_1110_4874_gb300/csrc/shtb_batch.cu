@@ -54,7 +54,8 @@ struct BatchPack {
 };
 
 struct BatchMG {                      // one map group of one plan group
-    double *u0, *u1, *qt;
+    double *u0, *u1;
+    QtView qt;
     int b0, nb;
 };
 
@@ -123,17 +124,17 @@ __device__ void ring_item(const BatchDev &bd, const BatchWork &w, shtb_dev::fx2 
 {
     const BatchGroupDev &G = bd.groups[w.g];
     const BatchMG &M = bd.mgs[w.mg];
-    const double2 *qt = reinterpret_cast<const double2 *>(M.qt);
+    const double2 *qt = reinterpret_cast<const double2 *>(M.qt.q);
     double *out = G.map_of_map[M.b0 + w.aux] + G.v.ring_start[w.idx];
     switch (w.kind) {
     case shtb_dev::kBluestein:
-        shtb_dev::phi_synth_ring_qt<shtb_dev::kBluestein, true>(G.v, w.idx, qt, w.aux, out, sm);
+        shtb_dev::phi_synth_ring_qt<shtb_dev::kBluestein, true>(G.v, w.idx, qt, M.qt.lp, w.aux, out, sm);
         break;
     case shtb_dev::kDirectBig:
-        shtb_dev::phi_synth_ring_qt<shtb_dev::kDirectBig, true>(G.v, w.idx, qt, w.aux, out, sm);
+        shtb_dev::phi_synth_ring_qt<shtb_dev::kDirectBig, true>(G.v, w.idx, qt, M.qt.lp, w.aux, out, sm);
         break;
     default:
-        shtb_dev::phi_synth_ring_qt<shtb_dev::kDirect, true>(G.v, w.idx, qt, w.aux, out, sm);
+        shtb_dev::phi_synth_ring_qt<shtb_dev::kDirect, true>(G.v, w.idx, qt, M.qt.lp, w.aux, out, sm);
         break;
     }
 }
@@ -220,7 +221,8 @@ struct shtb_batch_s {
     int nstreams = 1;
     struct GMapGroup {
         int b0, nb, real, stream;     // columns of the group, and its maps
-        double *u0, *u1, *qt;
+        double *u0, *u1;
+        QtView qt;
         double cost;
     };
     struct GPlanGroup {
@@ -386,7 +388,7 @@ int build_schedule(shtb_batch_s *b, int warps, int width, int lpt)
             if ((rc = balloc(b->sched_allocs, &d, entry * (size_t)bf.u_entries))) return rc;
             M.u1 = (double *)d;
             if ((rc = balloc(b->sched_allocs, &d, entry * (size_t)bf.qt_entries))) return rc;
-            M.qt = (double *)d;
+            M.qt = QtView{(double *)d, qt_pack(nb)};
             const int mg = (int)mgs.size();
             mgs.push_back(M);
             // each stage waits for the last non-empty stage before it
@@ -536,7 +538,7 @@ int build_graph_schedule(shtb_batch_s *b, int width, int nstreams)
             if ((rc = balloc(b->sched_allocs, &d, entry * (size_t)bf.u_entries))) return rc;
             M.u1 = (double *)d;
             if ((rc = balloc(b->sched_allocs, &d, entry * (size_t)bf.qt_entries))) return rc;
-            M.qt = (double *)d;
+            M.qt = QtView{(double *)d, qt_pack(nb)};
             order.push_back({M.cost, {(int)g, (int)P.mgs.size()}});
             P.mgs.push_back(M);
             b0 += nb;

@@ -17,23 +17,16 @@ __device__ __forceinline__ long long alm_off(int L, int m)
     return (long long)m * (2 * L + 1 - m) / 2 + m;
 }
 
-// q^t of a map group is stored map-major as complex values:
-// qt[((b * 2 + t) * nhalf + r) * (L + 1) + m], so the ring stage reads each
-// map's q_m of one ring contiguously in m.  Leaf outputs are addressed by the
-// entry e = (m * 2 + t) * nhalf + r; this writes the C = 2 NB components of e.
+// q^t of a map group (QtView): the ring stage reads each map's q_m of one
+// ring along m, the items write all maps of one entry e = (m * 2 + t) * nhalf + r.
 // Entries fit 32 bits (e < 2 (L + 1) nhalf), so the split of e runs as a
 // 32-bit division.
-__device__ __forceinline__ size_t qt_index(int e, int nhalf, int L, int c)
+__device__ __forceinline__ size_t qt_index(int e, int nhalf, int L, int lp, int c)
 {
     const unsigned mt = (unsigned)e / (unsigned)nhalf, r = (unsigned)e - mt * (unsigned)nhalf;
     const unsigned m = mt >> 1, t = mt & 1;
-    const unsigned b = (unsigned)c >> 1;
-    return ((((size_t)b * 2 + t) * nhalf + r) * (L + 1) + m) * 2 + (c & 1);
-}
-
-__device__ __forceinline__ void qt_store(double *qt, int e, int nhalf, int L, int c, double v)
-{
-    qt[qt_index(e, nhalf, L, c)] = v;
+    const unsigned b = (unsigned)c >> 1, pack = b >> lp;
+    return ((((((size_t)pack * 2 + t) * nhalf + r) * (L + 1) + m) << lp) + (b - (pack << lp))) * 2 + (c & 1);
 }
 
 // Every output of a residual block (one column) and of a level child (one
@@ -60,14 +53,14 @@ template <int C>
 struct ResOut {
     double *dst;                        // u entries of the block, or null: q^t entries ent
     const int *ent;
-    double *qt;
+    QtView qt;
     int nhalf, L;
     __device__ __forceinline__ int key(int n) const { return dst ? n : __ldg(ent + n); }
     template <int W>
     __device__ __forceinline__ void put(int n, bool add, int i, const double (&v)[W]) const
     {
         if (dst) st_comps(dst + (size_t)n * C, i, v, add);
-        else st_comps(qt + qt_index(n, nhalf, L, W * i), 0, v, add);
+        else st_comps(qt.q + qt_index(n, nhalf, L, qt.lp, W * i), 0, v, add);
     }
 };
 
@@ -76,7 +69,7 @@ struct ResOut {
 template <int NB, bool CG>
 __device__ __forceinline__ void bf_r_item(const BfRItem &it, int L, int nhalf, const int *__restrict__ ints,
                                           const uint2 *__restrict__ words, const double2 *ai, int nmaps,
-                                          int b0, double *ubuf, double *qt, int lane)
+                                          int b0, double *ubuf, QtView qt, int lane)
 {
     constexpr int C = 2 * NB;
     const long long aoff = alm_off(L, it.m) + it.t + 2 * it.j0;       // chain row j at aoff + 2j
@@ -134,7 +127,7 @@ struct LevelOut {
 template <int NB, bool CG, int RING = -1>
 __device__ __forceinline__ void bf_level_item(const BfItem &it, int L, int nhalf, const int *__restrict__ ints,
                                               const uint2 *__restrict__ words, const double *uin,
-                                              double *uout, double *qt, double *scr, int lane)
+                                              double *uout, QtView qt, double *scr, int lane)
 {
     constexpr int C = 2 * NB;
     double2 *scr2 = reinterpret_cast<double2 *>(scr);
@@ -148,12 +141,14 @@ __device__ __forceinline__ void bf_level_item(const BfItem &it, int L, int nhalf
         __syncwarp();
     }
     if (RING == 1 || (RING < 0 && it.to_rings)) {
+        // the entries of an item share (m, t); those of a lane share the map
         const int *__restrict__ ent = ints + it.out_off;
+        const int e0 = __ldg(ent);
+        double2 *q0 = reinterpret_cast<double2 *>(qt.q + qt_index(e0, nhalf, L, qt.lp, 2 * (lane % NB)));
+        const size_t ring = (size_t)(L + 1) << qt.lp;
 #pragma unroll 4
-        for (int i = lane; i < it.nc * NB; i += 32) {
-            const int cpos = i / NB, b = i - cpos * NB;
-            *reinterpret_cast<double2 *>(qt + qt_index(__ldg(ent + cpos), nhalf, L, 2 * b)) = scr2[i];
-        }
+        for (int i = lane / NB; i < it.nc; i += 32 / NB)
+            q0[(__ldg(ent + i) - e0) * (long long)ring] = scr2[i * NB + lane % NB];
     } else {
         double2 *dst = reinterpret_cast<double2 *>(uout + (size_t)it.out_off * C);
         for (int i = lane; i < it.nc * NB; i += 32) dst[i] = scr2[i];

@@ -19,7 +19,7 @@ namespace shtb_dev {
 template <int NB, bool CG>
 __device__ __forceinline__ void bf_r_rec_item(const BfRItem &it, const PlanView &v,
                                               const RecStart *__restrict__ rs, const int *__restrict__ ints,
-                                              const double2 *ai, int nmaps, int b0, double *ubuf, double *qt,
+                                              const double2 *ai, int nmaps, int b0, double *ubuf, QtView qt,
                                               int lane)
 {
     constexpr int C = 2 * NB, CPL = C < 8 ? C : 8, S = C / CPL, CPP = 32 / S;
@@ -61,7 +61,7 @@ __device__ __forceinline__ void bf_r_rec_item(const BfRItem &it, const PlanView 
         if (it.to_rings) {
             const int e = ints[it.out_off + s];
 #pragma unroll
-            for (int c = 0; c < CPL; ++c) qt_store(qt, e, nhalf, L, c0 + c, acc[c]);
+            for (int c = 0; c < CPL; ++c) qt.q[qt_index(e, nhalf, L, qt.lp, c0 + c)] = acc[c];
         } else {
             double *dst = ubuf + (size_t)(it.out_off + s) * C + c0;
 #pragma unroll

@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(32 * kBfWarps, 4)
 bf_r_kernel(PlanView v, const BfRItem *__restrict__ items, int nitems, const int *__restrict__ ints,
             const uint2 *__restrict__ words, const double2 *__restrict__ ai, int nmaps, int b0,
             double *__restrict__ ubuf0, double *__restrict__ ubuf1, const int *__restrict__ depth_par,
-            double *__restrict__ qt)
+            QtView qt)
 {
     const int lane = threadIdx.x & 31;
     const int w = blockIdx.x * kBfWarps + (threadIdx.x >> 5);
@@ -109,7 +109,7 @@ template <int NB, bool RING>
 __global__ void __launch_bounds__(32 * kBfWarps, 4)
 bf_level_kernel(const BfItem *__restrict__ items, int nitems, int L, int nhalf, int maxnc,
                 const int *__restrict__ ints, const uint2 *__restrict__ words,
-                const double *__restrict__ uin, double *__restrict__ uout, double *__restrict__ qt)
+                const double *__restrict__ uin, double *__restrict__ uout, QtView qt)
 {
     extern __shared__ __align__(16) double sout[];     // [kBfWarps][maxnc * 2 NB]
     const int lane = threadIdx.x & 31;
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(32 * kBfWarps)
 bf_r_rec_kernel(PlanView v, const BfRItem *__restrict__ items, int nitems, const RecStart *__restrict__ rs,
                 const int *__restrict__ ints, const double2 *__restrict__ ai, int nmaps, int b0,
                 double *__restrict__ ubuf0, double *__restrict__ ubuf1, const int *__restrict__ depth_par,
-                double *__restrict__ qt)
+                QtView qt)
 {
     const int lane = threadIdx.x & 31;
     const int w = blockIdx.x * kBfWarps + (threadIdx.x >> 5);
@@ -139,7 +139,7 @@ bf_r_rec_kernel(PlanView v, const BfRItem *__restrict__ items, int nitems, const
 // residual blocks of one map group (maps b0 .. b0+NB-1 of ai)
 template <int NB>
 int launch_r(const shtb_plan_s *p, const double2 *ai, int nmaps, int b0, double *u0, double *u1,
-             double *qt, cudaStream_t st)
+             QtView qt, cudaStream_t st)
 {
     const BfPlanDev &bf = *p->bf;
     if (bf.n_ritems == 0) return SHTB_OK;
@@ -161,7 +161,7 @@ int launch_r(const shtb_plan_s *p, const double2 *ai, int nmaps, int b0, double 
 
 // butterfly levels of one map group, top down; level 1 writes q^t
 template <int NB>
-int launch_levels(const shtb_plan_s *p, double *u0, double *u1, double *qt, cudaStream_t st)
+int launch_levels(const shtb_plan_s *p, double *u0, double *u1, QtView qt, cudaStream_t st)
 {
     const BfPlanDev &bf = *p->bf;
     for (int lev = bf.depth_max; lev >= 1; --lev) {
@@ -187,7 +187,7 @@ int launch_levels(const shtb_plan_s *p, double *u0, double *u1, double *qt, cuda
 // group's q^t is the caller's array (the Legendre stage alone).
 template <int NB>
 int run_group(const shtb_plan_s *p, const double2 *ai, int columns, int b0, int real, double *u0, double *u1,
-              double *qt, double *map, cudaStream_t st)
+              QtView qt, double *map, cudaStream_t st)
 {
     shtb_plan_s *pp = const_cast<shtb_plan_s *>(p);
     const int ev_leg = profile_begin(pp, st);
@@ -591,7 +591,7 @@ int launch_bf_synth(const shtb_plan_s *p, const double2 *alm, double2 *ai, void 
     double *u1 = u0 + (size_t)bf.u_entries * entry;
     double *qt_ws = u1 + (size_t)bf.u_entries * entry;
     const int columns = padded ? padded_maps(nmaps) : nmaps;
-    // q^t of map b in the caller's [columns][2][nhalf][L+1] array (Legendre stage alone)
+    // q^t of map b in the caller's array of [columns][2][nhalf][L+1] complex (Legendre stage alone)
     const size_t qt_map = (size_t)4 * p->nhalf * (p->lmax + 1);
     const int ev = profile_begin(const_cast<shtb_plan_s *>(p), st);
     bf_interleave_kernel<<<stage_grid(p, columns), 256, 0, st>>>(p->view, alm, ai, nmaps, columns,
@@ -601,7 +601,8 @@ int launch_bf_synth(const shtb_plan_s *p, const double2 *alm, double2 *ai, void 
     profile_end(const_cast<shtb_plan_s *>(p), st, 4, ev);
     for (int b0 = 0; b0 < columns;) {
         const int nb = group_width(columns - b0), real = std::min(nb, nmaps - b0);
-        double *qt = qt_out ? qt_out + (size_t)b0 * qt_map : qt_ws;
+        const QtView qt = qt_out ? QtView{qt_out + (size_t)b0 * qt_map, padded ? qt_pack(nb) : 0}
+                                 : QtView{qt_ws, qt_pack(nb)};
         int rc;
         switch (nb) {
         case 8: rc = run_group<8>(p, ai, columns, b0, real, u0, u1, qt, map, st); break;
@@ -627,7 +628,7 @@ int launch_bf_synth_to_host(shtb_plan_s *p, const double2 *alm, double2 *ai, voi
     const size_t entry = 16;
     double *u0 = (double *)ws;
     double *u1 = u0 + (size_t)bf.u_entries * entry;
-    double *qt = u1 + (size_t)bf.u_entries * entry;
+    double *qt_ws = u1 + (size_t)bf.u_entries * entry;
     const int columns = padded_maps(nmaps);
     bf_interleave_kernel<<<stage_grid(p, columns), 256, 0, st>>>(p->view, alm, ai, nmaps, columns,
                                                                  p->bf->rec ? p->view.coef : nullptr);
@@ -635,6 +636,7 @@ int launch_bf_synth_to_host(shtb_plan_s *p, const double2 *alm, double2 *ai, voi
     ++p->launches;
     for (int b0 = 0; b0 < columns;) {
         const int nb = group_width(columns - b0), real = std::min(nb, nmaps - b0);
+        const QtView qt{qt_ws, qt_pack(nb)};
         int rc = launch_bf_legendre_group(p, ai, columns, b0, nb, u0, u1, qt, st);
         if (rc) return rc;
         // ring stage chunk by chunk; each chunk's pixels go back while the
@@ -694,7 +696,7 @@ int launch_bf_gather(const shtb_plan_s *p, const double2 *const *alm_of_map, dou
 }
 
 int launch_bf_legendre_group(const shtb_plan_s *p, const double2 *ai, int nmaps, int b0, int nb, double *u0,
-                             double *u1, double *qt, cudaStream_t st)
+                             double *u1, QtView qt, cudaStream_t st)
 {
     int rc;
     switch (nb) {

@@ -247,17 +247,23 @@ int launch_phi_synth(const shtb_plan_s *p, const double2 *q, double *map, int nm
                      cudaStream_t st, bool one_stream = false);
 int launch_phi_adjoint(const shtb_plan_s *p, const double *map, double2 *q, int nmaps,
                        cudaStream_t st);
-int launch_phi_synth_qt(const shtb_plan_s *p, const double *qt, int nb, double *map, int b0,
+// q^t of a map group: complex, in packs of 2^lp maps, map b's q^t_m(z_r) at
+// q[((((b >> lp) 2 + t) nhalf + r) (L + 1) + m) 2^lp + (b mod 2^lp)]
+struct QtView {
+    double *q;
+    int lp;
+};
+int launch_phi_synth_qt(const shtb_plan_s *p, QtView qt, int nb, double *map, int b0,
                         cudaStream_t st);
 // ... for the rings of chunk `chunk` only (shtb_plan_s::kPhiChunks runs)
-int launch_phi_synth_qt_chunk(const shtb_plan_s *p, const double *qt, int nb, double *map, int b0, int chunk,
+int launch_phi_synth_qt_chunk(const shtb_plan_s *p, QtView qt, int nb, double *map, int b0, int chunk,
                               cudaStream_t st);
 // ... writing map b0 + b to map_of_map[b0 + b] (device array of map pointers)
-int launch_phi_synth_qt_ptr(const shtb_plan_s *p, const double *qt, int nb, double *const *map_of_map,
+int launch_phi_synth_qt_ptr(const shtb_plan_s *p, QtView qt, int nb, double *const *map_of_map,
                             int b0, cudaStream_t st);
 
 // shtb_butterfly.cu
-// polarised synthesis (shtb_spin.cu): parity halves of F+ and F- (map-major,
+// polarised synthesis (shtb_spin.cu): parity halves of F+ and F- (packs of two,
 // inputs E, B per pair) -> ring-major Q_m, U_m spectra
 int launch_spin_combine(const shtb_plan_s *p, const double *qt_plus, const double *qt_minus, double2 *qring,
                         int npairs, cudaStream_t st);
@@ -289,11 +295,18 @@ inline int padded_maps(int nmaps, int width = 8)
 }
 // width of the group that starts `left` padded columns before the end
 inline int group_width(int left) { return left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1; }
+// QtView::lp of a group: two maps of a (ring, m) side by side, so that the
+// items, which hold one m, write whole 32-byte sectors of q^t (level 1 of 8
+// maps at Nside = 512 .38 -> .31 ms; the ring stage, which reads one map,
+// stays at 1.03).  Packs of 4 and 8 leave level 1 there and cost the ring
+// stage its coalescing (1.05 and 1.18 ms).
+inline int qt_pack(int nb) { return nb > 1 ? 1 : 0; }
 
 size_t bf_workspace_bytes(const shtb_plan_s *p);
 // map != nullptr: the whole synthesis; map == nullptr: the Legendre stage
-// alone, q^t of map b written to qt_out + b [2][nhalf][L+1] complex
-// (padded: ai and qt_out have padded_maps(nmaps) columns and maps)
+// alone, q^t written to qt_out: padded, ai and qt_out have
+// padded_maps(nmaps) columns and maps, in packs of two where there are
+// several; else map b at qt_out + b [2][nhalf][L+1] complex
 int launch_bf_synth(const shtb_plan_s *p, const double2 *alm, double2 *ai, void *ws, double *map,
                     int nmaps, cudaStream_t st, double *qt_out = nullptr, bool padded = true);
 // whole synthesis with the maps copied back to host memory as the ring
@@ -307,7 +320,7 @@ void bf_release(shtb_plan_s *p);
 int launch_bf_gather(const shtb_plan_s *p, const double2 *const *alm_of_map, double2 *ai, int nmaps,
                      cudaStream_t st);
 int launch_bf_legendre_group(const shtb_plan_s *p, const double2 *ai, int nmaps, int b0, int nb, double *u0,
-                             double *u1, double *qt, cudaStream_t st);
+                             double *u1, QtView qt, cudaStream_t st);
 // g and aacc with `columns` columns (a sum of group widths)
 int launch_bf_adjoint(const shtb_plan_s *p, const double2 *g, double2 *aacc, void *ws, double2 *alm,
                       int nmaps, int columns, cudaStream_t st);

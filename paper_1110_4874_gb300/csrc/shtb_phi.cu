@@ -70,13 +70,13 @@ struct MapOut {
 template <int KIND>
 __global__ void __launch_bounds__(phi_threads<KIND>(), phi_min_blocks<KIND>())
 phi_synth_qt_kernel(PlanView v, const int *__restrict__ rings, const double2 *__restrict__ qt,
-                    MapOut mo, int b0)
+                    int lp, MapOut mo, int b0)
 {
     extern __shared__ fx2 sm[];
     const int ring = rings[blockIdx.x];
     const int b = blockIdx.y;
     double *base = mo.table ? mo.table[b0 + b] : mo.map + (size_t)(b0 + b) * v.npix;
-    shtb_dev::phi_synth_ring_qt<KIND, false>(v, ring, qt, b, base + v.ring_start[ring], sm);
+    shtb_dev::phi_synth_ring_qt<KIND, false>(v, ring, qt, lp, b, base + v.ring_start[ring], sm);
 }
 
 template <int KIND>
@@ -196,38 +196,37 @@ int launch_set(const shtb_plan_s *p, bool synth, const void *in, void *out, int 
 }
 
 template <int KIND>
-int launch_qt_set(const shtb_plan_s *p, const double2 *qt, int nb, MapOut map, int b0, const RingSet &rs,
+int launch_qt_set(const shtb_plan_s *p, QtView qt, int nb, MapOut map, int b0, const RingSet &rs,
                   cudaStream_t st)
 {
     const PlanView v = p->view;
     return launch_parts<KIND>(p, rs, (const void *)phi_synth_qt_kernel<KIND>,
                               [&](const int *rings, int n, int threads, size_t smem) {
                                   phi_synth_qt_kernel<KIND><<<dim3((unsigned)n, (unsigned)nb), threads, smem, st>>>(
-                                      v, rings, qt, map, b0);
+                                      v, rings, (const double2 *)qt.q, qt.lp, map, b0);
                               });
 }
 
 template <int KIND>
-int launch_qt_kind(const shtb_plan_s *p, const double2 *qt, int nb, MapOut map, int b0, cudaStream_t st)
+int launch_qt_kind(const shtb_plan_s *p, QtView qt, int nb, MapOut map, int b0, cudaStream_t st)
 {
     return launch_qt_set<KIND>(p, qt, nb, map, b0, ring_set(p, KIND), st);
 }
 
 template <int KIND>
-int launch_qt_list(const shtb_plan_s *p, const double2 *qt, int nb, MapOut map, int b0,
+int launch_qt_list(const shtb_plan_s *p, QtView qt, int nb, MapOut map, int b0,
                    const shtb_plan_s::ChunkKind &ck, cudaStream_t st)
 {
     return launch_qt_set<KIND>(p, qt, nb, map, b0, RingSet{p->d_chunk_list + ck.off, ck.n, ck.len,
                                                            KIND == kBluestein ? ck.split : ck.n, ck.len_small}, st);
 }
 
-int launch_qt_all(const shtb_plan_s *p, const double *qt, int nb, MapOut mo, int b0, cudaStream_t st)
+int launch_qt_all(const shtb_plan_s *p, QtView qt, int nb, MapOut mo, int b0, cudaStream_t st)
 {
-    const double2 *q2 = (const double2 *)qt;
     int rc;
-    if ((rc = launch_qt_kind<kBluestein>(p, q2, nb, mo, b0, st))) return rc;
-    if ((rc = launch_qt_kind<kDirect>(p, q2, nb, mo, b0, st))) return rc;
-    return launch_qt_kind<kDirectBig>(p, q2, nb, mo, b0, st);
+    if ((rc = launch_qt_kind<kBluestein>(p, qt, nb, mo, b0, st))) return rc;
+    if ((rc = launch_qt_kind<kDirect>(p, qt, nb, mo, b0, st))) return rc;
+    return launch_qt_kind<kDirectBig>(p, qt, nb, mo, b0, st);
 }
 
 // Tables from doubles to halves, in place
@@ -242,30 +241,28 @@ __global__ void ring_pack_kernel(double2 *t, size_t n, int bits)
 
 }  // namespace
 
-int launch_phi_synth_qt(const shtb_plan_s *p, const double *qt, int nb, double *map, int b0,
+int launch_phi_synth_qt(const shtb_plan_s *p, QtView qt, int nb, double *map, int b0,
                         cudaStream_t st)
 {
-    const double2 *q2 = (const double2 *)qt;
     const MapOut mo{map, nullptr};
     return side_by_side(
-        p, st, [&](cudaStream_t s2) { return launch_qt_kind<kBluestein>(p, q2, nb, mo, b0, s2); },
-        [&](cudaStream_t s2) { return launch_qt_kind<kDirect>(p, q2, nb, mo, b0, s2); },
-        [&](cudaStream_t s2) { return launch_qt_kind<kDirectBig>(p, q2, nb, mo, b0, s2); });
+        p, st, [&](cudaStream_t s2) { return launch_qt_kind<kBluestein>(p, qt, nb, mo, b0, s2); },
+        [&](cudaStream_t s2) { return launch_qt_kind<kDirect>(p, qt, nb, mo, b0, s2); },
+        [&](cudaStream_t s2) { return launch_qt_kind<kDirectBig>(p, qt, nb, mo, b0, s2); });
 }
 
-int launch_phi_synth_qt_chunk(const shtb_plan_s *p, const double *qt, int nb, double *map, int b0, int chunk,
+int launch_phi_synth_qt_chunk(const shtb_plan_s *p, QtView qt, int nb, double *map, int b0, int chunk,
                               cudaStream_t st)
 {
-    const double2 *q2 = (const double2 *)qt;
     const MapOut mo{map, nullptr};
     const auto *ck = p->chunk_kind[chunk];
     int rc;
-    if ((rc = launch_qt_list<kBluestein>(p, q2, nb, mo, b0, ck[1], st))) return rc;
-    if ((rc = launch_qt_list<kDirect>(p, q2, nb, mo, b0, ck[0], st))) return rc;
-    return launch_qt_list<kDirectBig>(p, q2, nb, mo, b0, ck[2], st);
+    if ((rc = launch_qt_list<kBluestein>(p, qt, nb, mo, b0, ck[1], st))) return rc;
+    if ((rc = launch_qt_list<kDirect>(p, qt, nb, mo, b0, ck[0], st))) return rc;
+    return launch_qt_list<kDirectBig>(p, qt, nb, mo, b0, ck[2], st);
 }
 
-int launch_phi_synth_qt_ptr(const shtb_plan_s *p, const double *qt, int nb, double *const *map_of_map,
+int launch_phi_synth_qt_ptr(const shtb_plan_s *p, QtView qt, int nb, double *const *map_of_map,
                             int b0, cudaStream_t st)
 {
     return launch_qt_all(p, qt, nb, MapOut{nullptr, map_of_map}, b0, st);

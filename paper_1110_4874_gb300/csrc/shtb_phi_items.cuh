@@ -846,21 +846,20 @@ __device__ __forceinline__ void phi_synth_ring(const PlanView &v, int ring, cons
 }
 
 // ... with q_m formed from the two parity halves of the butterfly output,
-// stored map-major: qt[((b * 2 + t) * nhalf + r) * (L + 1) + m] (complex);
-// north rings (ring < nhalf) take q^0 + q^1, their mirrors q^0 - q^1.
+// stored as QtView says (qt, lp); north rings (ring < nhalf) take q^0 + q^1, their mirrors q^0 - q^1.
 template <int KIND, bool CG>
-__device__ __forceinline__ void phi_synth_ring_qt(const PlanView &v, int ring, const double2 *qt, int b,
+__device__ __forceinline__ void phi_synth_ring_qt(const PlanView &v, int ring, const double2 *qt, int lp, int b,
                                                   double *out_ring, fx2 *sm)
 {
     const int Z = v.nhalf, L = v.lmax;
     const bool north = ring < Z;
     const int r = north ? ring : v.nrings - 1 - ring;
-    const double2 *q0 = qt + ((size_t)(b * 2) * Z + r) * (L + 1);
-    const double2 *q1 = q0 + (size_t)Z * (L + 1);
+    const double2 *q0 = qt + ((((size_t)((b >> lp) * 2) * Z + r) * (L + 1)) << lp) + (b & ((1 << lp) - 1));
+    const double2 *q1 = q0 + ((size_t)Z * (L + 1) << lp);
     auto qat = [=](int m) {
-        const double2 x0 = ldq<CG>(q0 + m);
+        const double2 x0 = ldq<CG>(q0 + ((size_t)m << lp));
         if (m + 1 > L) return x0;
-        return cadd(x0, cneg_if(ldq<CG>(q1 + m), !north));
+        return cadd(x0, cneg_if(ldq<CG>(q1 + ((size_t)m << lp)), !north));
     };
     phi_synth_ring_at<KIND>(v, ring, qat, out_ring, sm);
 }

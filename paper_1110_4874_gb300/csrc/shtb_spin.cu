@@ -13,8 +13,8 @@
 
 namespace {
 
-// qp, qm: map-major parity halves, q[((b * 2 + t) * nhalf + r) * (L + 1) + m],
-// inputs b = 2 pair (E) and 2 pair + 1 (B).  qring: ring-major
+// qp, qm: parity halves in packs of two, q[(((pair 2 + t) nhalf + r) (L + 1) + m) 2 + i],
+// i = 0 (E) and 1 (B) of a pair.  qring: ring-major
 // [2 npairs][nrings][L + 1], Q then U per pair.  One CTA per (ring, pair).
 __global__ void spin_combine_kernel(int L, int nhalf, int nrings, const double2 *__restrict__ qp,
                                     const double2 *__restrict__ qm, double2 *__restrict__ qring)
@@ -23,18 +23,18 @@ __global__ void spin_combine_kernel(int L, int nhalf, int nrings, const double2 
     const bool north = ring < nhalf;
     const int r = north ? ring : nrings - 1 - ring;
     const size_t half = (size_t)nhalf * (L + 1);
-    auto at = [&](const double2 *q, int b, int m, bool odd_mirror) {
-        const double2 *q0 = q + ((size_t)(b * 2) * nhalf + r) * (L + 1);
-        const double2 x0 = q0[m];
-        const double2 x1 = m + 1 <= L ? q0[half + m] : make_double2(0.0, 0.0);   // chain t = 1 exists
+    auto at = [&](const double2 *q, int i, int m, bool odd_mirror) {
+        const double2 *q0 = q + (((size_t)(pair * 2) * nhalf + r) * (L + 1) + m) * 2 + i;
+        const double2 x0 = q0[0];
+        const double2 x1 = m + 1 <= L ? q0[2 * half] : make_double2(0.0, 0.0);   // chain t = 1 exists
         if (north) return make_double2(x0.x + x1.x, x0.y + x1.y);
         return odd_mirror ? make_double2(x1.x - x0.x, x1.y - x0.y) : make_double2(x0.x - x1.x, x0.y - x1.y);
     };
     double2 *Q = qring + ((size_t)(2 * pair) * nrings + ring) * (L + 1);
     double2 *U = Q + (size_t)nrings * (L + 1);
     for (int m = threadIdx.x; m <= L; m += blockDim.x) {
-        const double2 Ep = at(qp, 2 * pair, m, false), Bp = at(qp, 2 * pair + 1, m, false);
-        const double2 Em = at(qm, 2 * pair, m, true), Bm = at(qm, 2 * pair + 1, m, true);
+        const double2 Ep = at(qp, 0, m, false), Bp = at(qp, 1, m, false);
+        const double2 Em = at(qm, 0, m, true), Bm = at(qm, 1, m, true);
         Q[m] = make_double2(-(Ep.x - Bm.y), -(Ep.y + Bm.x));
         U[m] = make_double2(-(Bp.x + Em.y), -(Bp.y - Em.x));
     }
