@@ -28,7 +28,7 @@ namespace {
 
 using namespace shtb_dev;
 
-// threads per ring CTA: the Bluestein variant holds up to ~8.4k complex
+// most threads of a ring CTA: the Bluestein variant holds up to ~8.4k complex
 // values of shared memory per CTA (one CTA per SM at the longest rings), so
 // it runs twice the threads
 template <int KIND>
@@ -94,10 +94,10 @@ phi_adjoint_kernel(PlanView v, const int *__restrict__ rings, const double *__re
 // one launch per ring kind: grid (rings of that kind) x maps, shared memory
 // for the kind's longest transform.  The Bluestein list is cut in two:
 // rings [0, split) at phi_threads (one CTA per SM at the longest lengths),
-// rings [split, n) -- transforms of at most kBlueSmallM points -- at half the
-// threads with shared memory for their own longest transform, so that two
-// CTAs share an SM and one's barriers between FFT passes are covered by the
-// other's work.  Every body loops over blockDim.x.
+// rings [split, n) -- transforms of at most kBlueSmallM points -- with fewer
+// threads and with shared memory for their own longest transform, so that two
+// or more CTAs share an SM and one's barriers between FFT passes are covered
+// by the others' work.  Every body loops over blockDim.x.
 // shared memory of a transform of `len` entries: the points and, while a
 // spectrum is folded, a 16-bit exponent for each
 size_t ring_smem_bytes(int len) { return (sizeof(fx2) + sizeof(short)) * (size_t)len + 16; }
@@ -117,6 +117,22 @@ RingSet ring_set(const shtb_plan_s *p, int kind)
     return {p->d_big_rings, (int)p->big_rings.size(), p->max_K_big, (int)p->big_rings.size(), 0};
 }
 
+// Half the threads where no ring of the plan's kind is long: a radix-r pass
+// over K points is K / r butterflies, which leaves most of 256 threads idle at
+// each barrier, and twice the CTAs share an SM.  Ring stage of 8 maps, 256
+// threads -> 128: Nside = 256 .346 -> .314 ms, 512 1.029 -> .915, 640 1.529 ->
+// 1.395, 768 2.171 -> 2.056; 1024 3.748 -> 3.999, so the line lies between
+// the longest rings of the last two (direct K 1536 and 2048).  The plan's
+// longest ring decides, not the launch's, so that parts of a plan's rings
+// take the same sums as the whole.
+template <int KIND>
+int part_threads(const shtb_plan_s *p, bool small)
+{
+    if (KIND == kBluestein)
+        return !small ? phi_threads<KIND>() : p->max_M_small <= 3072 ? 128 : 256;
+    return (KIND == kDirect ? p->max_K_direct <= 1536 : p->max_K_big <= 3072) ? 128 : phi_threads<KIND>();
+}
+
 // launch(rings, n, threads, smem bytes) for each non-empty part of rs
 template <int KIND, class Launch>
 int launch_parts(const shtb_plan_s *p, const RingSet &rs, const void *kernel, Launch launch)
@@ -125,12 +141,12 @@ int launch_parts(const shtb_plan_s *p, const RingSet &rs, const void *kernel, La
     SHTB_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)ring_smem_bytes(rs.len)));
     if (rs.split > 0) {
-        launch(rs.rings, rs.split, phi_threads<KIND>(), ring_smem_bytes(rs.len));
+        launch(rs.rings, rs.split, part_threads<KIND>(p, false), ring_smem_bytes(rs.len));
         SHTB_CUDA_TRY(cudaGetLastError());
         ++p->launches;
     }
     if (rs.split < rs.n) {
-        launch(rs.rings + rs.split, rs.n - rs.split, phi_threads<KIND>() / 2,
+        launch(rs.rings + rs.split, rs.n - rs.split, part_threads<KIND>(p, true),
                ring_smem_bytes(rs.len_small));
         SHTB_CUDA_TRY(cudaGetLastError());
         ++p->launches;

@@ -90,3 +90,21 @@ def test_scales_zero_rings_and_non_finite_values():
         assert not torch.isfinite(torch.view_as_real(ab[1, 5])).all()
         rest = [i for i in range(plan.nrings) if i != 5]
         assert torch.equal(ab[1, rest], back[1, rest]) and torch.equal(ab[0], back[0])
+
+
+@pytest.mark.parametrize("nside", [768, 769])
+def test_rings_at_the_line_between_block_sizes(nside):
+    """Longest rings of 4 x 768 pixels run 128 threads a block, longer ones
+    256; the bound is that of the transforms above."""
+    lmax = 24
+    plan = sh.Plan(nside, lmax, 0.0)
+    rings = oracle.healpix_rings(nside)
+    q = spectrum(plan, "flat", 5)
+    want = oracle.phi_synth(rings, lmax, q)
+    maps = torch.empty(2, plan.npix, dtype=torch.float64, device="cuda")
+    sh.shtb_test_phi(plan.handle, torch.from_numpy(q).cuda(), maps, 2)
+    assert np.linalg.norm(maps.cpu().numpy() - want) <= 1e-15 * np.linalg.norm(want)
+    want_q = oracle.phi_adjoint(rings, lmax, want)
+    back = torch.empty(2, plan.nrings, lmax + 1, dtype=torch.complex128, device="cuda")
+    sh.shtb_test_phi_adjoint(plan.handle, torch.from_numpy(want).cuda(), back, 2)
+    assert np.linalg.norm(back.cpu().numpy() - want_q) <= 1e-15 * np.linalg.norm(want_q)
