@@ -242,6 +242,8 @@ int launch_adjoint_parity(const shtb_plan_s *p, const double2 *qadj, double2 *g,
 size_t legendre_adjoint_state_bytes(const shtb_plan_s *p);
 
 // shtb_phi.cu
+// the plan's two side streams and their events, made on first use
+int side_streams(shtb_plan_s *p);
 // one_stream: no side streams (the allocation-free call creates none)
 int launch_phi_synth(const shtb_plan_s *p, const double2 *q, double *map, int nmaps,
                      cudaStream_t st, bool one_stream = false);

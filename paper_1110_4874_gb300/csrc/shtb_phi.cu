@@ -181,10 +181,7 @@ template <class Blue, class Direct, class Big>
 int side_by_side(const shtb_plan_s *p, cudaStream_t st, Blue blue, Direct direct, Big big)
 {
     shtb_plan_s *pp = const_cast<shtb_plan_s *>(p);
-    if (!pp->ring_stream[0]) {
-        for (auto &s2 : pp->ring_stream) SHTB_CUDA_TRY(cudaStreamCreateWithFlags(&s2, cudaStreamNonBlocking));
-        for (auto &e : pp->ring_ev) SHTB_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    }
+    if (int rs = side_streams(pp)) return rs;
     SHTB_CUDA_TRY(cudaEventRecord(pp->ring_ev[0], st));
     for (cudaStream_t s2 : pp->ring_stream) SHTB_CUDA_TRY(cudaStreamWaitEvent(s2, pp->ring_ev[0], 0));
     int rc;
@@ -256,6 +253,14 @@ __global__ void ring_pack_kernel(double2 *t, size_t n, int bits)
 }
 
 }  // namespace
+
+int side_streams(shtb_plan_s *p)
+{
+    if (p->ring_stream[0]) return SHTB_OK;
+    for (auto &s2 : p->ring_stream) SHTB_CUDA_TRY(cudaStreamCreateWithFlags(&s2, cudaStreamNonBlocking));
+    for (auto &e : p->ring_ev) SHTB_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    return SHTB_OK;
+}
 
 int launch_phi_synth_qt(const shtb_plan_s *p, QtView qt, int nb, double *map, int b0,
                         cudaStream_t st)
