@@ -316,38 +316,26 @@ __device__ __forceinline__ int pass_bits(int Ns)
 template <int R, bool INV, class TW>
 __device__ __forceinline__ unsigned mx_pass(fx2 *x, int Ntot, int Nseq, int B, const TW &tw, int s)
 {
+    // twiddles are 1 in the first pass of decimation in time and the last of
+    // decimation in frequency
     const int Ns = B / R, step = Nseq / B;
+    const bool twiddled = Ns > 1;
     unsigned mag = 0;
-    if (Ns == 1) {
-        // the first pass of decimation in time, the last of decimation in
-        // frequency: every twiddle is 1
-        for (int t = threadIdx.x; t < Ntot / R; t += blockDim.x) {
-            fx2 a[R];
-#pragma unroll
-            for (int q = 0; q < R; ++q) a[q] = frshift(fshl(x[t * R + q], s), 2);
-            dft_small<R, INV ? 1 : -1>(a);
-#pragma unroll
-            for (int q = 0; q < R; ++q) {
-                x[t * R + q] = a[q];
-                mag |= fmag(a[q]);
-            }
-        }
-        return mag;
-    }
     for (int t = threadIdx.x; t < Ntot / R; t += blockDim.x) {
         const int j = t % Ns, base = (t - j) * R + j;
         fx2 a[R];
 #pragma unroll
         for (int q = 0; q < R; ++q) a[q] = fshl(x[base + q * Ns], s);
         a[0] = frshift(a[0], 2);
-        if constexpr (INV) {
+        if (INV && twiddled) {
 #pragma unroll
             for (int p = 1; p < R; ++p) a[p] = fmul(a[p], tw(p * j * step));
-            dft_small<R, 1>(a);
         } else {
 #pragma unroll
             for (int p = 1; p < R; ++p) a[p] = frshift(a[p], 2);
-            dft_small<R, -1>(a);
+        }
+        dft_small<R, INV ? 1 : -1>(a);
+        if (!INV && twiddled) {
             a[0] = frshift(a[0], 2);
 #pragma unroll
             for (int p = 1; p < R; ++p) a[p] = fmul<true>(a[p], tw(p * j * step));
