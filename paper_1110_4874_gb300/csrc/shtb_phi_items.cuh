@@ -454,22 +454,12 @@ struct RaderCtx {
     fx2 *scratch;
 };
 
-template <bool CONJ>
-__device__ void rader_pass(fx2 *x, int N, const RaderCtx &c, FxScale &sc);
-
 // One pass, its barrier before it included.  BIG: the radix-11 and radix-13
 // butterflies are compiled in (they need many more registers; only lengths
-// with those factors are run with BIG); RADER: a radix above 13 is a prime
-// done by Rader's algorithm (BIG kernels only)
-template <bool INV, bool BIG, bool RADER, class TW>
-__device__ __forceinline__ void mx_pass_any(int r, fx2 *x, int Ntot, int Nseq, int B, const TW &tw, FxScale &sc,
-                                            const RaderCtx *rc)
+// with those factors are run with BIG)
+template <bool INV, bool BIG, class TW>
+__device__ __forceinline__ void mx_pass_any(int r, fx2 *x, int Ntot, int Nseq, int B, const TW &tw, FxScale &sc)
 {
-    if constexpr (RADER)
-        if (r > 13) {
-            rader_pass<!INV>(x, Ntot, *rc, sc);
-            return;
-        }
     const int s = sc.enter(), Ns = B / r;
     unsigned mag = 0;
     switch (r) {
@@ -492,30 +482,30 @@ __device__ __forceinline__ void mx_pass_any(int r, fx2 *x, int Ntot, int Nseq, i
 // natural order in, position order out, exponent -1; Ntot / Nseq sequences
 // of Nseq points transformed side by side.  The results' size is left for
 // the caller's FxScale::enter, which is also the barrier after the last pass.
-template <bool BIG, bool RADER, class TW>
+template <bool BIG, class TW>
 __device__ __forceinline__ void fft_mx_dif(fx2 *x, int Ntot, int Nseq, const int *__restrict__ rl, const TW &tw,
-                                           FxScale &sc, const RaderCtx *rc = nullptr)
+                                           FxScale &sc)
 {
     const int n = rl[0];
     int B = Nseq;
     for (int i = 0; i < n; ++i) {
         const int r = rl[1 + i];
-        mx_pass_any<false, BIG, RADER>(r, x, Ntot, Nseq, B, tw, sc, rc);
+        mx_pass_any<false, BIG>(r, x, Ntot, Nseq, B, tw, sc);
         B /= r;
     }
 }
 
 // position order in, natural order out, exponent +1 (unnormalised)
-template <bool BIG, bool RADER, class TW>
+template <bool BIG, class TW>
 __device__ __forceinline__ void fft_mx_dit(fx2 *x, int Ntot, int Nseq, const int *__restrict__ rl, const TW &tw,
-                                           FxScale &sc, const RaderCtx *rc = nullptr)
+                                           FxScale &sc)
 {
     const int n = rl[0];
     int B = 1;
     for (int i = n - 1; i >= 0; --i) {
         const int r = rl[1 + i];
         B *= r;
-        mx_pass_any<true, BIG, RADER>(r, x, Ntot, Nseq, B, tw, sc, rc);
+        mx_pass_any<true, BIG>(r, x, Ntot, Nseq, B, tw, sc);
     }
 }
 
@@ -571,7 +561,7 @@ struct TwTable {
 __device__ __forceinline__ void bluestein_mx(fx2 *x, int M, const int4 *__restrict__ fb, const int *__restrict__ rl,
                                              const TwTable &tw, FxScale &sc)
 {
-    fft_mx_dif<false, false>(x, M, M, rl, tw, sc);
+    fft_mx_dif<false>(x, M, M, rl, tw, sc);
     const int s = sc.enter();
     unsigned mag = 0;
     for (int k = threadIdx.x; k < M; k += blockDim.x) {
@@ -581,7 +571,7 @@ __device__ __forceinline__ void bluestein_mx(fx2 *x, int M, const int4 *__restri
     }
     sc.e += 2;
     sc.leave(mag);
-    fft_mx_dit<false, false>(x, M, M, rl, tw, sc);
+    fft_mx_dit<false>(x, M, M, rl, tw, sc);
 }
 
 // x true = x 2^from in units of 2^to, to nearest
@@ -605,67 +595,150 @@ __device__ __forceinline__ fx2 frescale(fx2 a, int from, int to)
 // frequency before the product.  Exponent +1; CONJ = true gives exponent -1
 // as conj(DFT(conj a)).  The a_0 stay in the units they have when the pass
 // begins; at the end all points are in the convolution's units.
-template <bool CONJ>
-__device__ void rader_pass(fx2 *x, int N, const RaderCtx &c, FxScale &sc)
-{
-    const RaderInfo ri = *c.ri;
-    const int p = ri.p, n = ri.n, tot = (N / p) * n;
-    const int *__restrict__ ga = c.ints + ri.ga;
-    const int *__restrict__ gi = c.ints + ri.gi;
-    const int4 *__restrict__ G = c.tab + ri.G;
-    const int *__restrict__ rl = c.rad + ri.rl;
-    const TwTable tw{c.tab + ri.tw};
-    fx2 *S = c.scratch;
-    const int s0 = sc.enter();
-    const int e0 = sc.e + s0;                          // units of the a_0 left in x
-    unsigned mag = 0;
-    for (int e = threadIdx.x; e < tot; e += blockDim.x) {
-        const int b = e / n, v = e - b * n;
-        fx2 a = fshl(x[b * p + __ldg(gi + v)], s0);
-        if (CONJ) a = fconj(a);
-        S[e] = a;
-        mag |= fmag(a);
+struct RaderRun {
+    RaderCtx c;
+    RaderInfo ri;
+    int N, tot, e0, e1;                                // e0: units of the a_0 left in x; e1: of y_0
+
+    RaderRun() = default;
+    __device__ __forceinline__ RaderRun(const RaderCtx &c, int N) : c(c), ri(*c.ri), N(N), tot((N / ri.p) * ri.n) {}
+
+    template <bool CONJ>
+    __device__ __forceinline__ void gather(fx2 *x, FxScale &sc)
+    {
+        const int *__restrict__ gi = c.ints + ri.gi;
+        const int s0 = sc.enter();
+        e0 = sc.e + s0;
+        unsigned mag = 0;
+        for (int e = threadIdx.x; e < tot; e += blockDim.x) {
+            const int b = e / ri.n, v = e - b * ri.n;
+            fx2 a = fshl(x[b * ri.p + __ldg(gi + v)], s0);
+            if (CONJ) a = fconj(a);
+            c.scratch[e] = a;
+            mag |= fmag(a);
+        }
+        sc.leave(mag);
     }
-    sc.leave(mag);
-    fft_mx_dif<true, false>(S, tot, n, rl, tw, sc);
+
     // y_0 (and a_0 with the product) may need as many more bits as a_0 has
     // above the rest: both sides at a quarter of their size, in the larger units
-    const int s1 = sc.enter(), e1 = max(sc.e, e0) + 2;
-    mag = 0;
-    for (int e = threadIdx.x; e < tot; e += blockDim.x) {
-        const int b = e / n, v = e - b * n;
-        const fx2 A = frescale(fshl(S[e], s1), sc.e, e1);
-        fx2 C = fmul(A, __ldg(G + v));                 // e1 + 2
-        if (v == 0) {
-            fx2 a0 = frescale(CONJ ? fconj(x[b * p]) : x[b * p], e0, e1);
-            fx2 y0 = fadd(a0, A);
-            if (CONJ) y0 = fconj(y0);
-            x[b * p] = y0;                             // in units of 2^e1
-            mag |= fmag(frshift(y0, 2));
-            C = fadd(C, frshift(a0, 2));
+    template <bool CONJ>
+    __device__ __forceinline__ void product(fx2 *x, FxScale &sc)
+    {
+        const int4 *__restrict__ G = c.tab + ri.G;
+        fx2 *S = c.scratch;
+        const int s1 = sc.enter();
+        e1 = max(sc.e, e0) + 2;
+        unsigned mag = 0;
+        for (int e = threadIdx.x; e < tot; e += blockDim.x) {
+            const int b = e / ri.n, v = e - b * ri.n;
+            const fx2 A = frescale(fshl(S[e], s1), sc.e, e1);
+            fx2 C = fmul(A, __ldg(G + v));             // e1 + 2
+            if (v == 0) {
+                fx2 a0 = frescale(CONJ ? fconj(x[b * ri.p]) : x[b * ri.p], e0, e1);
+                fx2 y0 = fadd(a0, A);
+                if (CONJ) y0 = fconj(y0);
+                x[b * ri.p] = y0;                      // in units of 2^e1
+                mag |= fmag(frshift(y0, 2));
+                C = fadd(C, frshift(a0, 2));
+            }
+            S[e] = C;
+            mag |= fmag(C);
         }
-        S[e] = C;
-        mag |= fmag(C);
+        sc.e = e1 + 2;
+        sc.leave(mag);
     }
-    sc.e = e1 + 2;
-    sc.leave(mag);
-    fft_mx_dit<true, false>(S, tot, n, rl, tw, sc);
-    const int s2 = sc.enter(), e2 = max(sc.e, e1) + 1;
-    mag = 0;
-    for (int e = threadIdx.x; e < tot; e += blockDim.x) {
-        const int b = e / n, w = e - b * n;
-        fx2 y = frescale(fshl(S[e], s2), sc.e, e2);
-        if (CONJ) y = fconj(y);
-        x[b * p + __ldg(ga + w)] = y;
-        mag |= fmag(y);
-        if (w == 0) {
-            const fx2 y0 = frescale(x[b * p], e1, e2);
-            x[b * p] = y0;
-            mag |= fmag(y0);
+
+    template <bool CONJ>
+    __device__ __forceinline__ void scatter(fx2 *x, FxScale &sc)
+    {
+        const int *__restrict__ ga = c.ints + ri.ga;
+        const int s2 = sc.enter(), e2 = max(sc.e, e1) + 1;
+        unsigned mag = 0;
+        for (int e = threadIdx.x; e < tot; e += blockDim.x) {
+            const int b = e / ri.n, w = e - b * ri.n;
+            fx2 y = frescale(fshl(c.scratch[e], s2), sc.e, e2);
+            if (CONJ) y = fconj(y);
+            x[b * ri.p + __ldg(ga + w)] = y;
+            mag |= fmag(y);
+            if (w == 0) {
+                const fx2 y0 = frescale(x[b * ri.p], e1, e2);
+                x[b * ri.p] = y0;
+                mag |= fmag(y0);
+            }
         }
+        sc.e = e2;
+        sc.leave(mag);
     }
-    sc.e = e2;
-    sc.leave(mag);
+};
+
+// a ring's twiddles (TwRing) or, with J = 0, a table's (TwTable)
+struct TwAny {
+    const int4 *T;
+    int J;
+    __device__ __forceinline__ int4 operator()(int t) const
+    {
+        const int n = J ? 4 * t : t;
+        const bool neg = J && n >= J;
+        return wneg_if(__ldg(T + (neg ? n - J : n)), neg);
+    }
+};
+
+// fft_mx_dif and fft_mx_dit of a BIG ring, whose first (last) radix may be a
+// Rader prime.  The ring's passes and those of the convolution that go the
+// same way run through one body, in turn: the kernels are held by instruction
+// fetches, and a body of all radices each for the ring and for both ways of
+// the convolution was three where two do (Nside = 512, ring stage of 8 maps
+// .900 -> .862 ms, adjoint .983 -> .944; 256: .304 -> .279 and .347 -> .323).
+__device__ __forceinline__ void fft_big_dif(fx2 *x, int K, const int *__restrict__ rl, const TwRing &tw, FxScale &sc,
+                                            const RaderCtx *rc)
+{
+    RaderRun run = rc ? RaderRun(*rc, K) : RaderRun();
+#pragma unroll 1
+    for (int phase = 0; phase < (rc ? 2 : 1); ++phase) {
+        fx2 *y = phase ? rc->scratch : x;
+        const int *__restrict__ l = phase ? run.c.rad + run.ri.rl : rl;
+        const int Ntot = phase ? run.tot : K, Nseq = phase ? run.ri.n : K;
+        const TwAny w = phase ? TwAny{run.c.tab + run.ri.tw, 0} : TwAny{tw.T, tw.J};
+        const int n = l[0] - (rc && !phase);
+        int B = Nseq;
+        for (int i = 0; i < n; ++i) {
+            const int r = l[1 + i];
+            mx_pass_any<false, true>(r, y, Ntot, Nseq, B, w, sc);
+            B /= r;
+        }
+        if (rc && !phase) run.gather<true>(x, sc);
+    }
+    if (!rc) return;
+    run.product<true>(x, sc);
+    fft_mx_dit<true>(rc->scratch, run.tot, run.ri.n, run.c.rad + run.ri.rl, TwTable{run.c.tab + run.ri.tw}, sc);
+    run.scatter<true>(x, sc);
+}
+
+__device__ __forceinline__ void fft_big_dit(fx2 *x, int K, const int *__restrict__ rl, const TwRing &tw, FxScale &sc,
+                                            const RaderCtx *rc)
+{
+    RaderRun run = rc ? RaderRun(*rc, K) : RaderRun();
+    if (rc) {
+        run.gather<false>(x, sc);
+        fft_mx_dif<true>(rc->scratch, run.tot, run.ri.n, run.c.rad + run.ri.rl, TwTable{run.c.tab + run.ri.tw}, sc);
+        run.product<false>(x, sc);
+    }
+#pragma unroll 1
+    for (int phase = rc ? 0 : 1; phase < 2; ++phase) {
+        fx2 *y = phase ? x : rc->scratch;
+        const int *__restrict__ l = phase ? rl : run.c.rad + run.ri.rl;
+        const int Ntot = phase ? K : run.tot, Nseq = phase ? K : run.ri.n;
+        const TwAny w = phase ? TwAny{tw.T, tw.J} : TwAny{run.c.tab + run.ri.tw, 0};
+        int B = 1, i = l[0] - 1;
+        if (rc && phase) B = l[1 + i--];               // the Rader prime
+        for (; i >= 0; --i) {
+            const int r = l[1 + i];
+            B *= r;
+            mx_pass_any<true, true>(r, y, Ntot, Nseq, B, w, sc);
+        }
+        if (!phase) run.scatter<false>(x, sc);
+    }
 }
 
 // The Rader context of a ring of a BIG kernel (nullptr for other rings):
@@ -815,7 +888,8 @@ __device__ __forceinline__ void phi_synth_ring_at(const PlanView &v, int ring, Q
     }
     sc.leave(mag);
     if constexpr (BLUE) bluestein_mx(sm, M, ring_table(v.mfb) + v.ring_mfb[ring], rl, TwTable{ring_table(v.mtw) + v.ring_mtw[ring]}, sc);
-    else fft_mx_dit<BIG, BIG>(sm, K, K, rl, TwRing{T, J}, sc, rcp);
+    else if constexpr (BIG) fft_big_dit(sm, K, rl, TwRing{T, J}, sc, rcp);
+    else fft_mx_dit<false>(sm, K, K, rl, TwRing{T, J}, sc);
     const int sh = sc.enter();
     const int be = sc.e + (BLUE ? 2 : 0) + 1054;
     for (int n = threadIdx.x; n < K; n += blockDim.x) {
@@ -926,7 +1000,8 @@ __device__ __forceinline__ void phi_adjoint_ring(const PlanView &v, int ring, co
         sc.e += 2;
         sc.leave(mag);
     } else {
-        fft_mx_dif<BIG, BIG>(sm, K, K, rl, TwRing{T, J}, sc, rcp);
+        if constexpr (BIG) fft_big_dif(sm, K, rl, TwRing{T, J}, sc, rcp);
+        else fft_mx_dif<false>(sm, K, K, rl, TwRing{T, J}, sc);
     }
     const int sh = sc.enter();
     const int be = sc.e + 1 + (s ? 4 : 2) + 1054;
