@@ -31,11 +31,11 @@
 // loss would be one unit of a diagonal's sum.
 //
 // Measured (GB300, Nside = 512, L = 1024, eps = 1e-10; residual blocks plus
-// levels, FP64 FMA kernels before): 8 maps 5.31 -> 1.57 ms, 4 maps 2.79 ->
-// 1.23, 2 maps 1.69 -> 0.95, 1 map 0.93 -> 0.80; at 8 maps the adjoint's
+// levels, FP64 FMA kernels before): 8 maps 5.31 -> 1.50 ms, 4 maps 2.79 ->
+// 1.23, 2 maps 1.69 -> 0.95, 1 map 0.93 -> 0.79; at 8 maps the adjoint's
 // levels and residual blocks 5.75 -> 1.83 ms.  What bounds them now is the
 // latency of loads and of the integer chains at 16 warps an SM (issue slots
-// 42 % used, tensor pipe 20-27 %, FP64 pipe 1 %).
+// 41-52 % used, tensor pipe 17-29 %, FP64 pipe 1 %).
 //
 // Results do not depend on the other components, on how maps are grouped or
 // on the lane layout: the sums are exact, and chunks of 32 are added in FP64

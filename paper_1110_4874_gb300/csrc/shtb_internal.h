@@ -283,8 +283,8 @@ int launch_alm_quadrature_add(const shtb_plan_s *p, const double2 *g, double2 *a
                               bool first, cudaStream_t st);
 
 // Map groups.  The butterfly carries 8, 4, 2 or 1 maps an entry, and a group
-// of 4 costs little more than one of 1 (block products at Nside = 512: 0.80,
-// 0.95, 1.23 and 1.57 ms for 1, 2, 4 and 8 maps), so the maps left after the
+// of 4 costs little more than one of 1 (block products at Nside = 512: 0.79,
+// 0.95, 1.23 and 1.50 ms for 1, 2, 4 and 8 maps), so the maps left after the
 // eights are padded to the next of these widths and run as one group, in
 // place of several.  The a_lm-sided arrays [idx][maps] have padded_maps
 // columns; the padding repeats the last map and is never returned.

@@ -14,9 +14,11 @@
 // so adds an error of a few 2^-58 of the largest point, below the last place
 // of the FP64 numbers the ring is made from and turned into at the end.
 // Measured (Nside = 512, L = 1024, 8 maps; FP64 transforms before): ring
-// synthesis 1.80 -> 1.14 ms, adjoint 2.42 -> 1.16 ms; Nside = 1024: 7.60 ->
-// 3.90 and 9.79 -> 4.12 ms.  What bounds them now is the issue of integer
-// instructions (55 to 68 % of the slots at the direct lengths).
+// synthesis 1.80 -> .86 ms, adjoint 2.42 -> .94 ms; Nside = 1024: 7.60 ->
+// 3.76 and 9.79 -> 4.03 ms (1.14, 1.16, 3.90 and 4.12 by the change of
+// arithmetic alone).  What bounds them now is the issue of integer
+// instructions at the direct lengths (65 to 71 % of the slots) and latency
+// and instruction fetches at the others (36 to 49 %, 16 warps an SM).
 // Rings whose values hold an infinity or a NaN, or lie outside 1e-217 ..
 // 1e204, are summed directly in FP64 (ring_direct_*), as such values spread.
 #pragma once
