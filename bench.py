@@ -49,8 +49,9 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
 # valid only while the kernel's source files are unchanged.
 NCU_TRAFFIC = {
     "legendre_synth_kernel": {
-        "sources": ["paper_1110_4874_gb300/csrc/shtb_legendre.cu", "paper_1110_4874_gb300/csrc/shtb_limbs.cuh"],
-        "sha256": "3a4468e4f42288dc25261e3fb85dafc9428f4e56d0a3f61749e7c8923370b2f6",
+        "sources": ["paper_1110_4874_gb300/csrc/shtb_legendre.cu::legendre_synth_kernel",
+                    "paper_1110_4874_gb300/csrc/shtb_limbs.cuh"],
+        "sha256": "f80381d57e0e82704ed2c8f23125413a42d524caf0c5ef1c93a7d41deb956156",
         # measured at Nside=512, L=1024; every array scales with Nside*L (x16)
         "bytes": 16 * (122_818_560 + 215_400_960),
         "profile": "profiles/legendre_kernels_nside512_l1024_b8.md",

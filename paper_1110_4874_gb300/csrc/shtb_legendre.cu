@@ -25,7 +25,7 @@
 // for an integer multiply-add, held these kernels with both done in FP64.
 // Legendre stage, FP64 sums -> this (ms):
 //   nside 64, lmax 128, 1 map      synthesis  .047 -> .028  adjoint  .054 -> .037
-//   nside 100, lmax 255, 1 map                .095 -> .051           .140 -> .085
+//   nside 100, lmax 255, 1 map                .095 -> .051           .140 -> .068
 //   nside 256, lmax 512, 4 maps               .996 -> .418          1.385 -> .555
 //   nside 256, lmax 512, 8 maps              1.730 -> .711          2.416 -> .931
 //   nside 512, lmax 1024, 8 maps             12.22 -> 4.89          13.94 -> 5.48
@@ -381,10 +381,12 @@ __global__ void __launch_bounds__(256) adjoint_parity_kernel(PlanView v, const d
     }
 }
 
-// Warps of a CTA: an order's chains are as long as its tiles are many, and
+// Warps W of a CTA: an order's chains are as long as its tiles are many, and
 // orders are too few to fill the chip by themselves.  4, 8, 16 warps: .786,
-// .542, .682 ms at nside 256 with 4 maps, 1.31, .89, 1.06 with 8, .51, .35, .38 with 1.
-constexpr int kAdjWarps = 8;
+// .542, .682 ms at nside 256 with 4 maps, 1.31, .89, 1.06 with 8, .51, .35,
+// .38 with 1.  16 where that is a chunk of rings for each and 8 would take two
+// (5 to 8 chunks): .096 -> .076 ms at nside 128 with 1 map, .145 -> .114
+// with 4, .245 -> .191 with 8; nside 100 .085 -> .068, .132 -> .102, .214 -> .173.
 constexpr int kTilePad = 33;   // row stride (doubles) of the 32x32 tile: no bank conflicts
 
 // per warp: the tile of V and the limbs of 32 rings' g (the sums' trade later)
@@ -423,8 +425,8 @@ __device__ __noinline__ void plain_chain_adjoint(const PlanView &v, int m, int t
 
 // One CTA per m: the even warps take the even chain, the odd ones the odd
 // chain, each its share of the chunks of 32 rings.
-template <int NB>
-__global__ void __launch_bounds__(32 * kAdjWarps, 16 / kAdjWarps)
+template <int NB, int W>
+__global__ void __launch_bounds__(32 * W, 16 / W)
 legendre_adjoint_kernel(PlanView v, const double2 *__restrict__ g, double2 *__restrict__ aacc,
                         RecState *__restrict__ state, int nmaps, int b0)
 {
@@ -450,7 +452,7 @@ legendre_adjoint_kernel(PlanView v, const double2 *__restrict__ g, double2 *__re
         const int jt = ti * 32;
         LegSums<C> sums;
         sums.clear(Z);
-        for (int c = set; c < nchunk && jt < n; c += kAdjWarps / 2) {
+        for (int c = set; c < nchunk && jt < n; c += W / 2) {
             const int r = c * 32 + lane;
             const bool valid = r < Z;
             const int rr = valid ? r : Z - 1;
@@ -503,7 +505,7 @@ legendre_adjoint_kernel(PlanView v, const double2 *__restrict__ g, double2 *__re
             if (j >= (tt == 0 ? n0 : dchain_len(L, m, 1))) continue;
             double2 sum = make_double2(0.0, 0.0);
 #pragma unroll
-            for (int w = tt; w < kAdjWarps; w += 2) {
+            for (int w = tt; w < W; w += 2) {
                 const double *p = smd + (size_t)w * adjoint_warp_smem_doubles<NB>() + 2 * b * kTilePad + jj;
                 sum.x += p[0];
                 sum.y += p[kTilePad];
@@ -538,17 +540,33 @@ __global__ void alm_finish_kernel(PlanView v, const double2 *__restrict__ aacc,
     }
 }
 
-template <int NB>
+template <int NB, int W>
 int launch_adjoint_nb(const shtb_plan_s *p, const double2 *g, double2 *aacc, RecState *state,
                       int nmaps, int b0, cudaStream_t st)
 {
-    const size_t smem = sizeof(double) * adjoint_warp_smem_doubles<NB>() * kAdjWarps;
-    SHTB_CUDA_TRY(cudaFuncSetAttribute(legendre_adjoint_kernel<NB>,
+    const size_t smem = sizeof(double) * adjoint_warp_smem_doubles<NB>() * W;
+    SHTB_CUDA_TRY(cudaFuncSetAttribute(legendre_adjoint_kernel<NB, W>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    legendre_adjoint_kernel<NB><<<p->lmax + 1, 32 * kAdjWarps, smem, st>>>(p->view, g, aacc, state,
+    legendre_adjoint_kernel<NB, W><<<p->lmax + 1, 32 * W, smem, st>>>(p->view, g, aacc, state,
                                                                            nmaps, b0);
     ++p->launches;
     SHTB_CUDA_TRY(cudaGetLastError());
+    return SHTB_OK;
+}
+
+template <int W>
+int launch_adjoint_groups(const shtb_plan_s *p, const double2 *g, double2 *aacc, RecState *state, int nmaps,
+                          cudaStream_t st)
+{
+    for (int b0 = 0; b0 < nmaps;) {
+        const int left = nmaps - b0;
+        int rc;
+        if (left >= 8) { rc = launch_adjoint_nb<8, W>(p, g, aacc, state, nmaps, b0, st); b0 += 8; }
+        else if (left >= 4) { rc = launch_adjoint_nb<4, W>(p, g, aacc, state, nmaps, b0, st); b0 += 4; }
+        else if (left >= 2) { rc = launch_adjoint_nb<2, W>(p, g, aacc, state, nmaps, b0, st); b0 += 2; }
+        else { rc = launch_adjoint_nb<1, W>(p, g, aacc, state, nmaps, b0, st); b0 += 1; }
+        if (rc) return rc;
+    }
     return SHTB_OK;
 }
 
@@ -612,18 +630,11 @@ int launch_legendre_adjoint(const shtb_plan_s *p, const double2 *qadj, double2 *
     // ws: [g: (L+1)*2*Z*nmaps double2][state: (L+1)*Z RecState]
     double2 *g = (double2 *)ws;
     RecState *state = (RecState *)(g + (size_t)(p->lmax + 1) * 2 * p->nhalf * nmaps);
-    int rc0 = launch_adjoint_parity(p, qadj, g, nmaps, nmaps, st);
-    if (rc0) return rc0;
-    for (int b0 = 0; b0 < nmaps;) {
-        const int left = nmaps - b0;
-        int rc;
-        if (left >= 8) { rc = launch_adjoint_nb<8>(p, g, aacc, state, nmaps, b0, st); b0 += 8; }
-        else if (left >= 4) { rc = launch_adjoint_nb<4>(p, g, aacc, state, nmaps, b0, st); b0 += 4; }
-        else if (left >= 2) { rc = launch_adjoint_nb<2>(p, g, aacc, state, nmaps, b0, st); b0 += 2; }
-        else { rc = launch_adjoint_nb<1>(p, g, aacc, state, nmaps, b0, st); b0 += 1; }
-        if (rc) return rc;
-    }
-    return SHTB_OK;
+    int rc = launch_adjoint_parity(p, qadj, g, nmaps, nmaps, st);
+    if (rc) return rc;
+    const int nchunk = (p->nhalf + 31) / 32;           // the same warps for every map count: the same bits
+    return nchunk > 4 && nchunk <= 8 ? launch_adjoint_groups<16>(p, g, aacc, state, nmaps, st)
+                                     : launch_adjoint_groups<8>(p, g, aacc, state, nmaps, st);
 }
 
 int launch_alm_finish(const shtb_plan_s *p, const double2 *aacc, double2 *alm, int nmaps,

@@ -77,3 +77,17 @@ def test_non_finite_maps_stay_apart(bad):
     keep = [i for i in range(8) if i != 5]
     assert torch.equal(back[keep], want[keep])
     assert not torch.isfinite(back[5]).all()
+
+
+# 4, 5, 8 and 9 chunks of 32 half-rings: 8 and 16 warps an order
+@pytest.mark.parametrize("nside", [64, 65, 128, 129])
+@pytest.mark.parametrize("nmaps", [1, 2, 4, 8])
+def test_adjoint_at_the_lines_between_block_sizes(nside, nmaps):
+    lmax = 40
+    plan, rings = sh.Plan(nside, lmax, 0.0), orc.healpix_rings(nside)
+    f = torch.from_numpy(synthetic.gaussian_map(plan.npix, nmaps, seed=9)).cuda()
+    back = plan.adjoint(f)
+    want = orc.adjoint(rings, lmax, f[nmaps - 1].cpu().numpy())
+    got = back[nmaps - 1].cpu().numpy()
+    assert np.linalg.norm(got - want) <= 4 * (lmax + 16) * 2.0 ** -53 * np.linalg.norm(want)
+    assert torch.equal(plan.adjoint(f[nmaps - 1]), back[nmaps - 1])
