@@ -10,9 +10,13 @@
 // FP64 takes 16.  A ring's points share one power of two: every pass first
 // shifts them up so that the largest component has 61 bits (its size is known
 // from the pass before: one OR a component, one shared-memory OR a warp) and
-// then works without overflow, rounding its results to whole units.  A pass
-// so adds an error of a few 2^-58 of the largest point, below the last place
-// of the FP64 numbers the ring is made from and turned into at the end.
+// then works without overflow, rounding its results to whole units.  It scales
+// down by 2 to 6 bits (pass_bits), so its results keep 55 to 61 bits of the
+// largest point.  Relative rms error of a ring (Nside = 256, FP64 transforms ->
+// these; white noise, and with one pixel 1e5 times the rest): adjoint 2.5e-16
+// -> 1.6e-16 and 2.4e-16 -> 1.7e-16 where K is a power of two, 2.5..2.7e-16 ->
+// 1.7..2.0e-16 with a factor 3 to 13, Rader 4.0e-16 -> 3.1e-16 and 3.9e-16 ->
+// 3.4e-16, Bluestein 4.8e-16 -> 3.7e-16; synthesis the same to 10 %.
 // Measured (Nside = 512, L = 1024, 8 maps; FP64 transforms before): ring
 // synthesis 1.80 -> .86 ms, adjoint 2.42 -> .94 ms; Nside = 1024: 7.60 ->
 // 3.76 and 9.79 -> 4.03 ms (1.14, 1.16, 3.90 and 4.12 by the change of
@@ -115,9 +119,9 @@ __device__ __forceinline__ int4 wneg_if(int4 w, bool neg)
     return neg ? make_int4(-w.x, -w.y, -w.z, -w.w) : w;
 }
 
-// a w / 4 (CONJ: a conj(w) / 4) for |a| < 2^61.5: the products of the high
+// a w / 4 (CONJ: a conj(w) / 4) for |a| < 2^62: the products of the high
 // halves, and of high and low halves over 2^32, both exact in 64 bits; those
-// of the low halves are below a quarter of a unit
+// of the low halves are below half a unit
 template <bool CONJ = false>
 __device__ __forceinline__ fx2 fmul(fx2 a, int4 w)
 {
@@ -137,6 +141,24 @@ __device__ __forceinline__ fx2 fmul(fx2 a, int4 w)
     N += (long long)bh * cl;
     N += (long long)bl * ch;
     return make_longlong2(P + (M >> 32), Q + (N >> 32));
+}
+
+// a w 2^(k - 2), 0 <= k < 32, for tables of small entries, |a w| 2^(k - 2) < 2^61.5:
+// with the low halves' products, whose upper words the result still has
+__device__ __forceinline__ fx2 fmul_up(fx2 a, int4 w, int k)
+{
+    int ah, al, bh, bl;
+    halves(a.x, ah, al);
+    halves(a.y, bh, bl);
+    long long P = (long long)ah * w.y - (long long)bh * w.w;
+    long long M = (1LL << (31 - k)) + __mulhi(al, w.x) - __mulhi(bl, w.z);
+    M += (long long)ah * w.x + (long long)al * w.y;
+    M -= (long long)bh * w.z + (long long)bl * w.w;
+    long long Q = (long long)ah * w.w + (long long)bh * w.y;
+    long long N = (1LL << (31 - k)) + __mulhi(al, w.z) + __mulhi(bl, w.x);
+    N += (long long)ah * w.z + (long long)al * w.w;
+    N += (long long)bh * w.x + (long long)bl * w.y;
+    return make_longlong2((P << k) + (M >> (32 - k)), (Q << k) + (N >> (32 - k)));
 }
 
 // bits of the largest component so far: the OR of the components' upper words
@@ -189,7 +211,7 @@ struct FxScale {
 // position order.
 
 // cos and sin of 2 pi k / R for the odd radices, k < R: R = 3, 5, 7, 11, 13
-// at offsets 0, 3, 8, 15, 26, in units of 2^-59 as {low, high} halves
+// at offsets 0, 3, 8, 15, 26
 __host__ __device__ constexpr double root_cos(int k)
 {
     constexpr double t[39] = {
@@ -224,7 +246,15 @@ __host__ __device__ constexpr double root_sin(int k)
     -4.64723172043768562e-01};
     return t[k];
 }
-__host__ __device__ constexpr long long root_fix(double x) { return (long long)(x * 0x1p59); }
+// bits by which dft_small scales down: its roots are in units of 2^-(64 -
+// bits), the finest that keep its sums of mixed halves' products below 2^63
+// (units of 2^-59 for all left the points 52 to 54 bits, fewer than FP64's 53
+// of each point)
+__host__ __device__ constexpr int dft_bits(int R) { return R == 2 || R == 4 ? 0 : R <= 5 ? 2 : R == 7 ? 3 : 4; }
+__host__ __device__ constexpr long long root_fix(double x, int R)
+{
+    return (long long)(x * (double)(1LL << (64 - dft_bits(R))));
+}
 __host__ __device__ constexpr int root_low(long long v) { return (int)(unsigned)(v & 0xffffffffLL); }
 __host__ __device__ constexpr int root_high(long long v) { return (int)((v - root_low(v)) / (1LL << 32)); }
 
@@ -232,13 +262,6 @@ template <int R>
 __device__ __forceinline__ constexpr int root_off()
 {
     return R == 3 ? 0 : R == 5 ? 3 : R == 7 ? 8 : R == 11 ? 15 : 26;
-}
-
-// bits by which dft_small scales down
-template <int R>
-__device__ __forceinline__ constexpr int dft_bits()
-{
-    return R == 2 || R == 4 ? 0 : 5;
 }
 
 // y_q = 2^-dft_bits sum_p a_p e^{S 2 pi i p q / R}, in place (S = +1 or -1),
@@ -263,8 +286,8 @@ __device__ __forceinline__ void dft_small(fx2 (&a)[R])
         // odd R: pair p with R - p, y_q = A_q + S i B_q, y_{R-q} = A_q - S i
         // B_q; A and B are sums of products with constants, each kept as the
         // sum of the high halves' products and of the mixed ones (at most 6
-        // terms below 2^60.3)
-        constexpr int H = (R - 1) / 2, O = root_off<R>();
+        // terms of 2^59.5 + 2^(63 - dft_bits))
+        constexpr int H = (R - 1) / 2, O = root_off<R>(), D = dft_bits(R);
         int sh[H][2], sl[H][2], dh[H][2], dl[H][2];
         fx2 y0 = make_longlong2(a[0].x >> 1, a[0].y >> 1);
 #pragma unroll
@@ -277,7 +300,7 @@ __device__ __forceinline__ void dft_small(fx2 (&a)[R])
             y0.x += sp.x >> 1;
             y0.y += sp.y >> 1;
         }
-        const fx2 a0 = frshift(a[0], 5);
+        const fx2 a0 = frshift(a[0], D);
 #pragma unroll
         for (int q = 1; q <= H; ++q) {
             long long A[2], B[2];
@@ -286,7 +309,7 @@ __device__ __forceinline__ void dft_small(fx2 (&a)[R])
                 long long Ph = 0, Pm = 1LL << 31, Qh = 0, Qm = 1LL << 31;
 #pragma unroll
                 for (int p = 1; p <= H; ++p) {
-                    const long long cs = root_fix(root_cos(O + (p * q) % R)), sn = root_fix(root_sin(O + (p * q) % R));
+                    const long long cs = root_fix(root_cos(O + (p * q) % R), R), sn = root_fix(root_sin(O + (p * q) % R), R);
                     Ph += (long long)sh[p - 1][c] * root_high(cs);
                     Pm += (long long)sh[p - 1][c] * root_low(cs);
                     Pm += (long long)sl[p - 1][c] * root_high(cs);
@@ -301,8 +324,17 @@ __device__ __forceinline__ void dft_small(fx2 (&a)[R])
             a[q] = make_longlong2(A[0] + iB.x, A[1] + iB.y);
             a[R - q] = make_longlong2(A[0] - iB.x, A[1] - iB.y);
         }
-        a[0] = frshift(y0, 4);
+        a[0] = frshift(y0, D - 1);
     }
+}
+
+// bits by which the results of an odd radix, which dft_small leaves below
+// 2^59.9, are shifted up before their twiddles, a product of which scales
+// down by 2 and may end at 2^61.5
+template <int R>
+__device__ __forceinline__ constexpr int twiddle_up()
+{
+    return R == 2 || R == 4 ? 0 : R == 5 ? 1 : 2;
 }
 
 // one pass of radix R over Ntot points: back-to-back sequences of Nseq
@@ -312,7 +344,7 @@ __device__ __forceinline__ void dft_small(fx2 (&a)[R])
 template <int R, bool INV>
 __device__ __forceinline__ int pass_bits(int Ns)
 {
-    return 2 + dft_bits<R>() + (!INV && Ns > 1 ? 2 : 0);
+    return 2 + dft_bits(R) + (!INV && Ns > 1 ? 2 - twiddle_up<R>() : 0);
 }
 
 template <int R, bool INV, class TW>
@@ -338,9 +370,10 @@ __device__ __forceinline__ unsigned mx_pass(fx2 *x, int Ntot, int Nseq, int B, c
         }
         dft_small<R, INV ? 1 : -1>(a);
         if (!INV && twiddled) {
-            a[0] = frshift(a[0], 2);
+            constexpr int U = twiddle_up<R>();
+            if (U < 2) a[0] = frshift(a[0], U < 2 ? 2 - U : 1);
 #pragma unroll
-            for (int p = 1; p < R; ++p) a[p] = fmul<true>(a[p], tw(p * j * step));
+            for (int p = 1; p < R; ++p) a[p] = fmul<true>(fshl(a[p], U), tw(p * j * step));
         }
 #pragma unroll
         for (int q = 0; q < R; ++q) {
@@ -351,7 +384,7 @@ __device__ __forceinline__ unsigned mx_pass(fx2 *x, int Ntot, int Nseq, int B, c
     return mag;
 }
 
-// cos and sin of 2 pi k / R in units of 2^-59 as halves {low, high, low,
+// cos and sin of 2 pi k / R in units of 2^-60 as halves {low, high, low,
 // high}, k < R, for R = 11 and 13 at root_off<R>() - 15
 struct RootTable {
     int4 v[24];
@@ -360,7 +393,7 @@ constexpr RootTable make_root_table()
 {
     RootTable t{};
     for (int i = 0; i < 24; ++i) {
-        const long long c = root_fix(root_cos(15 + i)), n = root_fix(root_sin(15 + i));
+        const long long c = root_fix(root_cos(15 + i), 13), n = root_fix(root_sin(15 + i), 13);
         t.v[i].x = root_low(c);
         t.v[i].y = root_high(c);
         t.v[i].z = root_low(n);
@@ -380,7 +413,8 @@ static __constant__ RootTable kRoots = make_root_table();
 template <int R, bool INV, class TW>
 __device__ __forceinline__ unsigned mx_pass_odd(fx2 *x, int Ntot, int Nseq, int B, const TW &tw, int s)
 {
-    constexpr int H = (R - 1) / 2, O = root_off<R>() - 15;
+    constexpr int H = (R - 1) / 2, O = root_off<R>() - 15, D = dft_bits(R), U = twiddle_up<R>();
+    static_assert(D == dft_bits(13) && U == 2, "one table of roots, no shift after the twiddles");
     const int Ns = B / R, step = Nseq / B;
     const bool twiddled = Ns > 1;
     unsigned mag = 0;
@@ -407,10 +441,10 @@ __device__ __forceinline__ unsigned mx_pass_odd(fx2 *x, int Ntot, int Nseq, int 
             y0.x += sp.x >> 1;
             y0.y += sp.y >> 1;
         }
-        y0 = frshift(y0, !INV && twiddled ? 6 : 4);
+        y0 = frshift(y0, D - 1);
         x[base] = y0;
         mag |= fmag(y0);
-        const fx2 a05 = frshift(a0, 5);
+        const fx2 a0d = frshift(a0, D);
 #pragma unroll 1
         for (int q = 1; q <= H; ++q) {
             long long Ph[2] = {0, 0}, Pm[2] = {1LL << 31, 1LL << 31}, Qh[2] = {0, 0}, Qm[2] = {1LL << 31, 1LL << 31};
@@ -430,13 +464,13 @@ __device__ __forceinline__ unsigned mx_pass_odd(fx2 *x, int Ntot, int Nseq, int 
                     Qm[c] += (long long)dl[p][c] * w.w;
                 }
             }
-            const fx2 A = make_longlong2(a05.x + Ph[0] + (Pm[0] >> 32), a05.y + Ph[1] + (Pm[1] >> 32));
+            const fx2 A = make_longlong2(a0d.x + Ph[0] + (Pm[0] >> 32), a0d.y + Ph[1] + (Pm[1] >> 32));
             const fx2 Bv = make_longlong2(Qh[0] + (Qm[0] >> 32), Qh[1] + (Qm[1] >> 32));
             const fx2 iB = INV ? ftimes_i(Bv) : make_longlong2(Bv.y, -Bv.x);
             fx2 y = fadd(A, iB), z = fsub(A, iB);
             if (!INV && twiddled) {
-                y = fmul<true>(y, tw(q * j * step));
-                z = fmul<true>(z, tw((R - q) * j * step));
+                y = fmul<true>(fshl(y, U), tw(q * j * step));
+                z = fmul<true>(fshl(z, U), tw((R - q) * j * step));
             }
             x[base + q * Ns] = y;
             x[base + (R - q) * Ns] = z;
@@ -554,6 +588,10 @@ struct TwTable {
     __device__ __forceinline__ int4 operator()(int t) const { return __ldg(R + t); }
 };
 
+// fmul_up's bits for a filter of M points: its entries are below 1.7 / sqrt(M)
+// (checked for every K up to 4096), and 2^(bits - 2) <= sqrt(M) / 2
+__device__ __forceinline__ int blue_up(int M) { return (33 - __clz(M)) / 2; }
+
 // x[0..K) holds the input, zeros follow up to M; computes x[n] =
 // sum_k x_k e^{2 pi i k n / K} for n < K through Bluestein's chirp transform:
 // a cyclic convolution of length M (smooth, >= 2K - 1) with the chirp filter,
@@ -564,14 +602,14 @@ __device__ __forceinline__ void bluestein_mx(fx2 *x, int M, const int4 *__restri
                                              const TwTable &tw, FxScale &sc)
 {
     fft_mx_dif<false>(x, M, M, rl, tw, sc);
-    const int s = sc.enter();
+    const int s = sc.enter(), up = blue_up(M);
     unsigned mag = 0;
     for (int k = threadIdx.x; k < M; k += blockDim.x) {
-        const fx2 y = fmul(fshl(x[k], s), __ldg(fb + k));
+        const fx2 y = fmul_up(fshl(x[k], s), __ldg(fb + k), up);
         x[k] = y;
         mag |= fmag(y);
     }
-    sc.e += 2;
+    sc.e += 2 - up;
     sc.leave(mag);
     fft_mx_dit<false>(x, M, M, rl, tw, sc);
 }
@@ -596,7 +634,9 @@ __device__ __forceinline__ fx2 frescale(fx2 a, int from, int to)
 // the product's zero frequency, and y_0 = a_0 + (sum of alpha) is that
 // frequency before the product.  Exponent +1; CONJ = true gives exponent -1
 // as conj(DFT(conj a)).  The a_0 stay in the units they have when the pass
-// begins; at the end all points are in the convolution's units.
+// begins; at the end all points are in the convolution's units.  The stored
+// transform has modulus sqrt(p) / (p - 1) (1 / (p - 1) at zero), so that
+// products without the bits fmul_up keeps would end at 2^52 for p = 1000.
 struct RaderRun {
     RaderCtx c;
     RaderInfo ri;
@@ -622,32 +662,32 @@ struct RaderRun {
         sc.leave(mag);
     }
 
-    // y_0 (and a_0 with the product) may need as many more bits as a_0 has
-    // above the rest: both sides at a quarter of their size, in the larger units
+    // y_0 has units of its own, in which it and its two terms fit, and so has
+    // the product with a_0
     template <bool CONJ>
     __device__ __forceinline__ void product(fx2 *x, FxScale &sc)
     {
         const int4 *__restrict__ G = c.tab + ri.G;
         fx2 *S = c.scratch;
-        const int s1 = sc.enter();
-        e1 = max(sc.e, e0) + 2;
+        const int s1 = sc.enter(), up = (33 - __clz(ri.n)) / 2;    // 2^(up - 2) sqrt(p) / n <= .52
+        const int ec = sc.e + 2 - up, e2 = max(ec, e0) + 2;
+        e1 = max(sc.e, e0) + 1;
         unsigned mag = 0;
         for (int e = threadIdx.x; e < tot; e += blockDim.x) {
             const int b = e / ri.n, v = e - b * ri.n;
-            const fx2 A = frescale(fshl(S[e], s1), sc.e, e1);
-            fx2 C = fmul(A, __ldg(G + v));             // e1 + 2
+            const fx2 A = fshl(S[e], s1);
+            fx2 C = frescale(fmul_up(A, __ldg(G + v), up), ec, e2);
             if (v == 0) {
-                fx2 a0 = frescale(CONJ ? fconj(x[b * ri.p]) : x[b * ri.p], e0, e1);
-                fx2 y0 = fadd(a0, A);
+                const fx2 a0 = CONJ ? fconj(x[b * ri.p]) : x[b * ri.p];
+                C = fadd(C, frescale(a0, e0, e2));
+                fx2 y0 = fadd(frescale(a0, e0, e1), frescale(A, sc.e, e1));
                 if (CONJ) y0 = fconj(y0);
-                x[b * ri.p] = y0;                      // in units of 2^e1
-                mag |= fmag(frshift(y0, 2));
-                C = fadd(C, frshift(a0, 2));
+                x[b * ri.p] = y0;
             }
             S[e] = C;
             mag |= fmag(C);
         }
-        sc.e = e1 + 2;
+        sc.e = e2;
         sc.leave(mag);
     }
 
