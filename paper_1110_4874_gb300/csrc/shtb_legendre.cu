@@ -19,22 +19,25 @@
 // lets lane = j sum over the tile's rings.
 //
 // The recurrence runs in FP64; the sums over the maps, 2 NB of them a value
-// of V, are integer (LegSums): V and the a or g of a chain are cut to limbs
+// of V, are integer (LegSums): V and the a or g of a run of 32 are cut to limbs
 // at common exponents, and a product is three 32-bit multiply-adds.  The FP64
 // pipe, which takes a warp's DFMA in 16 clocks of an SM against half a clock
 // for an integer multiply-add, held these kernels with both done in FP64.
 // Legendre stage, FP64 sums -> this (ms):
-//   nside 64, lmax 128, 1 map      synthesis  .047 -> .028  adjoint  .054 -> .037
-//   nside 100, lmax 255, 1 map                .095 -> .051           .140 -> .068
-//   nside 256, lmax 512, 4 maps               .996 -> .418          1.385 -> .555
-//   nside 256, lmax 512, 8 maps              1.730 -> .711          2.416 -> .931
-//   nside 512, lmax 1024, 8 maps             12.22 -> 4.89          13.94 -> 5.48
+//   nside 64, lmax 128, 1 map      synthesis  .047 -> .031  adjoint  .054 -> .038
+//   nside 100, lmax 255, 1 map                .095 -> .056           .140 -> .070
+//   nside 256, lmax 512, 4 maps               .996 -> .443          1.385 -> .566
+//   nside 256, lmax 512, 8 maps              1.730 -> .766          2.416 -> .989
+//   nside 512, lmax 1024, 8 maps             12.22 -> 5.15          13.94 -> 5.93
 // What bounds them now is issue (48 % of the slots with 8 maps, the FP64 pipe
 // at 31 %) and, with few maps, the chain of dependent FMAs of the recurrence.
-// The sums keep 55 bits of a or g below the largest of a chain and 58 of V,
-// and end no further from the exact transform than sums of FMAs: over nside
-// 32..1024 both are 9.5e-16 .. 2.8e-14 of the result's norm away, which is the
-// recurrence's own rounding.
+// Precision: a or g are cut 49 bits or more below a run's largest, V 55 to 58
+// below its largest so far, the products of low limbs left out; a run whose
+// sizes differ enough for that to be less than FP64 keeps is summed in FP64.
+// So each ring and each coefficient is as close to the recurrence's values as
+// an FP64 sum of its terms, also beside much larger ones (one exponent for a
+// whole chain, .42 and .55 ms at nside 256 with 4 maps, left 1e-9 of
+// coefficients beside polar pixels 1e8 times the rest).
 #include <cuda_runtime.h>
 
 #include "shtb_internal.h"
@@ -77,9 +80,18 @@ __global__ void alm_prescale_kernel(PlanView v, const double2 *__restrict__ alm,
     }
 }
 
-// Range of effective exponents the integer sums take, for the a of a chain
-// (per component) and for the V of a ring (the recurrence starts at 1e-30)
-constexpr int kLegExpLo = 300, kLegExpHi = 1700;
+// What a run's integer sums take; other runs are summed in FP64 (plain_steps,
+// plain_rings).  Limbs are cut at one place for the whole run, and V grows
+// along a chain from the crop on, so a run whose large values meet a small V
+// and whose small ones a large V would lose what FP64 keeps: its largest
+// exponent lies in a range, every four neighbours have one at most kLegDrop
+// bits below any before them, the last two one at most kLegLast, and it has
+// kLegShort entries or more.
+constexpr int kLegExpLo = 300, kLegExpHi = 1700, kLegDrop = 7, kLegLast = 10, kLegShort = 8;
+// A component's scale, the exponent its limbs are cut at, is set a bit above
+// the largest of the run that needs it and kept for the runs whose largest
+// lies at it or up to kLegKeep bits below.
+constexpr int kLegKeep = 5;
 
 // Bits of V, so that sums of n products of 55-bit a and V fit: between two
 // carries 32 products of 27-bit by 30-bit high limbs stay below 2^62, and the
@@ -89,56 +101,98 @@ __device__ __forceinline__ int v_bits(int n)
     return 58 - max(0, 32 - __clz(n) - 13);
 }
 
-// The values of one chain that a warp's sums weight: `count` entries of C
-// components, entry i at src + i stride (doubles).  scan: the largest
-// exponent of each component over all of them, kept by lanes b < NB for
-// components 2b, 2b + 1 (0: zero; -1: take the component in FP64).
-template <int NB>
-__device__ __forceinline__ int2 scan_chain(const double *src, size_t stride, int count, int lane)
+// 1 for subnormals, 0 for zeros alone
+__device__ __forceinline__ unsigned exp_of(double v)
 {
-    constexpr int STEP = 32 / NB;
-    const int b = lane % NB, r = lane / NB;
-    int e0 = 0, e1 = 0;
-    unsigned nz0 = 0, nz1 = 0;
-#pragma unroll 4
-    for (int i = r; i < count; i += STEP) {
-        const double2 x = __ldg(reinterpret_cast<const double2 *>(src + (size_t)i * stride) + b);
-        e0 = max(e0, shtb_dev::exp_bits(x.x));
-        e1 = max(e1, shtb_dev::exp_bits(x.y));
-        nz0 |= (unsigned)__double2hiint(x.x) << 1 | (unsigned)__double2loint(x.x);
-        nz1 |= (unsigned)__double2hiint(x.y) << 1 | (unsigned)__double2loint(x.y);
-    }
-#pragma unroll
-    for (int o = NB; o < 32; o *= 2) {
-        e0 = max(e0, __shfl_xor_sync(0xffffffffu, e0, o));
-        e1 = max(e1, __shfl_xor_sync(0xffffffffu, e1, o));
-        nz0 |= __shfl_xor_sync(0xffffffffu, nz0, o);
-        nz1 |= __shfl_xor_sync(0xffffffffu, nz1, o);
-    }
-    if (e0 < kLegExpLo || e0 > kLegExpHi) e0 = nz0 ? -1 : 0;
-    if (e1 < kLegExpLo || e1 > kLegExpHi) e1 = nz1 ? -1 : 0;
-    return make_int2(e0, e1);
+    const unsigned u = (unsigned)__double2hiint(v) << 1 | (__double2loint(v) != 0 ? 1u : 0u);
+    return max(u >> 21, min(u, 1u));
 }
 
-// ... and entries [0, count) of them (at most 32) as limbs of 55 bits in lim
+// A run is the up to 32 values of a chain that a warp's sums weight next, of C
+// components each, entry i at src + i stride (doubles).  Components 2b, 2b + 1
+// belong to the lanes of b = lane mod NB, which hold entries r + q STEP, r =
+// lane / NB.
 template <int NB>
-__device__ __forceinline__ void chain_limbs(const double *src, size_t stride, int count, int2 e, int2 *lim, int lane)
-{
-    constexpr int STEP = 32 / NB;
-    const int b = lane % NB, r = lane / NB;
-    int4 *lim4 = reinterpret_cast<int4 *>(lim);
-#pragma unroll 2
-    for (int i = r; i < count; i += STEP) {
-        const double2 x = __ldg(reinterpret_cast<const double2 *>(src + (size_t)i * stride) + b);
-        const int2 l0 = e.x > 0 ? shtb_dev::to_limbs(x.x, 9 + e.x - shtb_dev::exp_bits(x.x)) : make_int2(0, 0);
-        const int2 l1 = e.y > 0 ? shtb_dev::to_limbs(x.y, 9 + e.y - shtb_dev::exp_bits(x.y)) : make_int2(0, 0);
-        lim4[i * NB + b] = make_int4(l0.x, l0.y, l1.x, l1.y);
+struct Run {
+    static constexpr int STEP = 32 / NB;
+    double2 x[NB];
+    __device__ __forceinline__ void load(const double *src, size_t stride, int count, int lane)
+    {
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+            const int i = q * STEP + lane / NB;
+            x[q] = i < count ? __ldg(reinterpret_cast<const double2 *>(src + (size_t)i * stride) + lane % NB)
+                             : make_double2(0.0, 0.0);
+        }
     }
+    // the largest exponent: 0 for a component of zeros, -1 for one to take in FP64
+    __device__ __forceinline__ int2 scan(int count, int lane) const
+    {
+        unsigned top = 0, drop = 0, last = 0;                        // two components in halves
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+            unsigned e = exp_of(x[q].x) | exp_of(x[q].y) << 16;      // of the four entries 4 (i / 4) ..
+            e = __vmaxu2(e, __shfl_xor_sync(0xffffffffu, e, NB));
+            if (q == (count - 1) / STEP) last = e;
+            e = __vmaxu2(e, __shfl_xor_sync(0xffffffffu, e, 2 * NB));
+            unsigned before = e;                                     // the largest up to them
+#pragma unroll
+            for (int o = 4 * NB; o < 32; o *= 2) {
+                const unsigned y = __shfl_up_sync(0xffffffffu, before, o);
+                if (lane >= o) before = __vmaxu2(before, y);
+            }
+            before = __vmaxu2(before, top);
+            if (((q * STEP + lane / NB) & ~3) < count) drop = __vmaxu2(drop, before - e);
+            top = NB == 8 ? before : __shfl_sync(0xffffffffu, before, 32 - NB + lane % NB);
+        }
+#pragma unroll
+        for (int o = 4 * NB; o < 32; o *= 2) drop = __vmaxu2(drop, __shfl_xor_sync(0xffffffffu, drop, o));
+        last = top - __shfl_sync(0xffffffffu, last, (count - 1) % STEP * NB + lane % NB);
+        auto one = [count](int e, int below, int end) {
+            return e == 0 ? 0 : e < kLegExpLo || e > kLegExpHi || below > kLegDrop || end > kLegLast || count < kLegShort ? -1 : e;
+        };
+        return make_int2(one(top & 0xffff, drop & 0xffff, last & 0xffff), one(top >> 16, drop >> 16, last >> 16));
+    }
+    // limbs of 55 bits at the scales of the components that e takes
+    __device__ __forceinline__ void limbs(int2 e, int2 scale, int2 *lim, int lane) const
+    {
+        int4 *lim4 = reinterpret_cast<int4 *>(lim);
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+            const int2 l0 = e.x > 0 ? shtb_dev::to_limbs(x[q].x, 9 + scale.x - shtb_dev::exp_bits(x[q].x)) : make_int2(0, 0);
+            const int2 l1 = e.y > 0 ? shtb_dev::to_limbs(x[q].y, 9 + scale.y - shtb_dev::exp_bits(x[q].y)) : make_int2(0, 0);
+            lim4[(q * STEP + lane / NB) * NB + lane % NB] = make_int4(l0.x, l0.y, l1.x, l1.y);
+        }
+    }
+};
+
+// entries of the next run of `left`: 32, or 24 where 32 would leave a short one
+__device__ __forceinline__ int run_length(int left)
+{
+    return left > 32 && left < 32 + kLegShort ? 32 - kLegShort : min(32, left);
+}
+
+// the scale for a run of largest exponent e: none where the run adds nothing
+// in integers, so that a sum is never moved to a V it has no products of
+__device__ __forceinline__ int next_scale(int scale, int e)
+{
+    return e <= 0 ? 0 : e <= scale && e >= scale - kLegKeep ? scale : e + 1;
+}
+
+__device__ __forceinline__ bool scale_left(int2 scale, int2 next)
+{
+    return (scale.x != 0 && scale.x != next.x) || (scale.y != 0 && scale.y != next.y);
+}
+
+// component c's of a pair on the lanes of b
+__device__ __forceinline__ int of_component(int2 v, int c)
+{
+    return __shfl_sync(0xffffffffu, c & 1 ? v.y : v.x, c >> 1);
 }
 
 // A warp's 32 running sums (one a lane) per component, on a common exponent E
 // of the V seen so far (0: none yet) with up to kHead bits to spare, so that a
-// growing V raises it only now and then: value (H 2^68 + P 2^28 + M) 2^28 2^(e_a + E - ..)
+// growing V raises it only now and then: value (H 2^68 + P 2^28 + M) 2^28 2^(scale + E - ..)
 constexpr int kHead = 3;
 // chain steps between two looks at E (one for every map count: the same bits)
 constexpr int kStep = 4;
@@ -204,6 +258,7 @@ struct LegSums {
             P[c] &= (1LL << 40) - 1;
         }
     }
+    __device__ __forceinline__ void drop(int c) { P[c] = M[c] = H[c] = 0; }
     // after a carry; a = X_a 2^(e_a - 1077), V = X_V 2^(E - 1022 - vb)
     __device__ __forceinline__ double value(int c, int ea) const
     {
@@ -234,18 +289,32 @@ struct Chain {
     }
 };
 
-// The sum of one component by FP64 FMAs along the recurrence, for chains
-// whose a hold an infinity, a NaN or extreme magnitudes
-__device__ __noinline__ double plain_chain_sum(const RecCoef *cf, const double *a, size_t stride, int jlo, int n,
-                                               Chain ch)
+// The products of the next `count` steps' V with the components (e < 0) that
+// integers do not take, in FP64; a: their first entry, component c's sum at
+// sum[32 c]
+template <int NB>
+__device__ __noinline__ void plain_steps(double v0, double v1, double v2, double v3, const double *a, size_t stride,
+                                         int count, int2 e, double *sum)
 {
-    double s = 0.0;
-    ch.begin(jlo);
-    for (int j = jlo; j < n; ++j) {
-        s = fma(a[(size_t)j * stride], ch.cur, s);
-        ch.step(j, cf[2 * j]);
+    static_assert(kStep == 4, "four steps");
+    const double V[kStep] = {v0, v1, v2, v3};
+    const unsigned pairs = __ballot_sync(0xffffffffu, min(e.x, e.y) < 0);
+#pragma unroll 1
+    for (int b = 0; b < NB; ++b) {
+        if (!(pairs >> b & 1)) continue;
+        double2 x[kStep], s = make_double2(sum[64 * b], sum[64 * b + 32]);
+#pragma unroll
+        for (int i = 0; i < kStep; ++i)
+            x[i] = __ldg(reinterpret_cast<const double2 *>(a + (size_t)min(i, count - 1) * stride) + b);
+#pragma unroll
+        for (int i = 0; i < kStep; ++i)
+            if (i < count) {
+                s.x = fma(x[i].x, V[i], s.x);
+                s.y = fma(x[i].y, V[i], s.y);
+            }
+        if (of_component(e, 2 * b) < 0) sum[64 * b] = s.x;
+        if (of_component(e, 2 * b + 1) < 0) sum[64 * b + 32] = s.y;
     }
-    return s;
 }
 
 // One warp per (m, 32 half-rings, parity); the two parities of a (m, rings)
@@ -258,6 +327,7 @@ legendre_synth_kernel(PlanView v, const double2 *__restrict__ ap, double2 *__res
 {
     constexpr int C = 2 * NB;
     __shared__ __align__(16) int2 slim[kWarpsPerBlock][32 * C];
+    __shared__ double ssum[kWarpsPerBlock][C][32];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int Z = v.nhalf, L = v.lmax;
@@ -273,9 +343,9 @@ legendre_synth_kernel(PlanView v, const double2 *__restrict__ ap, double2 *__res
     const int n = there ? dchain_len(L, m, t) : 0;
     int2 *lim = slim[warp];
 
-    double acc[C];
+    double *sum = &ssum[warp][0][lane];                                // component c at sum[32 c]
 #pragma unroll
-    for (int c = 0; c < C; ++c) acc[c] = 0.0;
+    for (int c = 0; c < C; ++c) sum[32 * c] = 0.0;
     Chain ch;
     ch.x = v.xarg[rr];
     ch.sform = v.xform[rr] != 0;
@@ -288,14 +358,31 @@ legendre_synth_kernel(PlanView v, const double2 *__restrict__ ap, double2 *__res
         const RecCoef *__restrict__ cf = v.coef + off;                // step j at cf[2 j]
         const double *a = reinterpret_cast<const double *>(ap + (size_t)off * nmaps + b0);
         const size_t stride = (size_t)4 * nmaps;                      // doubles between chain entries
-        const int2 ea = scan_chain<NB>(a + (size_t)jlo * stride, stride, n - jlo, lane);
         LegSums<C> sums;
         sums.clear(n);
+        int2 scale = make_int2(0, 0);
+        // integer sums so far, of the components whose next scale is another, into sum
+        auto settle = [&](int2 next) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const int e = of_component(scale, c);
+                if (e == 0 || e == of_component(next, c)) continue;
+                sum[32 * c] += sums.value(c, e);
+                sums.drop(c);
+            }
+        };
         ch.begin(jlo);
-        for (int jb = jlo; jb < n; jb += 32) {
-            const int nj = min(32, n - jb);
+        for (int jb = jlo, nj; jb < n; jb += nj) {
+            nj = run_length(n - jb);
+            Run<NB> run;
+            run.load(a + (size_t)jb * stride, stride, nj, lane);
+            const int2 ea = run.scan(nj, lane);
+            const bool plain = __any_sync(0xffffffffu, min(ea.x, ea.y) < 0);
+            const int2 next = make_int2(next_scale(scale.x, ea.x), next_scale(scale.y, ea.y));
+            if (__any_sync(0xffffffffu, scale_left(scale, next))) settle(next);
+            scale = next;
             __syncwarp();
-            chain_limbs<NB>(a + (size_t)jb * stride, stride, nj, ea, lim, lane);
+            run.limbs(ea, scale, lim, lane);
             __syncwarp();
             for (int i0 = 0; i0 < nj; i0 += kStep) {
                 double V[kStep];
@@ -313,32 +400,24 @@ legendre_synth_kernel(PlanView v, const double2 *__restrict__ ap, double2 *__res
 #pragma unroll
                 for (int i = 0; i < kStep; ++i)
                     if (i0 + i < nj) sums.add(V[i], lim + (i0 + i) * C);
+                if (plain)
+                    plain_steps<NB>(V[0], V[1], V[2], V[3], a + (size_t)(jb + i0) * stride, stride, nj - i0, ea, sum);
             }
             sums.carry();
         }
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-            const int e = __shfl_sync(0xffffffffu, c & 1 ? ea.y : ea.x, c >> 1);
-            acc[c] = sums.value(c, e);
-            if (e < 0) acc[c] = plain_chain_sum(cf, a + c, stride, jlo, n, ch);
-        }
+        settle(make_int2(-1, -1));
     }
 
     // q(+z) = q^0 + q^1 by the even warp, q(-z) = q^0 - q^1 by the odd one
     __syncthreads();
-    double *trade = reinterpret_cast<double *>(lim);                   // [C][32]
-#pragma unroll
-    for (int c = 0; c < C; ++c) trade[c * 32 + lane] = acc[c];
-    __syncthreads();
     if (!valid || (t == 1 && r == Z - 1)) return;                      // the equator ring has no mirror
-    const double *other = reinterpret_cast<const double *>(slim[warp ^ 1]);
+    const double *other = &ssum[warp ^ 1][0][lane];
     const int ring = t == 0 ? r : v.nrings - 1 - r;
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
-        const double ox = other[2 * b * 32 + lane], oy = other[(2 * b + 1) * 32 + lane];
+        const double x = sum[64 * b], y = sum[64 * b + 32], ox = other[64 * b], oy = other[64 * b + 32];
         q[((size_t)(b0 + b) * v.nrings + ring) * (L + 1) + m] =
-            t == 0 ? make_double2(acc[2 * b] + ox, acc[2 * b + 1] + oy)
-                   : make_double2(ox - acc[2 * b], oy - acc[2 * b + 1]);
+            t == 0 ? make_double2(x + ox, y + oy) : make_double2(ox - x, oy - y);
     }
 }
 
@@ -396,30 +475,38 @@ __host__ __device__ constexpr size_t adjoint_warp_smem_doubles()
     return 32 * kTilePad + 32 * 2 * NB;
 }
 
-// One component's a_j = sum_r V_j(r) g_r of a chain in FP64, by one warp
-// (lane = ring), for chains whose g hold an infinity, a NaN or extreme
-// magnitudes.  dst: the component in aacc, entry j at dst + j dstride.
-__device__ __noinline__ void plain_chain_adjoint(const PlanView &v, int m, int t, const double *gc, size_t gstride,
-                                                 double *dst, size_t dstride, int lane)
+// most chunks of rings a warp takes
+__host__ __device__ constexpr int adjoint_warp_chunks(int nchunk, int W) { return (nchunk + W / 2 - 1) / (W / 2); }
+
+// A run of rings' products with the components (e < 0) that integers do not
+// take, in FP64, lane = chain step; rings whose V is cropped there are left
+// out.  buf: 32 double2 of the warp's
+template <int NB>
+__device__ __noinline__ void plain_rings(const double *row, const double *g, size_t stride, int count, int2 e,
+                                         double2 *buf, double *acc, int lane)
 {
-    const int Z = v.nhalf, n = dchain_len(v.lmax, m, t);
-    const RecCoef *cf = v.coef + dalm_index(v.lmax, m, m) + t;
-    for (int c0 = 0; c0 < Z; c0 += 32) {
-        const int r = c0 + lane, rr = min(r, Z - 1);
-        const size_t base = ((size_t)m * 2 + t) * Z + rr;
-        Chain ch;
-        ch.x = v.xarg[rr];
-        ch.sform = v.xform[rr] != 0;
-        ch.js = r < Z ? v.jstart[base] : n;
-        ch.start = v.vstart[base];
-        const double gv = r < Z ? gc[(size_t)rr * gstride] : 0.0;
-        ch.begin(0);
-        for (int j = 0; j < n; ++j) {
-            double s = r < Z && j >= ch.js ? ch.cur * gv : 0.0;
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) dst[(size_t)j * dstride] = c0 ? dst[(size_t)j * dstride] + s : s;
-            ch.step(j, cf[2 * j]);
-        }
+    const unsigned pairs = __ballot_sync(0xffffffffu, min(e.x, e.y) < 0);
+#pragma unroll 1
+    for (int b = 0; b < NB; ++b) {
+        if (!(pairs >> b & 1)) continue;
+        __syncwarp();
+        buf[lane] = lane < count ? __ldg(reinterpret_cast<const double2 *>(g + (size_t)lane * stride) + b) : make_double2(0.0, 0.0);
+        __syncwarp();
+        double2 s[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s[i] = make_double2(0.0, 0.0);
+#pragma unroll 1
+        for (int r = 0; r < 32; r += 4)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const double v = row[r + i];
+                const double2 x = buf[r + i];
+                const bool there = exp_of(v) != 0;
+                s[i].x = fma(v, there ? x.x : 0.0, s[i].x);
+                s[i].y = fma(v, there ? x.y : 0.0, s[i].y);
+            }
+        if (of_component(e, 2 * b) < 0) acc[2 * b] += (s[0].x + s[1].x) + (s[2].x + s[3].x);
+        if (of_component(e, 2 * b + 1) < 0) acc[2 * b + 1] += (s[0].y + s[1].y) + (s[2].y + s[3].y);
     }
 }
 
@@ -445,13 +532,35 @@ legendre_adjoint_kernel(PlanView v, const double2 *__restrict__ g, double2 *__re
     double2 *st = reinterpret_cast<double2 *>(state + (size_t)blockIdx.x * Z) + t;   // ring r at st[2 r]
     const double *gm = reinterpret_cast<const double *>(g + ((size_t)m * 2 + t) * Z * nmaps + b0);
     const size_t gstride = (size_t)2 * nmaps;                         // doubles between rings
-    const int2 eg = scan_chain<NB>(gm, gstride, Z, lane);
     const int ntiles = (n0 + 31) >> 5;
+    // the largest exponents of this warp's runs of g: chunk set + i W/2 at se[i NB + b]
+    short2 *se = reinterpret_cast<short2 *>(smd + (size_t)W * adjoint_warp_smem_doubles<NB>()) +
+               (size_t)warp * adjoint_warp_chunks(nchunk, W) * NB;
+    for (int c = set, i = 0; c < nchunk; c += W / 2, ++i) {
+        Run<NB> run;
+        run.load(gm + (size_t)c * 32 * gstride, gstride, min(32, Z - c * 32), lane);
+        const int2 e = run.scan(min(32, Z - c * 32), lane);
+        if (lane < NB) se[i * NB + lane] = make_short2((short)e.x, (short)e.y);
+    }
+    __syncwarp();
 
     for (int ti = 0; ti < ntiles; ++ti) {
         const int jt = ti * 32;
         LegSums<C> sums;
         sums.clear(Z);
+        int2 scale = make_int2(0, 0);
+        double acc[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) acc[c] = 0.0;
+        auto settle = [&](int2 next) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const int e = of_component(scale, c);
+                if (e == 0 || e == of_component(next, c)) continue;
+                acc[c] += sums.value(c, e);
+                sums.drop(c);
+            }
+        };
         for (int c = set; c < nchunk && jt < n; c += W / 2) {
             const int r = c * 32 + lane;
             const bool valid = r < Z;
@@ -477,7 +586,16 @@ legendre_adjoint_kernel(PlanView v, const double2 *__restrict__ g, double2 *__re
                 if (j < n) ch.step(j, cf[2 * j]);
             }
             if (valid) st[2 * r] = make_double2(ch.cur, ch.prev);
-            chain_limbs<NB>(gm + (size_t)c * 32 * gstride, gstride, min(32, Z - c * 32), eg, lim, lane);
+            const double *gc = gm + (size_t)c * 32 * gstride;
+            const int nr = min(32, Z - c * 32);
+            const short2 es = se[(c - set) / (W / 2) * NB + lane % NB];
+            const int2 eg = make_int2(es.x, es.y);
+            const int2 next = make_int2(next_scale(scale.x, eg.x), next_scale(scale.y, eg.y));
+            if (__any_sync(0xffffffffu, scale_left(scale, next))) settle(next);
+            scale = next;
+            Run<NB> run;
+            run.load(gc, gstride, nr, lane);
+            run.limbs(eg, scale, lim, lane);
             __syncwarp();
             // lane = chain step: sum over the tile's 32 rings (those past the last have V = 0)
             const double *row = tile + lane * kTilePad;
@@ -488,15 +606,14 @@ legendre_adjoint_kernel(PlanView v, const double2 *__restrict__ g, double2 *__re
 #pragma unroll 4
             for (int r2 = 0; r2 < 32; ++r2) sums.add(row[r2], lim + r2 * C);
             sums.carry();
+            if (__any_sync(0xffffffffu, min(eg.x, eg.y) < 0)) plain_rings<NB>(row, gc, gstride, nr, eg, reinterpret_cast<double2 *>(lim), acc, lane);
             __syncwarp();
         }
+        settle(make_int2(-1, -1));
         // add the warps' partial sums of each parity and store them
         double *mine = tile;                            // [C][32], rows of 33
 #pragma unroll
-        for (int c = 0; c < C; ++c) {
-            const int e = __shfl_sync(0xffffffffu, c & 1 ? eg.y : eg.x, c >> 1);
-            mine[c * kTilePad + lane] = sums.value(c, e);
-        }
+        for (int c = 0; c < C; ++c) mine[c * kTilePad + lane] = acc[c];
         __syncthreads();
         for (int i = threadIdx.x; i < 2 * 32 * NB; i += blockDim.x) {
             const int tt = i / (32 * NB), rem = i - tt * 32 * NB;
@@ -514,12 +631,6 @@ legendre_adjoint_kernel(PlanView v, const double2 *__restrict__ g, double2 *__re
         }
         __syncthreads();
     }
-    if (set == 0 && n > 0)
-        for (int c = 0; c < C; ++c)
-            if (__shfl_sync(0xffffffffu, c & 1 ? eg.y : eg.x, c >> 1) < 0)
-                plain_chain_adjoint(v, m, t, gm + c, gstride,
-                                    reinterpret_cast<double *>(aacc + (size_t)(off + t) * nmaps + b0) + c,
-                                    (size_t)4 * nmaps, lane);
 }
 
 // alm[b][idx] = c_m sigma_idx aacc[idx][b], c_0 = 1 (Im a_l0 = 0), c_m = 2
@@ -544,7 +655,8 @@ template <int NB, int W>
 int launch_adjoint_nb(const shtb_plan_s *p, const double2 *g, double2 *aacc, RecState *state,
                       int nmaps, int b0, cudaStream_t st)
 {
-    const size_t smem = sizeof(double) * adjoint_warp_smem_doubles<NB>() * W;
+    const size_t smem = sizeof(double) * adjoint_warp_smem_doubles<NB>() * W +
+                        sizeof(short2) * NB * W * adjoint_warp_chunks((p->nhalf + 31) / 32, W);
     SHTB_CUDA_TRY(cudaFuncSetAttribute(legendre_adjoint_kernel<NB, W>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     legendre_adjoint_kernel<NB, W><<<p->lmax + 1, 32 * W, smem, st>>>(p->view, g, aacc, state,
