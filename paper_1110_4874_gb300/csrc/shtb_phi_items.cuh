@@ -878,25 +878,31 @@ __device__ __forceinline__ void phi_synth_ring_at(const PlanView &v, int ring, Q
         emax = max(emax, f >> 20);
     };
     // A short ring folds many terms onto few k (J = 4: L / 2 each): up to 32
-    // neighbouring threads then share one k's terms
+    // neighbouring threads then share one k's terms, as many as kFoldThreads
+    // gives each k, whatever the block's size: the sums, and so the maps, are
+    // the same bits in the ring kernels (128 to 512 threads) and in the batch
+    // kernel (32 a warp of its schedule)
+    constexpr int kFoldThreads = 128;
     int parts = 1;
-    while (parts < 32 && 2 * parts * K <= (int)blockDim.x) parts *= 2;
+    while (parts < 32 && 2 * parts * K <= kFoldThreads) parts *= 2;
     if (parts == 1) {
         for (int k = threadIdx.x; k < K; k += blockDim.x) pack(k, fold_G(qat, L, J, s, k), fold_G(qat, L, J, s, k + K));
     } else {
-        const int k = threadIdx.x / parts, part = threadIdx.x & (parts - 1);
-        double2 G0 = make_double2(0.0, 0.0), G1 = G0;
-        if (k < K) {
-            G0 = fold_part(qat, L, J, s, k, part, parts);
-            G1 = fold_part(qat, L, J, s, k + K, part, parts);
+        for (int i = threadIdx.x; i < ((K * parts + 31) & ~31); i += blockDim.x) {    // whole warps
+            const int k = i / parts, part = i & (parts - 1);
+            double2 G0 = make_double2(0.0, 0.0), G1 = G0;
+            if (k < K) {
+                G0 = fold_part(qat, L, J, s, k, part, parts);
+                G1 = fold_part(qat, L, J, s, k + K, part, parts);
+            }
+            for (int o = 1; o < parts; o *= 2) {
+                G0.x += __shfl_xor_sync(0xffffffffu, G0.x, o);
+                G0.y += __shfl_xor_sync(0xffffffffu, G0.y, o);
+                G1.x += __shfl_xor_sync(0xffffffffu, G1.x, o);
+                G1.y += __shfl_xor_sync(0xffffffffu, G1.y, o);
+            }
+            if (k < K && part == 0) pack(k, G0, G1);
         }
-        for (int o = 1; o < parts; o *= 2) {
-            G0.x += __shfl_xor_sync(0xffffffffu, G0.x, o);
-            G0.y += __shfl_xor_sync(0xffffffffu, G0.y, o);
-            G1.x += __shfl_xor_sync(0xffffffffu, G1.x, o);
-            G1.y += __shfl_xor_sync(0xffffffffu, G1.y, o);
-        }
-        if (k < K && part == 0) pack(k, G0, G1);
     }
     emax = (int)__reduce_max_sync(0xffffffffu, (unsigned)emax);
     any = __reduce_or_sync(0xffffffffu, any);
