@@ -496,15 +496,11 @@ int check_spin(shtb_plan p, const void *a, const void *b, int npairs, const char
 template <class Plus, class Minus>
 int both_operators(shtb_plan_s *q, cudaStream_t st, Plus plus, Minus minus)
 {
-    int rc;
-    if ((rc = side_streams(q))) return rc;
-    SHTB_CUDA_TRY(cudaEventRecord(q->ring_ev[0], st));
-    SHTB_CUDA_TRY(cudaStreamWaitEvent(q->ring_stream[0], q->ring_ev[0], 0));
-    rc = minus(q->ring_stream[0]);
-    if (!rc) rc = plus(st);
-    SHTB_CUDA_TRY(cudaEventRecord(q->ring_ev[1], q->ring_stream[0]));
-    SHTB_CUDA_TRY(cudaStreamWaitEvent(st, q->ring_ev[1], 0));
-    return rc;
+    if (int rc = side_streams(q)) return rc;
+    return fork_join(st, q->ring_stream, q->ring_ev, 1, [&] {
+        const int rc = minus(q->ring_stream[0]);
+        return rc ? rc : plus(st);
+    });
 }
 
 // E, B of every pair -> Q, U (2 npairs inputs and maps)
@@ -638,7 +634,10 @@ int shtb_synthesize_host(shtb_plan p, const double *alm_host, double *map_host, 
         // compressed plans: the maps come back ring chunk by ring chunk,
         // overlapping the rest of the ring stage
         if (p->profiling) ++p->prof_calls;
-        if ((rc = launch_bf_synth_to_host(p, w.alm, w.ap, w.bf, w.map, map_host, nmaps, st))) return rc;
+        if ((rc = launch_bf_synth_to_host(p, w.alm, w.ap, w.bf, w.map, map_host, nmaps, st))) {
+            cudaStreamSynchronize(st);             // no copy into the caller's buffer outlives the call
+            return rc;
+        }
     } else {
         if ((rc = run_synthesis(p, w.alm, w.map, nmaps, st))) return rc;
         SHTB_CUDA_TRY(cudaMemcpyAsync(map_host, w.map, sizeof(double) * (size_t)nmaps * p->npix,

@@ -573,23 +573,18 @@ int enqueue_graph(shtb_batch_s *b, cudaStream_t st)
     int rc;
     for (auto &P : b->gg)
         if ((rc = launch_bf_gather(P.plan, P.alm_tab, P.ai, P.columns, st))) return rc;
-    // fork: every side stream starts after the gathers
-    SHTB_CUDA_TRY(cudaEventRecord(b->fork_join[0], st));
-    for (int s = 1; s < b->nstreams; ++s) SHTB_CUDA_TRY(cudaStreamWaitEvent(b->side[s - 1], b->fork_join[0], 0));
-    for (auto &P : b->gg) {
-        for (auto &M : P.mgs) {
-            cudaStream_t ss = M.stream == 0 ? st : b->side[M.stream - 1];
-            if ((rc = launch_bf_legendre_group(P.plan, P.ai, P.columns, M.b0, M.nb, M.u0, M.u1, M.qt, ss)))
-                return rc;
-            if ((rc = launch_phi_synth_qt_ptr(P.plan, M.qt, M.real, P.map_tab, M.b0, ss))) return rc;
+    // every side stream starts after the gathers
+    return fork_join(st, b->side.data(), b->fork_join.data(), b->nstreams - 1, [&] {
+        for (auto &P : b->gg) {
+            for (auto &M : P.mgs) {
+                cudaStream_t ss = M.stream == 0 ? st : b->side[M.stream - 1];
+                if ((rc = launch_bf_legendre_group(P.plan, P.ai, P.columns, M.b0, M.nb, M.u0, M.u1, M.qt, ss)))
+                    return rc;
+                if ((rc = launch_phi_synth_qt_ptr(P.plan, M.qt, M.real, P.map_tab, M.b0, ss))) return rc;
+            }
         }
-    }
-    // join
-    for (int s = 1; s < b->nstreams; ++s) {
-        SHTB_CUDA_TRY(cudaEventRecord(b->fork_join[s], b->side[s - 1]));
-        SHTB_CUDA_TRY(cudaStreamWaitEvent(st, b->fork_join[s], 0));
-    }
-    return SHTB_OK;
+        return (int)SHTB_OK;
+    });
 }
 
 int enqueue(shtb_batch_s *b, cudaStream_t st)

@@ -634,30 +634,32 @@ int launch_bf_synth_to_host(shtb_plan_s *p, const double2 *alm, double2 *ai, voi
                                                                  p->bf->rec ? p->view.coef : nullptr);
     SHTB_CUDA_TRY(cudaGetLastError());
     ++p->launches;
-    for (int b0 = 0; b0 < columns;) {
+    int rc = SHTB_OK;
+    for (int b0 = 0; b0 < columns && !rc;) {
         const int nb = group_width(columns - b0), real = std::min(nb, nmaps - b0);
         const QtView qt{qt_ws, qt_pack(nb)};
-        int rc = launch_bf_legendre_group(p, ai, columns, b0, nb, u0, u1, qt, st);
-        if (rc) return rc;
+        rc = launch_bf_legendre_group(p, ai, columns, b0, nb, u0, u1, qt, st);
         // ring stage chunk by chunk; each chunk's pixels go back while the
         // next chunk (or the next map group) computes
-        for (int c = 0; c < NCH; ++c) {
-            if ((rc = launch_phi_synth_qt_chunk(p, qt, real, map, b0, c, st))) return rc;
+        auto copy_back = [&](int c) -> int {
             const long long p0 = p->chunk_pix[c], p1 = p->chunk_pix[c + 1];
-            if (p1 == p0) continue;
-            SHTB_CUDA_TRY(cudaEventRecord(p->chunk_ev[c], st));
-            SHTB_CUDA_TRY(cudaStreamWaitEvent(p->copy_stream, p->chunk_ev[c], 0));
+            if (p1 == p0) return SHTB_OK;
+            if (int bad = join_stream(p->copy_stream, st, p->chunk_ev[c])) return bad;
             for (int b = b0; b < b0 + real; ++b)
                 SHTB_CUDA_TRY(cudaMemcpyAsync(map_host + (size_t)b * p->npix + p0, map + (size_t)b * p->npix + p0,
                                               sizeof(double) * (size_t)(p1 - p0), cudaMemcpyDeviceToHost,
                                               p->copy_stream));
+            return SHTB_OK;
+        };
+        for (int c = 0; c < NCH && !rc; ++c) {
+            rc = launch_phi_synth_qt_chunk(p, qt, real, map, b0, c, st);
+            if (!rc) rc = copy_back(c);
         }
         b0 += nb;
     }
-    // the caller's stream completes after the last copy
-    SHTB_CUDA_TRY(cudaEventRecord(p->chunk_ev[0], p->copy_stream));
-    SHTB_CUDA_TRY(cudaStreamWaitEvent(st, p->chunk_ev[0], 0));
-    return SHTB_OK;
+    // the caller's stream completes after the last copy, also when a launch failed
+    const int joined = join_stream(st, p->copy_stream, p->chunk_ev[0]);
+    return rc ? rc : joined;
 }
 
 int launch_bf_adjoint(const shtb_plan_s *p, const double2 *g, double2 *aacc, void *ws, double2 *alm,

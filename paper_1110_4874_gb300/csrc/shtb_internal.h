@@ -32,6 +32,33 @@ struct NvtxRange {
                              std::string(#expr) + ": " + cudaGetErrorString(e_));      \
     } while (0)
 
+// st waits for what s2 holds so far
+inline int join_stream(cudaStream_t st, cudaStream_t s2, cudaEvent_t ev)
+{
+    SHTB_CUDA_TRY(cudaEventRecord(ev, s2));
+    SHTB_CUDA_TRY(cudaStreamWaitEvent(st, ev, 0));
+    return SHTB_OK;
+}
+
+// n side streams forked from st, body() enqueues on st and on them, and they
+// are joined to st again -- also when a launch in body fails, so that nothing
+// enqueued before it outlives the caller's order.  ev: n + 1 events
+template <class Body>
+int fork_join(cudaStream_t st, const cudaStream_t *side, const cudaEvent_t *ev, int n, Body body)
+{
+    SHTB_CUDA_TRY(cudaEventRecord(ev[0], st));
+    int rc = SHTB_OK, forked = 0;
+    for (; forked < n && !rc; ++forked)
+        if (cudaError_t e = cudaStreamWaitEvent(side[forked], ev[0], 0))
+            rc = shtb_fail(SHTB_ECUDA, std::string("forking a stream: ") + cudaGetErrorString(e));
+    if (!rc) rc = body();
+    for (int i = 0; i < forked; ++i) {
+        const int joined = join_stream(st, side[i], ev[1 + i]);
+        if (!rc) rc = joined;
+    }
+    return rc;
+}
+
 // ------------------------------------------------------------ plan layout
 // Index of coefficient (l, m) in the m-major a_lm layout.
 inline long long alm_index(int lmax, int l, int m)

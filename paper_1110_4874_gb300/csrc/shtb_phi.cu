@@ -182,15 +182,11 @@ int side_by_side(const shtb_plan_s *p, cudaStream_t st, Blue blue, Direct direct
 {
     shtb_plan_s *pp = const_cast<shtb_plan_s *>(p);
     if (int rs = side_streams(pp)) return rs;
-    SHTB_CUDA_TRY(cudaEventRecord(pp->ring_ev[0], st));
-    for (cudaStream_t s2 : pp->ring_stream) SHTB_CUDA_TRY(cudaStreamWaitEvent(s2, pp->ring_ev[0], 0));
-    int rc;
-    if ((rc = blue(st)) || (rc = direct(pp->ring_stream[0])) || (rc = big(pp->ring_stream[1]))) return rc;
-    for (int i = 0; i < 2; ++i) {
-        SHTB_CUDA_TRY(cudaEventRecord(pp->ring_ev[1 + i], pp->ring_stream[i]));
-        SHTB_CUDA_TRY(cudaStreamWaitEvent(st, pp->ring_ev[1 + i], 0));
-    }
-    return SHTB_OK;
+    return fork_join(st, pp->ring_stream, pp->ring_ev, 2, [&] {
+        int rc = blue(st);
+        if (!rc) rc = direct(pp->ring_stream[0]);
+        return rc ? rc : big(pp->ring_stream[1]);
+    });
 }
 
 int launch_set(const shtb_plan_s *p, bool synth, const void *in, void *out, int nmaps,
