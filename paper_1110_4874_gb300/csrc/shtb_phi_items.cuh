@@ -23,8 +23,9 @@
 // arithmetic alone).  What bounds them now is the issue of integer
 // instructions at the direct lengths (65 to 71 % of the slots) and latency
 // and instruction fetches at the others (36 to 49 %, 16 warps an SM).
-// Rings whose values hold an infinity or a NaN, or lie outside 1e-217 ..
-// 1e204, are summed directly in FP64 (ring_direct_*), as such values spread.
+// Rings whose largest value lies outside 1e-217 .. 1e204 are brought into that
+// range by a power of two; rings that hold an infinity or a NaN are filled with
+// NaN.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -818,53 +819,46 @@ struct RingAux {
     unsigned any;
 };
 
-// Range of the block exponent that the fixed-point path takes
-constexpr int kRingExpLo = 300, kRingExpHi = 1700;
+// Range of the block exponent that the fixed-point path takes, and the power
+// of two that brings any other finite one into it: values above it are only
+// renamed (their units), values below it are lifted first (subnormals among
+// them); either way the results are scaled back
+constexpr int kRingExpLo = 300, kRingExpHi = 1700, kRingLift = 600;
 
-// the ring's direct sum in FP64, for values the fixed-point path does not take
-template <class QAt>
-__device__ __noinline__ void ring_direct_synth(const int4 *T, int J, int s, int L, QAt qat, double *out)
+__device__ __forceinline__ double2 scaled(double2 z, int n)
 {
-    for (int j = threadIdx.x; j < J; j += blockDim.x) {
-        double f = qat(0).x;
-        for (int m = 1; m <= L; ++m) {
-            const int k = (int)(((long long)m * (2 * j + s)) % (2 * J));
-            const double2 w = ring_unfix(T[k < J ? k : k - J], k >= J), q = qat(m);
-            f += 2.0 * (q.x * w.x - q.y * w.y);
-        }
-        out[j] = f;
-    }
+    const double f = shtb::pow2(n);
+    return make_double2(z.x * f, z.y * f);
 }
 
-// Pixels of one ring from its q_m (m = 0..L): fold (Eq. tau) and pack the
-// Hermitian spectrum into a half-length complex FFT in one step,
-// Z_k = G_k A_k + G_{k+K} B_k (the plan's fold weights A, B hold the phi_0
-// phase, the packing twiddle and, on Bluestein rings, the chirp), transform,
-// and write f_{2n}, f_{2n+1} as the real and imaginary parts of z_n.  The
-// fold's sums are FP64; each Z_k is formed in fixed point with its own
-// exponent, and once the largest is known all are brought to it.  All threads
-// of the block take part; sm holds the transform's entries (K direct, K plus
-// the Rader scratch, M Bluestein) and K 16-bit exponents after them.
-template <int KIND, class QAt>
-__device__ __forceinline__ void phi_synth_ring_at(const PlanView &v, int ring, QAt qat, double *out_ring, fx2 *sm)
+// out[0 .. n) of a ring of zeros or (a value is not finite) of NaN
+__device__ __forceinline__ void ring_fill(double2 *out, int n, bool zero)
 {
-    constexpr bool BLUE = KIND == kBluestein, BIG = KIND == kDirectBig;
-    __shared__ RingAux aux;
-    const int L = v.lmax;
-    const int J = v.ring_J[ring], K = J / 2, s = v.ring_s[ring];
-    const int4 *__restrict__ T = ring_table(v.tw) + v.ring_tw[ring];
-    const int4 *__restrict__ AB = ring_table(v.ab) + v.ring_ab[ring];
-    const int *__restrict__ rl = v.rad + v.ring_rad[ring];
-    RaderCtx rc;
-    const RaderCtx *rcp = BIG ? rader_ctx(v, ring, K, sm, rc) : nullptr;
-    const int M = BLUE ? v.ring_mx[ring] : 0;
-    const int entries = BLUE ? M : BIG && rcp ? K + (K / rcp->ri->p) * rcp->ri->n : K;
-    short *ex = reinterpret_cast<short *>(sm + entries);
-    if (threadIdx.x == 0) aux = RingAux{{0, 0, 0}, 0, 0};
+    const double f = zero ? 0.0 : __longlong_as_double(0x7ff8000000000000LL);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) out[i] = make_double2(f, f);
     __syncthreads();
+}
+
+__device__ __forceinline__ void ring_scale_back(double2 *out, int n, int lift)
+{
+    for (int i = threadIdx.x; i < n; i += blockDim.x) out[i] = scaled(out[i], -lift);
+}
+
+// The fold of a ring's spectrum: entry k at sm, in units 2^(f - 1080), and f
+// in ex, at the transform's position of k; the largest f and whether any value
+// is not zero in aux.  LIFT: of 2^kRingLift times the spectrum.
+template <bool BLUE, bool LIFT, class QAt>
+__device__ __forceinline__ void ring_fold(QAt qat, int L, int J, int s, const int4 *__restrict__ AB,
+                                          const int *__restrict__ rl, fx2 *sm, short *ex, RingAux &aux)
+{
+    const int K = J / 2;
     int emax = 0;
     unsigned any = 0;
     auto pack = [&](int k, double2 G0, double2 G1) {
+        if (LIFT) {
+            G0 = scaled(G0, kRingLift);
+            G1 = scaled(G1, kRingLift);
+        }
         const int f = max(max(exp_field(G0.x), exp_field(G0.y)), max(exp_field(G1.x), exp_field(G1.y)));
         any |= nonzero_bits(G0.x) | nonzero_bits(G0.y) | nonzero_bits(G1.x) | nonzero_bits(G1.y);
         const int f3 = f + (3 << 20);
@@ -873,7 +867,7 @@ __device__ __forceinline__ void phi_synth_ring_at(const PlanView &v, int ring, Q
         const fx2 X1 = make_longlong2(ring_fix(G1.x, (f3 - exp_field(G1.x)) >> 20),
                                       ring_fix(G1.y, (f3 - exp_field(G1.y)) >> 20));
         const int pos = BLUE ? k : fft_pos(k, K, rl);
-        sm[pos] = fadd(fmul(X0, __ldg(AB + 2 * k)), fmul(X1, __ldg(AB + 2 * k + 1)));    // units 2^(f - 1080)
+        sm[pos] = fadd(fmul(X0, __ldg(AB + 2 * k)), fmul(X1, __ldg(AB + 2 * k + 1)));
         ex[pos] = (short)(f >> 20);
         emax = max(emax, f >> 20);
     };
@@ -910,19 +904,63 @@ __device__ __forceinline__ void phi_synth_ring_at(const PlanView &v, int ring, Q
         atomicMax(&aux.emax, emax);
         atomicOr(&aux.any, any);
     }
+}
+
+template <bool BLUE, class QAt>
+__device__ __noinline__ void ring_fold_lifted(QAt qat, int L, int J, int s, const int4 *AB, const int *rl,
+                                              fx2 *sm, short *ex, RingAux &aux)
+{
+    ring_fold<BLUE, true>(qat, L, J, s, AB, rl, sm, ex, aux);
+}
+
+// Pixels of one ring from its q_m (m = 0..L): fold (Eq. tau) and pack the
+// Hermitian spectrum into a half-length complex FFT in one step,
+// Z_k = G_k A_k + G_{k+K} B_k (the plan's fold weights A, B hold the phi_0
+// phase, the packing twiddle and, on Bluestein rings, the chirp), transform,
+// and write f_{2n}, f_{2n+1} as the real and imaginary parts of z_n.  The
+// fold's sums are FP64; each Z_k is formed in fixed point with its own
+// exponent, and once the largest is known all are brought to it.  All threads
+// of the block take part; sm holds the transform's entries (K direct, K plus
+// the Rader scratch, M Bluestein) and K 16-bit exponents after them.
+template <int KIND, class QAt>
+__device__ __forceinline__ void phi_synth_ring_at(const PlanView &v, int ring, QAt qat, double *out_ring, fx2 *sm)
+{
+    constexpr bool BLUE = KIND == kBluestein, BIG = KIND == kDirectBig;
+    __shared__ RingAux aux;
+    const int L = v.lmax;
+    const int J = v.ring_J[ring], K = J / 2, s = v.ring_s[ring];
+    const int4 *__restrict__ T = ring_table(v.tw) + v.ring_tw[ring];
+    const int4 *__restrict__ AB = ring_table(v.ab) + v.ring_ab[ring];
+    const int *__restrict__ rl = v.rad + v.ring_rad[ring];
+    RaderCtx rc;
+    const RaderCtx *rcp = BIG ? rader_ctx(v, ring, K, sm, rc) : nullptr;
+    const int M = BLUE ? v.ring_mx[ring] : 0;
+    const int entries = BLUE ? M : BIG && rcp ? K + (K / rcp->ri->p) * rcp->ri->n : K;
+    short *ex = reinterpret_cast<short *>(sm + entries);
+    if (threadIdx.x == 0) aux = RingAux{{0, 0, 0}, 0, 0};
     __syncthreads();
-    emax = aux.emax;
+    ring_fold<BLUE, false>(qat, L, J, s, AB, rl, sm, ex, aux);
+    __syncthreads();
+    int emax = aux.emax, lift = 0, renamed = 0;
     double2 *out = reinterpret_cast<double2 *>(out_ring);
     if (emax < kRingExpLo || emax > kRingExpHi) {
-        if (!aux.any) {
-            for (int n = threadIdx.x; n < K; n += blockDim.x) out[n] = make_double2(0.0, 0.0);
-        } else {
-            ring_direct_synth(T, J, s, L, qat, out_ring);
+        if (emax == 0x7ff || !aux.any) {
+            ring_fill(out, K, emax != 0x7ff);
+            return;
         }
-        __syncthreads();
-        return;
+        lift = emax < kRingExpLo ? kRingLift : -kRingLift;
+        if (lift < 0) {
+            renamed = lift;
+        } else {
+            __syncthreads();
+            if (threadIdx.x == 0) aux.emax = 0;
+            __syncthreads();
+            ring_fold_lifted<BLUE>(qat, L, J, s, AB, rl, sm, ex, aux);
+            __syncthreads();
+            emax = aux.emax;
+        }
     }
-    FxScale sc{aux.slot, 0, emax - 1080};
+    FxScale sc{aux.slot, 0, emax + renamed - 1080};
     unsigned mag = 0;
     for (int p = threadIdx.x; p < (BLUE ? M : K); p += blockDim.x) {
         if (BLUE && p >= K) {
@@ -945,6 +983,7 @@ __device__ __forceinline__ void phi_synth_ring_at(const PlanView &v, int ring, Q
         if (BLUE) z = fmul(z, ring_root(T, J, 2 * n * n));
         out[n] = make_double2(fix_to_double(z.x, be), fix_to_double(z.y, be));
     }
+    if (lift) ring_scale_back(out, K, lift);
     __syncthreads();
 }
 
@@ -974,7 +1013,46 @@ __device__ __forceinline__ void phi_synth_ring_qt(const PlanView &v, int ring, c
     phi_synth_ring_at<KIND>(v, ring, qat, out_ring, sm);
 }
 
-static __device__ __noinline__ void ring_direct_adjoint(const int4 *T, int J, int s, int L, const double *f, double2 *outq);
+// A ring's pixels as points of exponent emax (2^20 times it): z_n in units of
+// 2^(emax - 1083), with the chirp on Bluestein rings; returns their size
+template <bool BLUE>
+__device__ __forceinline__ unsigned ring_load(const double2 *in, int K, int M, const int4 *__restrict__ T, int J,
+                                              int emax, int lift, fx2 *sm)
+{
+    const int e3 = emax + (3 << 20);
+    unsigned mag = 0;
+    for (int n = threadIdx.x; n < (BLUE ? M : K); n += blockDim.x) {
+        if (BLUE && n >= K) {
+            sm[n] = make_longlong2(0, 0);
+            continue;
+        }
+        double2 zd = __ldg(in + n);
+        if (lift) zd = scaled(zd, lift);
+        fx2 z = make_longlong2(ring_fix(zd.x, (e3 - exp_field(zd.x)) >> 20), ring_fix(zd.y, (e3 - exp_field(zd.y)) >> 20));
+        if (BLUE) z = fmul(fconj(z), ring_root(T, J, 2 * n * n));    // forward = conj(inverse(conj))
+        sm[n] = z;
+        mag |= fmag(z);
+    }
+    return mag;
+}
+
+// ... of 2^kRingLift times the pixels, whose largest exponent is left in aux
+template <bool BLUE>
+__device__ __noinline__ unsigned ring_load_lifted(const double2 *in, int K, int M, const int4 *T, int J, RingAux &aux, fx2 *sm)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) aux.emax = 0;
+    __syncthreads();
+    int emax = 0;
+    for (int n = threadIdx.x; n < K; n += blockDim.x) {
+        const double2 z = scaled(in[n], kRingLift);
+        emax = max(emax, max(exp_field(z.x), exp_field(z.y)));
+    }
+    emax = (int)__reduce_max_sync(0xffffffffu, (unsigned)emax);
+    if ((threadIdx.x & 31) == 0) atomicMax(&aux.emax, emax);
+    __syncthreads();
+    return ring_load<BLUE>(in, K, M, T, J, aux.emax, kRingLift, sm);
+}
 
 // Adjoint of one ring: q_adj[m] = sum_j f_j e^{-i m phi_j}, m = 0..L, from
 // z_n = f_{2n} + i f_{2n+1}, Zf = DFT(z) with exponent -1 (position order, or
@@ -996,7 +1074,7 @@ __device__ __forceinline__ void phi_adjoint_ring(const PlanView &v, int ring, co
     if (threadIdx.x == 0) aux = RingAux{{0, 0, 0}, 0, 0};
     __syncthreads();
     const double2 *in = reinterpret_cast<const double2 *>(f_ring);
-    int emax = 0;
+    int emax = 0, lift = 0;
     unsigned any = 0;
     for (int n = threadIdx.x; n < K; n += blockDim.x) {
         const double2 z = __ldg(in + n);
@@ -1011,28 +1089,21 @@ __device__ __forceinline__ void phi_adjoint_ring(const PlanView &v, int ring, co
     }
     __syncthreads();
     emax = aux.emax;
-    if (emax < kRingExpLo << 20 || emax > kRingExpHi << 20) {
-        if (!aux.any) {
-            for (int m = threadIdx.x; m <= L; m += blockDim.x) outq[m] = make_double2(0.0, 0.0);
-        } else {
-            ring_direct_adjoint(T, J, s, L, f_ring, outq);
-        }
-        __syncthreads();
-        return;
-    }
-    FxScale sc{aux.slot, 0, (emax >> 20) - 1083};
-    const int e3 = emax + (3 << 20);
     unsigned mag = 0;
-    for (int n = threadIdx.x; n < (BLUE ? M : K); n += blockDim.x) {
-        if (BLUE && n >= K) {
-            sm[n] = make_longlong2(0, 0);
-            continue;
+    FxScale sc{aux.slot, 0, 0};
+    if (emax < kRingExpLo << 20 || emax > kRingExpHi << 20) {
+        if (emax == 0x7ff00000 || !aux.any) {
+            ring_fill(outq, L + 1, emax != 0x7ff00000);
+            return;
         }
-        const double2 zd = __ldg(in + n);
-        fx2 z = make_longlong2(ring_fix(zd.x, (e3 - exp_field(zd.x)) >> 20), ring_fix(zd.y, (e3 - exp_field(zd.y)) >> 20));
-        if (BLUE) z = fmul(fconj(z), ring_root(T, J, 2 * n * n));    // forward = conj(inverse(conj))
-        sm[n] = z;
-        mag |= fmag(z);
+        lift = emax < kRingExpLo << 20 ? kRingLift : -kRingLift;
+    }
+    if (lift <= 0) {
+        sc.e = (emax >> 20) + lift - 1083;
+        mag = ring_load<BLUE>(in, K, M, T, J, emax, 0, sm);
+    } else {
+        mag = ring_load_lifted<BLUE>(in, K, M, T, J, aux, sm);
+        sc.e = (aux.emax >> 20) - 1083;
     }
     if (BLUE) sc.e += 2;
     sc.leave(mag);
@@ -1066,21 +1137,8 @@ __device__ __forceinline__ void phi_adjoint_ring(const PlanView &v, int ring, co
         if (s) F = fmul<true>(F, ring_root(T, J, m));
         outq[m] = make_double2(fix_to_double(F.x, be), fix_to_double(F.y, be));
     }
+    if (lift) ring_scale_back(outq, L + 1, lift);
     __syncthreads();
-}
-
-static __device__ __noinline__ void ring_direct_adjoint(const int4 *T, int J, int s, int L, const double *f, double2 *outq)
-{
-    for (int m = threadIdx.x; m <= L; m += blockDim.x) {
-        double2 q = make_double2(0.0, 0.0);
-        for (int j = 0; j < J; ++j) {
-            const int k = (int)(((long long)m * (2 * j + s)) % (2 * J));
-            const double2 w = ring_unfix(T[k < J ? k : k - J], k >= J);
-            q.x += f[j] * w.x;
-            q.y -= f[j] * w.y;
-        }
-        outq[m] = q;
-    }
 }
 
 }  // namespace shtb_dev

@@ -36,11 +36,5 @@ __device__ __forceinline__ int2 ring_half_pack(double v, int bits)
 
 __device__ __forceinline__ const int4 *ring_table(const double2 *p) { return reinterpret_cast<const int4 *>(p); }
 
-__device__ __forceinline__ double2 ring_unfix(int4 w, bool neg)
-{
-    const double s = neg ? -0x1p-62 : 0x1p-62;
-    return make_double2((double)((long long)w.y * 4294967296LL + w.x) * s, (double)((long long)w.w * 4294967296LL + w.z) * s);
-}
-
 }  // namespace shtb_dev
 #endif
