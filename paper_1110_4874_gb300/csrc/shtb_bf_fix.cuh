@@ -39,8 +39,7 @@
 //
 // Results do not depend on the other components, on how maps are grouped or
 // on the lane layout: the sums are exact, and chunks of 32 are added in FP64
-// in order.  A component whose chunk holds an infinity or a NaN is taken by a
-// plain FP64 loop (fix_slow_dot), so such values spread as they would in FP64.
+// in order.  A component whose chunk holds an infinity or a NaN gives NaN.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -129,11 +128,20 @@ __device__ __forceinline__ void vec_digits(uint2 a, uint2 b, unsigned (&h)[6])
     h[5] = f16_field(__byte_perm(a.x, b.x, 0x5410));
 }
 
-// Chunk exponents the fast path takes (effective, biased): results and all
-// intermediate shifts then stay in range.  Others -- an all-zero component,
-// one holding an infinity or a NaN, magnitudes below 1e-217 or above 1e204 --
-// go through fix_plain (zeros: zero digits).
-constexpr int kFixExpLo = 300, kFixExpHi = 1700;
+// Chunk exponents the digits are made at (effective, biased): results and all
+// intermediate shifts then stay in range.  A component of magnitudes below
+// 1e-217 or above 1e204 is brought there by 2^+-kFixLift and its outputs
+// brought back; one that is not finite gets zero digits and its outputs NaN.
+constexpr int kFixExpLo = 300, kFixExpHi = 1700, kFixLift = 600;
+// what a component's outputs need (two bits): nothing, 2^-kFixLift, 2^kFixLift, NaN
+enum { kFixAsIs = 0, kFixLifted = 1, kFixLowered = 2, kFixNaN = 3 };
+
+__device__ __forceinline__ double fix_after(double v, int what)
+{
+    if (what == kFixAsIs) return v;
+    return v * (what == kFixLifted ? shtb::pow2(-kFixLift) : what == kFixLowered ? shtb::pow2(kFixLift)
+                                                                               : __longlong_as_double(0x7ff8000000000000LL));
+}
 
 // The sums of the six diagonals, V = sum_d acc_d 2^{10 (5 - d)}, without
 // their low 8 bits (2^-62 of the largest possible sum): |V| < 2^71
@@ -175,48 +183,49 @@ __device__ __forceinline__ double fix_to_double(long long Y, int be0)
 // A vector's chunk is digitised by pairs of entries (2i, 2i + 1), W components
 // of each on a lane.  NP pairs a lane: raw values in, 2^20 x the largest
 // exponent of each component out; reduce(e) takes the maximum over the lanes
-// that share a component.  Components outside the fast path's range get zero
-// digits and, unless they are zero, their bit in `plain`.
+// that share a component.  Components outside the digits' range are brought
+// into it and what their outputs need is left in `after`, two bits each.
 template <bool EXPN, int NP, int W, class Max>
-__device__ __forceinline__ void vec_scale(double (&raw)[NP][2][W], const int (&sh)[NP][2], int (&ev)[W], int &plain,
+__device__ __forceinline__ void vec_scale(double (&raw)[NP][2][W], const int (&sh)[NP][2], int (&ev)[W], int &after,
                                           const Max &reduce)
 {
-#pragma unroll
-    for (int c = 0; c < W; ++c) {
-        int e = -(1 << 30), er = 0;
+    auto largest = [&](int c, int &field) {
+        int e = -(1 << 30);
+        field = 0;
 #pragma unroll
         for (int q = 0; q < NP; ++q)
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
                 const int f = __double2hiint(raw[q][p][c]) & 0x7ff00000;
-                if (EXPN) e = max(e, f);
-                else {
-                    e = max(e, f + sh[q][p]);
-                    er = max(er, f);
-                }
+                e = max(e, EXPN ? f : f + sh[q][p]);
+                if (!EXPN) field = max(field, f);
             }
-        ev[c] = reduce(e);
-        if (!EXPN && reduce(er) == 0x7ff00000) ev[c] = 0x7ff00000;
-    }
-    plain = 0;
+        return reduce(e);
+    };
     bool rare = false;
 #pragma unroll
-    for (int c = 0; c < W; ++c) rare |= ev[c] < kFixExpLo << 20 || ev[c] > kFixExpHi << 20;
+    for (int c = 0; c < W; ++c) {
+        int field;
+        ev[c] = largest(c, field);
+        if (!EXPN && reduce(field) == 0x7ff00000) ev[c] = 0x7ff00000;
+        rare |= ev[c] < kFixExpLo << 20 || ev[c] > kFixExpHi << 20;
+    }
+    after = 0;
     if (!__any_sync(0xffffffffu, rare)) return;
 #pragma unroll
     for (int c = 0; c < W; ++c) {
-        unsigned nz = 0;
+        const bool in = ev[c] >= kFixExpLo << 20 && ev[c] <= kFixExpHi << 20, finite = ev[c] != 0x7ff00000;
+        const bool low = ev[c] < kFixExpLo << 20;
+        const double f = in ? 1.0 : shtb::pow2(low ? kFixLift : -kFixLift);
+        int field, e;
 #pragma unroll
         for (int q = 0; q < NP; ++q)
 #pragma unroll
-            for (int p = 0; p < 2; ++p)
-                nz |= (unsigned)__double2hiint(raw[q][p][c]) << 1 | (unsigned)__double2loint(raw[q][p][c]);
-        nz = (unsigned)reduce(nz ? 1 : 0);
-        if (ev[c] >= kFixExpLo << 20 && ev[c] <= kFixExpHi << 20) continue;
-        if (nz) plain |= 1 << c;
-        ev[c] = kFixExpLo << 20;
-#pragma unroll
-        for (int q = 0; q < NP; ++q) raw[q][0][c] = raw[q][1][c] = 0.0;
+            for (int p = 0; p < 2; ++p) raw[q][p][c] = finite ? raw[q][p][c] * f : 0.0;
+        e = largest(c, field);
+        const bool zero = e < kFixExpLo << 20;                       // (a lifted value lies above it)
+        if (!in) after |= (!finite ? kFixNaN : zero ? kFixAsIs : low ? kFixLifted : kFixLowered) << 2 * c;
+        ev[c] = zero ? kFixExpLo << 20 : e;
     }
 }
 
@@ -228,28 +237,6 @@ __device__ __forceinline__ void vec_pair(double v0, double v1, int sh0, int sh1,
     const uint2 x0 = vec_fix(v0, (EXPN ? e7 - f0 : e7 - f0 - sh0) >> 20);
     const uint2 x1 = vec_fix(v1, (EXPN ? e7 - f1 : e7 - f1 - sh1) >> 20);
     vec_digits(x0, x1, h);
-}
-
-// The components of the mask `plain` over entries [k0, k1): FP64 FMAs from
-// zero, in order, added to the zeros the fast path left.
-template <int C, class Vec, class Out>
-__device__ __forceinline__ void fix_plain(const uint2 *T, int sk, int sn, int k0, int k1, int nn, const Vec &vec,
-                                          const Out &out, int plain, int lane)
-{
-    __syncwarp();
-#pragma unroll 1
-    for (int i = lane; i < nn * C; i += 32) {
-        const int n = i / C, c = i - n * C;
-        if (!(plain >> c & 1)) continue;
-        double v[1] = {0.0};
-#pragma unroll 1
-        for (int k = k0; k < k1; ++k) {
-            const uint2 w = T[(size_t)k * sk + (size_t)n * sn];
-            v[0] = fma(shtb::fix_unpack((unsigned long long)w.y << 32 | w.x), vec.value(k, c), v[0]);
-        }
-        out.put(out.key(n), true, c, v);
-    }
-    __syncwarp();
 }
 
 // One chunk of kc entries from k0 on, NG = ceil(kc / 8) groups of 8: the
@@ -279,7 +266,7 @@ __device__ __forceinline__ void fix_chunk_wide(const uint2 *__restrict__ T, int 
     };
     load_words(0);
     unsigned A[NS][6][4];                                            // digit fragments of the k16 (or k8) steps
-    int ev[2], plain;                                                // chunk exponents, 2^20 e
+    int ev[2], after;                                                // chunk exponents, 2^20 e
     {
         double raw[NG][2][2];
         int sh[NG][2];                                               // 2^20 x the entry's own exponent
@@ -295,7 +282,7 @@ __device__ __forceinline__ void fix_chunk_wide(const uint2 *__restrict__ T, int 
                     if (!EXPN) sh[q][p] = vec.shift(k0 + k) << 20;
                 }
             }
-        vec_scale<EXPN>(raw, sh, ev, plain, [](int e) {
+        vec_scale<EXPN>(raw, sh, ev, after, [](int e) {
             e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
             return max(e, __shfl_xor_sync(0xffffffffu, e, 2));
         });
@@ -309,6 +296,7 @@ __device__ __forceinline__ void fix_chunk_wide(const uint2 *__restrict__ T, int 
                 for (int j = 0; j < 6; ++j) A[q >> 1][j][(q & 1) * 2 + c] = h[j];
             }
     }
+    const bool rare = __any_sync(0xffffffffu, after != 0);
     for (int n0 = 0; n0 < nn; n0 += 8) {
         // where the tile's outputs go is looked up before the products
         int key[2];
@@ -338,23 +326,26 @@ __device__ __forceinline__ void fix_chunk_wide(const uint2 *__restrict__ T, int 
         }
         // columns 2t and 2t + 1 of the tile; the column's exponent comes
         // from the lane that loaded its words
+        int E[2];
 #pragma unroll
-        for (int x = 0; x < 2; ++x) {
-            const int E = EXPN ? __shfl_sync(0xffffffffu, Eg, (2 * t + x) * 4) : 0;
-            if (n0 + 2 * t + x >= nn) continue;
-            double v[2];
+        for (int x = 0; x < 2; ++x) E[x] = EXPN ? __shfl_sync(0xffffffffu, Eg, (2 * t + x) * 4) : 0;
+        auto finish = [&](auto back) {
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const int f = x + 2 * c;
-                const long long Y = fix_combine(acc[0][f], acc[1][f], acc[2][f], acc[3][f], acc[4][f], acc[5][f]);
-                v[c] = fix_to_double(Y, E + (ev[c] >> 20) + (1054 - 1079));
+            for (int x = 0; x < 2; ++x) {
+                if (n0 + 2 * t + x >= nn) continue;
+                double v[2];
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    const int f = x + 2 * c;
+                    const long long Y = fix_combine(acc[0][f], acc[1][f], acc[2][f], acc[3][f], acc[4][f], acc[5][f]);
+                    v[c] = back(fix_to_double(Y, E[x] + (ev[c] >> 20) + (1054 - 1079)), c);
+                }
+                out.put(key[x], k0 > 0, g, v);
             }
-            out.put(key[x], k0 > 0, g, v);
-        }
+        };
+        if (!rare) finish([](double v, int) { return v; });
+        else finish([after](double v, int c) { return fix_after(v, after >> 2 * c & 3); });
     }
-    if (__any_sync(0xffffffffu, plain != 0))
-        fix_plain<C>(T, sk, sn, k0, k0 + kc, nn, vec, out, (int)__reduce_or_sync(0xffffffffu, (unsigned)plain << 2 * g),
-                     lane);
 }
 
 // 2, 4 or 8 components: 16 outputs are the MMA's rows and the components its
@@ -387,7 +378,7 @@ __device__ __forceinline__ void fix_chunk_narrow(const uint2 *__restrict__ T, in
     };
     load_words(0, 0);
     unsigned B[NS][2][6];                                            // digit fragments
-    int ev[2], plain;
+    int ev[2], after;
     {
         // pair PL r + lane / C of component lane mod C
         double raw[NP][2][1];
@@ -405,7 +396,7 @@ __device__ __forceinline__ void fix_chunk_narrow(const uint2 *__restrict__ T, in
                     if (!EXPN) sh[r][p] = vec.shift(k0 + k) << 20;
                 }
             }
-        vec_scale<EXPN>(raw, sh, e, plain, [](int x) {
+        vec_scale<EXPN>(raw, sh, e, after, [](int x) {
 #pragma unroll
             for (int o = C; o < 32; o *= 2) x = max(x, __shfl_xor_sync(0xffffffffu, x, o));
             return x;
@@ -427,8 +418,13 @@ __device__ __forceinline__ void fix_chunk_narrow(const uint2 *__restrict__ T, in
         // exponents of the components this lane finishes
         ev[0] = __shfl_sync(0xffffffffu, e[0], C == 2 ? t & 1 : (2 * t) & (C - 1));
         ev[1] = __shfl_sync(0xffffffffu, e[0], C == 2 ? t & 1 : (2 * t + 1) & (C - 1));
-        plain = (int)__ballot_sync(0xffffffffu, plain != 0) & ((1 << C) - 1);     // lanes 0 .. C-1: one a component
+        if (__any_sync(0xffffffffu, after != 0)) {
+            const int a0 = __shfl_sync(0xffffffffu, after, C == 2 ? t & 1 : (2 * t) & (C - 1));
+            const int a1 = __shfl_sync(0xffffffffu, after, C == 2 ? t & 1 : (2 * t + 1) & (C - 1));
+            after = a0 | a1 << 2;
+        }
     }
+    const bool rare = __any_sync(0xffffffffu, after != 0);
     for (int n0 = 0; n0 < nn; n0 += 16) {
         constexpr int NOUT = C == 8 ? 2 : 1;                         // rows this lane finishes
         int key[NOUT];
@@ -461,49 +457,52 @@ __device__ __forceinline__ void fix_chunk_narrow(const uint2 *__restrict__ T, in
                 }
         }
         // rows g and g + 8, columns 2t and 2t + 1
-        if constexpr (C == 2) {
-            // both components of both rows on every t: lane t takes row g + 8 (t / 2), component t mod 2
-            float f[6];
+        auto finish = [&](auto back) {
+            if constexpr (C == 2) {
+                // both components of both rows on every t: lane t takes row g + 8 (t / 2), component t mod 2
+                float f[6];
 #pragma unroll
-            for (int d = 0; d < 6; ++d) {
-                const float lo = t & 1 ? acc[d][1] : acc[d][0], hi = t & 1 ? acc[d][3] : acc[d][2];
-                f[d] = t & 2 ? hi : lo;
-            }
-            if (n0 + g + 8 * (t >> 1) < nn) {
-                const double v[1] = {fix_to_double(fix_combine(f[0], f[1], f[2], f[3], f[4], f[5]),
-                                                   (t & 2 ? E[1] : E[0]) + (ev[0] >> 20) + (1054 - 1079))};
-                out.put(key[0], k0 > 0, t & 1, v);
-            }
-        } else if constexpr (C == 4) {
-            // lanes t and t + 2 hold components 2 (t mod 2), + 1: one takes row g, the other row g + 8
-            if (n0 + g + 8 * (t >> 1) < nn) {
-                double v[2];
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    float f[6];
-#pragma unroll
-                    for (int d = 0; d < 6; ++d) f[d] = t & 2 ? acc[d][2 + c] : acc[d][c];
-                    v[c] = fix_to_double(fix_combine(f[0], f[1], f[2], f[3], f[4], f[5]),
-                                         (t & 2 ? E[1] : E[0]) + (ev[c] >> 20) + (1054 - 1079));
+                for (int d = 0; d < 6; ++d) {
+                    const float lo = t & 1 ? acc[d][1] : acc[d][0], hi = t & 1 ? acc[d][3] : acc[d][2];
+                    f[d] = t & 2 ? hi : lo;
                 }
-                out.put(key[0], k0 > 0, t & 1, v);
-            }
-        } else {
-#pragma unroll
-            for (int x = 0; x < 2; ++x) {
-                if (n0 + g + 8 * x >= nn) continue;
-                double v[2];
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    const int f = 2 * x + c;
-                    v[c] = fix_to_double(fix_combine(acc[0][f], acc[1][f], acc[2][f], acc[3][f], acc[4][f], acc[5][f]),
-                                         E[x] + (ev[c] >> 20) + (1054 - 1079));
+                if (n0 + g + 8 * (t >> 1) < nn) {
+                    const double v[1] = {back(fix_to_double(fix_combine(f[0], f[1], f[2], f[3], f[4], f[5]),
+                                                            (t & 2 ? E[1] : E[0]) + (ev[0] >> 20) + (1054 - 1079)), 0)};
+                    out.put(key[0], k0 > 0, t & 1, v);
                 }
-                out.put(key[x], k0 > 0, t, v);
+            } else if constexpr (C == 4) {
+                // lanes t and t + 2 hold components 2 (t mod 2), + 1: one takes row g, the other row g + 8
+                if (n0 + g + 8 * (t >> 1) < nn) {
+                    double v[2];
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        float f[6];
+#pragma unroll
+                        for (int d = 0; d < 6; ++d) f[d] = t & 2 ? acc[d][2 + c] : acc[d][c];
+                        v[c] = back(fix_to_double(fix_combine(f[0], f[1], f[2], f[3], f[4], f[5]),
+                                                  (t & 2 ? E[1] : E[0]) + (ev[c] >> 20) + (1054 - 1079)), c);
+                    }
+                    out.put(key[0], k0 > 0, t & 1, v);
+                }
+            } else {
+#pragma unroll
+                for (int x = 0; x < 2; ++x) {
+                    if (n0 + g + 8 * x >= nn) continue;
+                    double v[2];
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        const int f = 2 * x + c;
+                        v[c] = back(fix_to_double(fix_combine(acc[0][f], acc[1][f], acc[2][f], acc[3][f], acc[4][f], acc[5][f]),
+                                                  E[x] + (ev[c] >> 20) + (1054 - 1079)), c);
+                    }
+                    out.put(key[x], k0 > 0, t, v);
+                }
             }
-        }
+        };
+        if (!rare) finish([](double v, int) { return v; });
+        else finish([after](double v, int c) { return fix_after(v, after >> 2 * c & 3); });
     }
-    if (plain) fix_plain<C>(T, sk, sn, k0, k0 + kc, nn, vec, out, plain, lane);
 }
 
 template <int C, bool EXPN, int NG, class Vec, class Out>
@@ -519,8 +518,7 @@ __device__ __forceinline__ void fix_chunk(const uint2 *__restrict__ T, int sk, i
 // vec[k]; add: v goes on top of an earlier chunk.  EXPN: the words' exponents
 // belong to n (a column is contracted over), else to k (vec.shift(k) returns
 // them).  vec.load(k, i, x): components W i .. of entry k, called once for
-// each entry and component; vec.value(k, c): component c.  All 32 lanes take
-// part.  The words of up to 7 entries past kn are read (and meet zero
+// each entry and component.  All 32 lanes take part.  The words of up to 7 entries past kn are read (and meet zero
 // digits): plan arrays are allocated with that slack.
 template <int C, bool EXPN, class Vec, class Out>
 __device__ __forceinline__ void fix_product(const uint2 *__restrict__ T, int sk, int sn, int kn, int nn, const Vec &vec,

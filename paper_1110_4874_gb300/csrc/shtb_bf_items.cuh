@@ -46,7 +46,6 @@ struct ResVec {
         ld_comps<CG ? Ld::kL2 : Ld::kGlobal>(a0 + (size_t)k * astride, i, x);
     }
     __device__ __forceinline__ int shift(int) const { return 0; }
-    __device__ __forceinline__ double value(int k, int c) const { return __ldcg(a0 + (size_t)k * astride + c); }
 };
 
 template <int C>
@@ -103,7 +102,6 @@ struct LevelVec {
         st_comps(scr + __ldg(ipos + k) * C, i, x, second);
     }
     __device__ __forceinline__ int shift(int) const { return 0; }
-    __device__ __forceinline__ double value(int k, int c) const { return __ldcg(u + (size_t)k * C + c); }
 };
 
 template <int C>

@@ -248,7 +248,6 @@ struct AdjLevelVec {
         const uint2 w = __ldg(T + d);
         return shtb::fix_word_exp(w.x, w.y);
     }
-    __device__ __forceinline__ double value(int d, int c) const { return in[dpos[d] * C + c]; }
 };
 
 // u_i: the identity entry plus the dense product (later chunks on top)
@@ -340,7 +339,6 @@ struct AdjResVec {
         const uint2 w = __ldg(R + s);
         return shtb::fix_word_exp(w.x, w.y);
     }
-    __device__ __forceinline__ double value(int s, int c) const { return at(s)[c]; }
 };
 
 template <int C>

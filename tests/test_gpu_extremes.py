@@ -95,3 +95,49 @@ def test_extreme_rings_cost_little():
         q, f = r.q * p, r.f * p
         assert ms(lambda: r.synth(q)) <= 2 * t_s + 0.05, p
         assert ms(lambda: r.adjoint(f)) <= 2 * t_a + 0.05, p
+
+
+def coefficients(plan, nmaps):
+    g = torch.Generator(device="cuda").manual_seed(5)
+    a = torch.randn(nmaps, plan.nalm, 2, dtype=torch.float64, device="cuda", generator=g)
+    a[:, :plan.lmax + 1, 1] = 0
+    return torch.view_as_complex(a)
+
+
+# compressed plans, several chunks of 32 (max_depth 0) and many levels
+@pytest.mark.parametrize("nside,lmax,opts", [(32, 80, {}), (16, 70, {"max_depth": 0}), (64, 200, {"leaf_cols": 17})])
+@pytest.mark.parametrize("nmaps", [1, 2, 4, 8])
+def test_compressed_plans_scale_exactly_by_powers_of_two(nside, lmax, opts, nmaps):
+    """Nothing is subnormal: the operator's elements and their products are zero
+    or above 2^-120."""
+    plan = sh.Plan(nside, lmax, 1e-10, **opts)
+    a = coefficients(plan, nmaps)
+    maps = plan.synthesize(a)
+    back = plan.adjoint(maps)
+    for power in (-850, -700, 700, 850, 980):
+        p = 2.0 ** power
+        assert torch.equal(plan.synthesize(a * p), maps * p), power
+        assert torch.equal(plan.adjoint(maps * p), back * p), power
+    # one map of another scale, or not finite, leaves the rest alone
+    for x in BAD + [2.0 ** -850, 2.0 ** 900]:
+        b, f = a.clone(), maps.clone()
+        b[0] *= x
+        f[0] *= x
+        assert torch.equal(plan.synthesize(b)[1:], maps[1:])
+        assert torch.equal(plan.adjoint(f)[1:], back[1:])
+        if x in BAD or x != x:
+            assert not torch.isfinite(plan.synthesize(b)[0]).any()
+            assert not torch.isfinite(torch.view_as_real(plan.adjoint(f)[0])[lmax + 1:]).any()
+
+
+@pytest.mark.parametrize("eps,most", [(1e-10, 2), (0.0, 4)])       # uncompressed sums take FP64 there
+@pytest.mark.parametrize("nmaps", [1, 8])
+def test_extreme_maps_cost_little(eps, most, nmaps):
+    plan = sh.Plan(256, 512, eps)
+    a = coefficients(plan, nmaps)
+    maps = plan.synthesize(a)
+    t_s, t_a = ms(lambda: plan.synthesize(a)), ms(lambda: plan.adjoint(maps))
+    for x in BAD + [2.0 ** -850, 2.0 ** 900]:
+        b, f = a * x, maps * x
+        assert ms(lambda: plan.synthesize(b)) <= most * t_s + 0.05, x
+        assert ms(lambda: plan.adjoint(f)) <= most * t_a + 0.05, x
