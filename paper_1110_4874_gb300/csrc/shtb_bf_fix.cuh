@@ -1,8 +1,8 @@
 // Block products of the butterfly, out[n][c] = sum_k T[k][n] v[k][c], on the
 // tensor cores, to the last place of FP64: both factors are fixed-point
 // numbers cut into six signed digits of radix 2^10, the digit products run as
-// f16 MMAs whose FP32 sums are whole numbers below 2^24 and so exact, and the
-// sums are put together in integer arithmetic and rounded to double once.
+// f16 MMAs whose FP32 sums are whole numbers, exact up to 2^24 (see below), and
+// the sums are put together in integer arithmetic and rounded to double once.
 //
 // Why: the FP64 pipe does 2 FMAs a clock on an SM (a warp's DFMA occupies it
 // for 16 clocks), the legacy f16 MMA 1024.  21 digit products of 10 bits a
@@ -23,12 +23,16 @@
 // sums 24 times.  On the compressed Legendre blocks of Nside = 256, L = 512
 // the relative rms error is 0.9e-16 with the words' 54 bits, against 1.6e-16
 // of the FMA chain.
-// Exactness of the FP32 sums over 32 entries: |t_0| <= 256, |u_0| <= 128, the
-// other digits at most 512, so diagonals 0, 1, 2 stay below 2^20, 2^22.6 and
-// 2^23.9.  Diagonals 3 to 5 could pass 2^24 only if three quarters of the
-// largest possible digits met with one sign in every product, which the
-// digits of T (of interpolation weights and Legendre functions) do not; the
-// loss would be one unit of a diagonal's sum.
+// FP32 sums over 32 entries: |t_0| <= 256, |u_0| <= 128, the other digits at
+// most 512, so diagonals 0, 1, 2 stay below 2^20, 2^22.6 and 2^23.9 and are
+// exact.  Diagonals 3, 4 and 5 have 2^24.5, 2^24.9 and 2^25.2 as their largest
+// and pass 2^24, from where a sum is rounded to even, at 73, 53 and 42 % of it:
+// only if digits that large meet with one sign in all entries and pairs.  A unit
+// of diagonal 3, 4 or 5 is 2^-45, 2^-55 or 2^-65 of max|T| max|v|.  Digits of T
+// (interpolation weights and Legendre functions) are as good as random, ten
+// standard deviations away from that; where they repeat along a sum (the
+// constant l = 0 function, over a block's rings) the worst vector brings
+// diagonals 3 and 4 to 76 and 95 % of 2^24, and diagonal 5 past it.
 //
 // Measured (GB300, Nside = 512, L = 1024, eps = 1e-10; residual blocks plus
 // levels, FP64 FMA kernels before): 8 maps 5.31 -> 1.50 ms, 4 maps 2.79 ->
@@ -38,8 +42,10 @@
 // 41-52 % used, tensor pipe 17-29 %, FP64 pipe 1 %).
 //
 // Results do not depend on the other components, on how maps are grouped or
-// on the lane layout: the sums are exact, and chunks of 32 are added in FP64
-// in order.  A component whose chunk holds an infinity or a NaN gives NaN.
+// on the lane layout: the sums are exact (but for the vectors just named), and
+// chunks of 32 are added in FP64 in order.  The digits of -x are not those of x
+// negated, so a negated input gives the negated result up to its last place.
+// A component whose chunk holds an infinity or a NaN gives NaN.
 #pragma once
 
 #include <cuda_runtime.h>
