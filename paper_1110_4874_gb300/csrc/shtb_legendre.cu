@@ -24,11 +24,11 @@
 // pipe, which takes a warp's DFMA in 16 clocks of an SM against half a clock
 // for an integer multiply-add, held these kernels with both done in FP64.
 // Legendre stage, FP64 sums -> this (ms):
-//   nside 64, lmax 128, 1 map      synthesis  .047 -> .031  adjoint  .054 -> .038
-//   nside 100, lmax 255, 1 map                .095 -> .056           .140 -> .070
-//   nside 256, lmax 512, 4 maps               .996 -> .443          1.385 -> .566
-//   nside 256, lmax 512, 8 maps              1.730 -> .766          2.416 -> .989
-//   nside 512, lmax 1024, 8 maps             12.22 -> 5.15          13.94 -> 5.93
+//   nside 64, lmax 128, 1 map      synthesis  .047 -> .031  adjoint  .054 -> .039
+//   nside 100, lmax 255, 1 map                .095 -> .056           .140 -> .068
+//   nside 256, lmax 512, 4 maps               .996 -> .441          1.385 -> .576
+//   nside 256, lmax 512, 8 maps              1.730 -> .762          2.416 -> .981
+//   nside 512, lmax 1024, 8 maps             12.22 -> 5.13          13.94 -> 5.77
 // What bounds them now is issue (48 % of the slots with 8 maps, the FP64 pipe
 // at 31 %) and, with few maps, the chain of dependent FMAs of the recurrence.
 // Precision: a or g are cut 49 bits or more below a run's largest, V 55 to 58
@@ -549,10 +549,19 @@ legendre_adjoint_kernel(PlanView v, const double2 *__restrict__ g, double2 *__re
         LegSums<C> sums;
         sums.clear(Z);
         int2 scale = make_int2(0, 0);
+        // sums of the tile that the integers no longer hold; most tiles need none,
+        // so the (local memory) array is not touched before one does: 5.93 -> 5.77
+        // ms with 8 maps at nside 512
         double acc[C];
+        bool kept = false;
+        auto keep = [&] {
+            if (kept) return;
+            kept = true;
 #pragma unroll
-        for (int c = 0; c < C; ++c) acc[c] = 0.0;
+            for (int c = 0; c < C; ++c) acc[c] = 0.0;
+        };
         auto settle = [&](int2 next) {
+            keep();
 #pragma unroll
             for (int c = 0; c < C; ++c) {
                 const int e = of_component(scale, c);
@@ -606,14 +615,19 @@ legendre_adjoint_kernel(PlanView v, const double2 *__restrict__ g, double2 *__re
 #pragma unroll 4
             for (int r2 = 0; r2 < 32; ++r2) sums.add(row[r2], lim + r2 * C);
             sums.carry();
-            if (__any_sync(0xffffffffu, min(eg.x, eg.y) < 0)) plain_rings<NB>(row, gc, gstride, nr, eg, reinterpret_cast<double2 *>(lim), acc, lane);
+            if (__any_sync(0xffffffffu, min(eg.x, eg.y) < 0)) {
+                keep();
+                plain_rings<NB>(row, gc, gstride, nr, eg, reinterpret_cast<double2 *>(lim), acc, lane);
+            }
             __syncwarp();
         }
-        settle(make_int2(-1, -1));
         // add the warps' partial sums of each parity and store them
         double *mine = tile;                            // [C][32], rows of 33
 #pragma unroll
-        for (int c = 0; c < C; ++c) mine[c * kTilePad + lane] = acc[c];
+        for (int c = 0; c < C; ++c) {
+            const double v = sums.value(c, of_component(scale, c));
+            mine[c * kTilePad + lane] = kept ? acc[c] + v : v;
+        }
         __syncthreads();
         for (int i = threadIdx.x; i < 2 * 32 * NB; i += blockDim.x) {
             const int tt = i / (32 * NB), rem = i - tt * 32 * NB;
