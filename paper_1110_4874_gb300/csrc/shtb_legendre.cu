@@ -85,8 +85,8 @@ __global__ void alm_prescale_kernel(PlanView v, const double2 *__restrict__ alm,
 // along a chain from the crop on, so a run whose large values meet a small V
 // and whose small ones a large V would lose what FP64 keeps: its largest
 // exponent lies in a range, every four neighbours have one at most kLegDrop
-// bits below any before them, the last two one at most kLegLast, and it has
-// kLegShort entries or more.
+// bits below any before them, the last two one at most kLegLast, and a run of a
+// (a chain's end) has kLegShort entries or more.
 constexpr int kLegExpLo = 300, kLegExpHi = 1700, kLegDrop = 7, kLegLast = 10, kLegShort = 8;
 // A component's scale, the exponent its limbs are cut at, is set a bit above
 // the largest of the run that needs it and kept for the runs whose largest
@@ -126,7 +126,7 @@ struct Run {
         }
     }
     // the largest exponent: 0 for a component of zeros, -1 for one to take in FP64
-    __device__ __forceinline__ int2 scan(int count, int lane) const
+    __device__ __forceinline__ int2 scan(int count, int least, int lane) const
     {
         unsigned top = 0, drop = 0, last = 0;                        // two components in halves
 #pragma unroll
@@ -148,8 +148,8 @@ struct Run {
 #pragma unroll
         for (int o = 4 * NB; o < 32; o *= 2) drop = __vmaxu2(drop, __shfl_xor_sync(0xffffffffu, drop, o));
         last = top - __shfl_sync(0xffffffffu, last, (count - 1) % STEP * NB + lane % NB);
-        auto one = [count](int e, int below, int end) {
-            return e == 0 ? 0 : e < kLegExpLo || e > kLegExpHi || below > kLegDrop || end > kLegLast || count < kLegShort ? -1 : e;
+        auto one = [count, least](int e, int below, int end) {
+            return e == 0 ? 0 : e < kLegExpLo || e > kLegExpHi || below > kLegDrop || end > kLegLast || count < least ? -1 : e;
         };
         return make_int2(one(top & 0xffff, drop & 0xffff, last & 0xffff), one(top >> 16, drop >> 16, last >> 16));
     }
@@ -376,7 +376,7 @@ legendre_synth_kernel(PlanView v, const double2 *__restrict__ ap, double2 *__res
             nj = run_length(n - jb);
             Run<NB> run;
             run.load(a + (size_t)jb * stride, stride, nj, lane);
-            const int2 ea = run.scan(nj, lane);
+            const int2 ea = run.scan(nj, kLegShort, lane);
             const bool plain = __any_sync(0xffffffffu, min(ea.x, ea.y) < 0);
             const int2 next = make_int2(next_scale(scale.x, ea.x), next_scale(scale.y, ea.y));
             if (__any_sync(0xffffffffu, scale_left(scale, next))) settle(next);
@@ -533,13 +533,16 @@ legendre_adjoint_kernel(PlanView v, const double2 *__restrict__ g, double2 *__re
     const double *gm = reinterpret_cast<const double *>(g + ((size_t)m * 2 + t) * Z * nmaps + b0);
     const size_t gstride = (size_t)2 * nmaps;                         // doubles between rings
     const int ntiles = (n0 + 31) >> 5;
+    const int Zt = Z - t;                                             // the odd functions vanish on the equator
     // the largest exponents of this warp's runs of g: chunk set + i W/2 at se[i NB + b]
     short2 *se = reinterpret_cast<short2 *>(smd + (size_t)W * adjoint_warp_smem_doubles<NB>()) +
                (size_t)warp * adjoint_warp_chunks(nchunk, W) * NB;
+    // (a last run of few rings is no chain's end: V is level about the equator)
+    auto rings = [&](int c) { return max(1, min(32, Zt - c * 32)); };
     for (int c = set, i = 0; c < nchunk; c += W / 2, ++i) {
         Run<NB> run;
-        run.load(gm + (size_t)c * 32 * gstride, gstride, min(32, Z - c * 32), lane);
-        const int2 e = run.scan(min(32, Z - c * 32), lane);
+        run.load(gm + (size_t)c * 32 * gstride, gstride, rings(c), lane);
+        const int2 e = run.scan(rings(c), 1, lane);
         if (lane < NB) se[i * NB + lane] = make_short2((short)e.x, (short)e.y);
     }
     __syncwarp();
@@ -596,7 +599,7 @@ legendre_adjoint_kernel(PlanView v, const double2 *__restrict__ g, double2 *__re
             }
             if (valid) st[2 * r] = make_double2(ch.cur, ch.prev);
             const double *gc = gm + (size_t)c * 32 * gstride;
-            const int nr = min(32, Z - c * 32);
+            const int nr = rings(c);
             const short2 es = se[(c - set) / (W / 2) * NB + lane % NB];
             const int2 eg = make_int2(es.x, es.y);
             const int2 next = make_int2(next_scale(scale.x, eg.x), next_scale(scale.y, eg.y));

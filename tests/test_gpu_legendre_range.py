@@ -118,3 +118,29 @@ def test_each_coefficient_of_an_adjoint(setting, kind):
         one = torch.empty_like(out[:n])
         sh.shtb_test_legendre_adjoint(plan.handle, Ft[:n].contiguous(), one, n)
         assert torch.equal(one, out[:n])
+
+
+@pytest.mark.parametrize("nside", [129, 130, 131, 144])                  # last runs of 2, 4, 6 and 32 rings
+def test_adjoint_beside_a_bright_equator(nside):
+    """The equator adds nothing to the odd chains: their coefficients stay exact
+    beside it.  The even functions have their extremum there."""
+    lmax, half = 150, 2 * nside
+    plan = sh.Plan(nside, lmax, 0.0)
+    rng = np.random.default_rng(23)
+    F = rng.standard_normal((2, plan.nrings, lmax + 1)) + 1j * rng.standard_normal((2, plan.nrings, lmax + 1))
+    F[0, half - 1] *= 1e12
+    F[..., 0].imag = 0
+    out = torch.empty(2, plan.nalm, dtype=torch.complex128, device="cuda")
+    sh.shtb_test_legendre_adjoint(plan.handle, torch.from_numpy(F).cuda(), out, 2)
+    for b in (0, 1):
+        got = out[b].cpu().numpy()
+        south = np.zeros((half, lmax + 1), dtype=complex)
+        south[:-1] = F[b, :half - 1:-1]
+        for m in (0, 1, 5, 40, 100, 150):
+            P = np.array([sh.shtb_test_host_recurrence(nside, lmax, m, r) for r in range(half)])
+            at = int(synthetic.alm_index(lmax, m, m))
+            for t, g in enumerate((F[b, :half, m] + south[:, m], F[b, :half, m] - south[:, m])):
+                cm, R = (1 if m == 0 else 2), P[:, t::2].T
+                size = cm * (np.abs(R) @ np.abs(g))
+                err = np.abs(got[at:at + lmax - m + 1][t::2] - cm * exact(R, g))
+                assert np.all(err <= (half + 8) * ULP * size), (b, m, t)
