@@ -40,7 +40,7 @@ UNIT = "ms/map"
 # GB300 FP64 pipe: 152 SMs x 2 DFMA/clock/SM x 2 flop x 2.070 GHz max SM clock
 # (2 DFMA/clock/SM is NVIDIA's published 1.25 TFLOP/s FP64 rate for GB300
 # divided over 152 SMs at 2070 MHz).  The transforms do their products in
-# exact integer and digit arithmetic off this pipe, so it is no bound of
+# integer and digit arithmetic off this pipe, so it is no bound of
 # theirs: the line reports how many times its rate they reach.
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
 
@@ -51,9 +51,9 @@ NCU_TRAFFIC = {
     "legendre_synth_kernel": {
         "sources": ["paper_1110_4874_gb300/csrc/shtb_legendre.cu::legendre_synth_kernel",
                     "paper_1110_4874_gb300/csrc/shtb_limbs.cuh"],
-        "sha256": "f80381d57e0e82704ed2c8f23125413a42d524caf0c5ef1c93a7d41deb956156",
+        "sha256": "8fb014e9be4c24d757652bf606e61541789360bce0d03a0eb1a4767585091ad3",
         # measured at Nside=512, L=1024; every array scales with Nside*L (x16)
-        "bytes": 16 * (122_818_560 + 215_400_960),
+        "bytes": 16 * (122_549_760 + 214_859_008),
         "profile": "profiles/legendre_kernels_nside512_l1024_b8.md",
     },
     # butterfly kernels: DRAM bytes of one synthesis of 8 maps at Nside=2048,
@@ -65,17 +65,17 @@ NCU_TRAFFIC = {
     "bf_level_kernel": {
         "sources": ["paper_1110_4874_gb300/csrc/shtb_bf_items.cuh", "paper_1110_4874_gb300/csrc/shtb_bf_fix.cuh",
                     "paper_1110_4874_gb300/csrc/shtb_butterfly.cu::bf_level_kernel"],
-        "sha256": "8bb4e2c2b504e3737be5cd617797e5c9aac5213d70ddf8a464218538762a3660",
-        # (2132.2 + 766.2) MB x 4,266,029,163 / 140,986,926 dense elements
-        "bytes": round((2132213504 + 766156288) * 4_266_029_163 / 140_986_926),
+        "sha256": "39f08d3b46fab83e47da8c556d0e923eff1ccc4744465f32c1207ae6f1016f66",
+        # (2132.5 + 765.0) MB x 4,266,029,163 / 140,986,926 dense elements
+        "bytes": round((2132501504 + 765021696) * 4_266_029_163 / 140_986_926),
         "profile": "profiles/butterfly_kernels_nside512_l1024_b8.md",
     },
     "bf_r_kernel": {
         "sources": ["paper_1110_4874_gb300/csrc/shtb_bf_items.cuh", "paper_1110_4874_gb300/csrc/shtb_bf_fix.cuh",
                     "paper_1110_4874_gb300/csrc/shtb_butterfly.cu::bf_r_kernel"],
-        "sha256": "c68eb66b48af022d788ad241197b3d26bd5e23e72bc139132bdbf683cab664c8",
+        "sha256": "679a02e950ae6ec24e774d6acab6d5a0662c1ba88602ded5277ab9f2b0a1e9cc",
         # (448.9 + 194.4) MB x 787,402,057 / 46,195,210 stored residual elements
-        "bytes": round((448_886_784 + 194_392_320) * 787_402_057 / 46_195_210),
+        "bytes": round((448_887_552 + 194_345_472) * 787_402_057 / 46_195_210),
         "profile": "profiles/butterfly_kernels_nside512_l1024_b8.md",
     },
 }

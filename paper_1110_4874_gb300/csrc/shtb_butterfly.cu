@@ -13,7 +13,7 @@
 // q_m(-z) = q^0 - q^1 (Eq. q-even-odd2) straight from the two parity halves.
 // One warp per work item; all maps of a group (up to 8, 2 real components
 // each) are carried per entry so every stored matrix element is read once
-// per group.  The dense products run on the tensor cores in exact fixed-point
+// per group.  The dense products run on the tensor cores in fixed-point
 // digits (shtb_bf_fix.cuh).
 #include <cuda_runtime.h>
 

@@ -18,8 +18,8 @@
 // 1.7..2.0e-16 with a factor 3 to 13, Rader 4.0e-16 -> 3.1e-16 and 3.9e-16 ->
 // 3.4e-16, Bluestein 4.8e-16 -> 3.7e-16; synthesis the same to 10 %.
 // Measured (Nside = 512, L = 1024, 8 maps; FP64 transforms before): ring
-// synthesis 1.80 -> .86 ms, adjoint 2.42 -> .94 ms; Nside = 1024: 7.60 ->
-// 3.76 and 9.79 -> 4.03 ms (1.14, 1.16, 3.90 and 4.12 by the change of
+// synthesis 1.80 -> .87 ms, adjoint 2.42 -> .96 ms; Nside = 1024: 7.60 ->
+// 3.83 and 9.79 -> 4.05 ms (1.14, 1.16, 3.90 and 4.12 by the change of
 // arithmetic alone).  What bounds them now is the issue of integer
 // instructions at the direct lengths (65 to 71 % of the slots) and latency
 // and instruction fetches at the others (36 to 49 %, 16 warps an SM).
